@@ -17,9 +17,16 @@
 // the diagonal part; the block offsets of the tuples reached by changing
 // the levels of i and j are tabulated per (tuple, pair) on the host.
 //
-// The kernel adds these terms to y after the diagonal gather (gmv_kernel):
-// one thread per output, the two factors' rows walked as a sum-factorised
-// double loop.
+// B_ij depends on the two 1D indices alone, not on which pair, on d or on
+// the other directions, so it is tabulated once as a 2D sparse-grid matrix:
+// row (a_i, a_j), one value per column (b_i, b_j) with the four terms already
+// added, columns sorted by l(b_i) + l(b_j) so that the truncation at L is a
+// prefix of the row.  cross_rows_kernel adds -K_ij B_ij x to y after the
+// diagonal gather (gmv_kernel): one warp per output, the lanes striding over
+// the row.  Index sets whose table would exceed X2_MAX_ENT entries (the 2D
+// row count times some hundred: level 9, degree 3 is below, level 11 is
+// above) keep cross_kernel: one thread per output, the two factors' rows
+// walked as a sum-factorised double loop.
 #include <algorithm>
 #include <cmath>
 #include <map>
@@ -29,6 +36,140 @@
 namespace {
 
 constexpr int XT = 4;  // stored 1D matrices: Q, P^T, E^T, P
+
+constexpr int64_t X2_MAX_ENT = int64_t(1) << 26;  // 1.3 GB of entries and values, FP64 and FP32
+
+// The entries of the 2D rows: CTA a_i, one warp per a_j, the lanes over the
+// product of the two unions of columns.  Column (b_i, b_j) of level sum s
+// stands behind the columns of smaller sums (the prefix length of s - 1) and
+// of the same sum with smaller l(b_i), in order of b_i, then b_j.
+__global__ void __launch_bounds__(256) cross_fill_kernel(int H, int N, int kp1, const int* __restrict__ uptr,
+                                                         const int* __restrict__ ucol,
+                                                         const double* __restrict__ uval,
+                                                         const int* __restrict__ upto, const int* __restrict__ row0,
+                                                         const int* __restrict__ ptr, const int* __restrict__ len,
+                                                         int2* __restrict__ ent, double* __restrict__ val,
+                                                         float* __restrict__ valf) {
+    const int nl = N + 1, lane = threadIdx.x & 31;
+    const int ai = blockIdx.x;
+    auto level = [&](int a) {
+        const int q = a / kp1;
+        return q == 0 ? 0 : 32 - __clz(q);
+    };
+    auto start = [&](int a, int l) { return l ? upto[a * nl + l - 1] : 0; };  // first column of level l in row a
+    const int ni = uptr[ai + 1] - uptr[ai];
+    for (int aj = threadIdx.x >> 5; aj < (kp1 << (N - level(ai))); aj += blockDim.x >> 5) {
+        const int row = row0[ai] + aj;
+        const int nj = uptr[aj + 1] - uptr[aj];
+        for (int i = 0; i < ni; ++i) {
+            const int bi = ucol[uptr[ai] + i], li = level(bi);
+            const double* vi = uval + (size_t)(uptr[ai] + i) * XT;
+            for (int j = lane; j < nj; j += 32) {
+                const int bj = ucol[uptr[aj] + j], lj = level(bj), s = li + lj;
+                if (s > N) break;  // columns ascend, and so do their levels
+                int pos = s ? len[row * nl + s - 1] : 0;
+                for (int l = 0; l < li; ++l)
+                    pos += (upto[ai * nl + l] - start(ai, l)) * (upto[aj * nl + s - l] - start(aj, s - l));
+                pos += (i - start(ai, li)) * (upto[aj * nl + lj] - start(aj, lj)) + (j - start(aj, lj));
+                const double* vj = uval + (size_t)(uptr[aj] + j) * XT;
+                const double t0 = vi[0] * vj[1], t1 = vi[1] * vj[0], t2 = vi[2] * vj[3], t3 = vi[3] * vj[2];
+                double v = (t0 + t1) - (t2 + t3);
+                // terms that cancel leave only their rounding
+                if (fabs(v) <= 4e-16 * (fabs(t0) + fabs(t1) + fabs(t2) + fabs(t3))) v = 0.0;
+                const int ti = bi - (li == 0 ? 0 : kp1 << (li - 1)), tj = bj - (lj == 0 ? 0 : kp1 << (lj - 1));
+                const int at = ptr[row] + pos;
+                ent[at] = make_int2(ti | (tj << 16), li | (lj << 8));
+                val[at] = v;
+                valf[at] = (float)v;
+            }
+        }
+    }
+}
+
+// The mixed-derivative terms from the table of 2D rows.  cross_kernel spends
+// four FP64 multiply-adds and a block position (a loop over the directions)
+// on every column, in the order of its longest rows; the table leaves one
+// multiply-add and two integer ones, over entries (16 bytes) that stay in
+// L2.  One warp per output because the rows are uneven: those of low levels
+// reach every cell (thousands of columns), most have some hundred, so a
+// thread per output waits for the longest; the warps of a CTA take
+// consecutive outputs, which share rows and block offsets.  d = 3, level 5,
+// degree 2 (7 344 outputs, 549 000 entries): a matvec of both launches takes
+// 36 us, with cross_kernel 1.13 ms.
+template <typename T>
+__global__ void __launch_bounds__(256) cross_rows_kernel(int dof, int d, int N, int kp1, int ntuples,
+                                                         const int32_t* __restrict__ levels,
+                                                         const int64_t* __restrict__ offsets, int npairs,
+                                                         const int* __restrict__ pair_ij,
+                                                         const double* __restrict__ kij, const int* __restrict__ row0,
+                                                         const int* __restrict__ ptr, const int* __restrict__ len,
+                                                         const int2* __restrict__ ent, const T* __restrict__ val,
+                                                         const int64_t* __restrict__ grp,
+                                                         const int64_t* __restrict__ xoff, const T* __restrict__ x,
+                                                         T* __restrict__ y) {
+    const int lane = threadIdx.x & 31;
+    const int warps = (int)((gridDim.x * blockDim.x) >> 5);
+    for (int g = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5); g < dof; g += warps) {
+        int lo = 0, hi = ntuples;  // offsets[lo] <= g < offsets[hi]
+        while (hi - lo > 1) {
+            const int mid = (lo + hi) >> 1;
+            if (offsets[mid] <= g) lo = mid;
+            else hi = mid;
+        }
+        const int e0 = g - (int)offsets[lo];
+        int lsum = 0;
+        for (int m = 0; m < d; ++m) lsum += levels[lo * d + m];
+        T acc_all = T(0);
+        for (int p = 0; p < npairs; ++p) {
+            const int i = pair_ij[2 * p], j = pair_ij[2 * p + 1];
+            // the output's position is (((o n_i + t_i) mid + c) n_j + t_j) in + r:
+            // o over the directions before i, c between, r after j
+            int rest = e0, in = 1, mid = 1, r = 0, c = 0, o = 0, ti = 0, tj = 0, li = 0, lj = 0, mul = 1;
+            for (int m = d - 1; m >= 0; --m) {
+                const int l = levels[lo * d + m], n_l = l == 0 ? kp1 : kp1 << (l - 1);
+                const int q = rest / n_l, t = rest - q * n_l;
+                rest = q;
+                if (m == j) {
+                    tj = t;
+                    lj = l;
+                    mul = 1;
+                } else if (m == i) {
+                    ti = t;
+                    li = l;
+                    mul = 1;
+                } else if (m > j) {
+                    r += t * mul;
+                    in = mul *= n_l;
+                } else if (m > i) {
+                    c += t * mul;
+                    mid = mul *= n_l;
+                } else {
+                    o += t * mul;
+                    mul *= n_l;
+                }
+            }
+            const int L = N - (lsum - li - lj);
+            const int ai = (li == 0 ? 0 : kp1 << (li - 1)) + ti, aj = (lj == 0 ? 0 : kp1 << (lj - 1)) + tj;
+            const int row = row0[ai] + aj;
+            const int qe = ptr[row] + len[row * (N + 1) + L];
+            const int64_t* offs = xoff + grp[(int64_t)lo * npairs + p];
+            T acc = T(0);
+#pragma unroll 4
+            for (int q = ptr[row] + lane; q < qe; q += 32) {
+                const int2 en = ent[q];
+                const int bi = en.x & 0xffff, bj = en.x >> 16;
+                const int mi = en.y & 0xff, mj = en.y >> 8;
+                const int ni = mi == 0 ? kp1 : kp1 << (mi - 1), nj = mj == 0 ? kp1 : kp1 << (mj - 1);
+                const int pos = (((o * ni + bi) * mid + c) * nj + bj) * in + r;
+                acc += val[q] * x[(int)offs[mi * (L + 1) + mj] + pos];
+            }
+            acc_all += (T)kij[p] * acc;
+        }
+#pragma unroll
+        for (int s = 16; s > 0; s >>= 1) acc_all += __shfl_xor_sync(0xffffffffu, acc_all, s);
+        if (lane == 0) y[g] -= acc_all;
+    }
+}
 
 template <typename T>
 __global__ void __launch_bounds__(256) cross_kernel(int64_t dof, int d, int N, int kp1, int64_t ntuples,
@@ -111,7 +252,7 @@ __global__ void __launch_bounds__(256) cross_kernel(int64_t dof, int d, int N, i
 
 }  // namespace
 
-// Host tables of the mixed-derivative terms of op for the tensor K (d x d,
+// Tables of the mixed-derivative terms of op for the tensor K (d x d,
 // row-major, symmetric); no-op when K is diagonal.
 void build_cross_tables(sgk_op* op, const double* K) {
     const sgk_index* idx = op->idx;
@@ -209,6 +350,67 @@ void build_cross_tables(sgk_op* op, const double* K) {
             grp[(size_t)tu * op->npairs + p] = it->second;
         }
     }
+    // the pair form as 2D rows: per 1D index the union of the four factors'
+    // columns (ascending, so by level), counted per level; the row starts and
+    // the prefix lengths follow from the counts, the entries are filled in on
+    // the device
+    std::vector<int> uptr(1, 0), upto((size_t)H * nl, 0), ucol;
+    std::vector<double> uval;
+    for (int a = 0; a < H; ++a) {
+        int e[XT], end[XT];
+        for (int X = 0; X < XT; ++X) {
+            e[X] = ptr[(size_t)X * (H + 1) + a];
+            end[X] = ptr[(size_t)X * (H + 1) + a + 1];
+        }
+        for (;;) {
+            int b = H;
+            for (int X = 0; X < XT; ++X)
+                if (e[X] < end[X]) b = std::min(b, col[e[X]]);
+            if (b == H) break;
+            ucol.push_back(b);
+            for (int X = 0; X < XT; ++X) uval.push_back(e[X] < end[X] && col[e[X]] == b ? val[e[X]++] : 0.0);
+            int l = 0;
+            while ((kp1 << l) <= b) ++l;
+            for (int m = l; m < nl; ++m) ++upto[(size_t)a * nl + m];
+        }
+        uptr.push_back((int)ucol.size());
+    }
+    std::vector<int> ptr2, len2, row2(H);
+    int64_t total = 0;
+    const auto at_level = [&](int a, int l) { return upto[(size_t)a * nl + l] - (l ? upto[(size_t)a * nl + l - 1] : 0); };
+    for (int ai = 0, li = 0; ai < H && total <= X2_MAX_ENT; ++ai) {
+        while ((kp1 << li) <= ai) ++li;
+        row2[ai] = (int)ptr2.size();
+        for (int aj = 0; aj < (kp1 << (N - li)) && total <= X2_MAX_ENT; ++aj) {
+            ptr2.push_back((int)total);
+            int64_t n = 0;
+            for (int L = 0; L < nl; ++L) {  // columns with l(b_i) + l(b_j) <= L
+                for (int l = 0; l <= L; ++l) n += (int64_t)at_level(ai, l) * at_level(aj, L - l);
+                len2.push_back((int)n);
+            }
+            total += n;
+        }
+    }
+    if (total <= X2_MAX_ENT && idx->dof < (int64_t(1) << 31) && len2.size() < (size_t(1) << 31)) {
+        cudaStream_t s2 = op->ctx->stream;
+        DevBuf<int> d_uptr, d_ucol, d_upto;
+        DevBuf<double> d_uval;
+        d_uptr.upload(uptr, s2);
+        d_ucol.upload(ucol, s2);
+        d_uval.upload(uval, s2);
+        d_upto.upload(upto, s2);
+        op->x2_ptr.upload(ptr2, s2);
+        op->x2_len.upload(len2, s2);
+        op->x2_row.upload(row2, s2);
+        op->x2_ent.alloc(total);
+        op->x2_val.alloc(total);
+        op->x2_valf.alloc(total);
+        cross_fill_kernel<<<H, 256, 0, s2>>>(H, N, kp1, d_uptr.p, d_ucol.p, d_uval.p, d_upto.p, op->x2_row.p,
+                                             op->x2_ptr.p, op->x2_len.p, op->x2_ent.p, op->x2_val.p, op->x2_valf.p);
+        check_launch("cross_fill_kernel");
+        count_launch(op->ctx);
+        SGK_CUDA_CHECK(cudaStreamSynchronize(s2));
+    }
     cudaStream_t s = op->ctx->stream;
     op->x_pairs.upload(pij, s);
     op->x_kij.upload(kij, s);
@@ -234,6 +436,18 @@ void op_cross_matvec(const sgk_op* op, const T* x, T* y) {
     const T* vals = sizeof(T) == 8 ? reinterpret_cast<const T*>(op->x_val.p) : reinterpret_cast<const T*>(op->x_valf.p);
     const int grid = (int)std::min<int64_t>((idx->dof + 255) / 256, (int64_t)ctx->num_sms * 8);
     KTimer kt(ctx, KC_MATVEC);
+    if (op->x2_ent.p) {
+        const T* v2 =
+            sizeof(T) == 8 ? reinterpret_cast<const T*>(op->x2_val.p) : reinterpret_cast<const T*>(op->x2_valf.p);
+        const int wgrid = (int)std::min<int64_t>((idx->dof + 7) / 8, (int64_t)ctx->num_sms * 16);
+        cross_rows_kernel<T><<<wgrid, 256, 0, ctx->stream>>>(
+            (int)idx->dof, idx->d, idx->n, idx->k + 1, (int)idx->ntuples, idx->d_levels.p, idx->d_offsets.p,
+            op->npairs, op->x_pairs.p, op->x_kij.p, op->x2_row.p, op->x2_ptr.p, op->x2_len.p, op->x2_ent.p, v2,
+            op->x_grp.p, op->x_off.p, x, y);
+        check_launch("cross_rows_kernel");
+        count_launch(ctx);
+        return;
+    }
     cross_kernel<T><<<grid, 256, 0, ctx->stream>>>(idx->dof, idx->d, idx->n, idx->k + 1, idx->ntuples,
                                                    idx->d_levels.p, idx->d_offsets.p, op->npairs, op->x_pairs.p,
                                                    op->x_kij.p, op->x_ptr.p, op->x_col.p, vals, op->x_rlen.p,

@@ -340,6 +340,14 @@ struct sgk_op {
     DevBuf<float> x_valf;
     DevBuf<int64_t> x_grp, x_off;
     int64_t x_nnz = 0;
+    // the pair form B_ij as one table of 2D rows (shared by every pair, see
+    // cross.cu): entries {t_i | t_j << 16, l_i | l_j << 8} with their values
+    // in FP64 and FP32, row starts, prefix lengths per level and the first
+    // row of every 1D index a_i; empty when the table would be too large
+    DevBuf<int2> x2_ent;
+    DevBuf<double> x2_val;
+    DevBuf<float> x2_valf;
+    DevBuf<int> x2_ptr, x2_len, x2_row;
 };
 constexpr int64_t GMV_LIST_MAX = int64_t(1) << 24;
 

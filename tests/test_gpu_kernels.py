@@ -1,0 +1,59 @@
+"""Kernels at the sizes where their tiling can go wrong, against the FP64 oracle.
+
+Tolerances (relative, coefficient 2-norm) follow tests/test_gpu_parity.py:
+FP64 and double-float components 1e-12 (sums of at most some thousand terms
+in another order, double-float carrying 48 bits), FP32 1e-5.
+"""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+from oracle.index_set import IndexSet as OIndex  # noqa: E402
+from oracle.operator import (DIRICHLET0, PERIODIC, cross_blocks_1d, sipg_1d,  # noqa: E402
+                             sparse_matvec_general)
+from paper_1810_11111_gb300 import sgkiif  # noqa: E402
+
+pytestmark = [pytest.mark.gpu,
+              pytest.mark.skipif(not torch.cuda.is_available(), reason="needs a CUDA device")]
+
+
+def rel(a, b):
+    return float(np.linalg.norm(np.asarray(a) - np.asarray(b)) / max(np.linalg.norm(b), 1e-300))
+
+
+def dev(x, dtype=torch.float64):
+    return torch.as_tensor(np.asarray(x), dtype=dtype, device="cuda").contiguous()
+
+
+@pytest.fixture(scope="module", params=[sgkiif.SGK_FP64, sgkiif.SGK_MIXED], ids=["fp64", "mixed"])
+def ctx(request):
+    c = sgkiif.Context(0, torch.cuda.current_stream().cuda_stream, request.param)
+    yield c
+    c.close()
+
+
+@pytest.mark.parametrize("d,n,k,pairs,bc", [
+    (2, 0, 2, [(0, 1)], PERIODIC),            # one tuple
+    (2, 1, 3, [(0, 1)], DIRICHLET0),
+    (3, 5, 1, [(0, 2)], PERIODIC),            # a direction between the pair
+    (3, 4, 3, [(1, 2)], DIRICHLET0),          # a direction before the pair
+    (4, 3, 2, [(0, 1), (1, 3)], PERIODIC),    # directions after and between
+    (5, 2, 1, [(0, 4), (2, 3)], DIRICHLET0),
+])
+def test_mixed_derivative_rows(ctx, d, n, k, pairs, bc):
+    K = np.diag(np.linspace(1.0, 0.6, d))
+    for i, j in pairs:
+        K[i, j] = K[j, i] = 0.2 + 0.05 * j
+    idx = sgkiif.IndexSet(ctx, d, n, k)
+    op = sgkiif.Operator(ctx, idx, K, bc)
+    P, E = cross_blocks_1d(n, k, bc)
+    dtype, tol = ((torch.float64, 1e-12) if ctx.precision == sgkiif.SGK_FP64 else (torch.float32, 1e-5))
+    xd = dev(np.random.default_rng(d + n).standard_normal(idx.dof), dtype)
+    yd = torch.empty_like(xd)
+    op.matvec(xd.data_ptr(), yd.data_ptr(), ctx.precision)
+    torch.cuda.synchronize()
+    want = sparse_matvec_general(OIndex(d, n, k), sipg_1d(n, k, bc), P, E, K, xd.double().cpu().numpy())
+    assert rel(yd.double().cpu().numpy(), want) <= tol
+    op.close()
+    idx.close()
