@@ -23,10 +23,10 @@
 // added, columns sorted by l(b_i) + l(b_j) so that the truncation at L is a
 // prefix of the row.  cross_rows_kernel adds -K_ij B_ij x to y after the
 // diagonal gather (gmv_kernel): one warp per output, the lanes striding over
-// the row.  Index sets whose table would exceed X2_MAX_ENT entries (the 2D
-// row count times some hundred: level 9, degree 3 is below, level 11 is
-// above) keep cross_kernel: one thread per output, the two factors' rows
-// walked as a sum-factorised double loop.
+// the row.  Index sets whose table would exceed X2_MAX_ENT entries (level 8,
+// degree 2 holds 42 M of the 67 M, level 8, degree 3 twice the limit) keep
+// cross_kernel: one thread per output, the two factors' rows walked as a
+// sum-factorised double loop.
 #include <algorithm>
 #include <cmath>
 #include <map>
