@@ -414,15 +414,18 @@ void quad_build(Quad& Q, const sgk_index* idx, int q, int nspecies, bool need_ja
     gauss_legendre(q, xg, wg);
     const double h = std::ldexp(1.0, -N);
     std::vector<double> B(q * kp1), w1(q);
+    Q.P_host.assign(q * kp1, 0.0);
     for (int g = 0; g < q; ++g) {
         std::vector<double> P(kp1 + 1, 0.0);
         P[0] = 1.0;
         P[1] = xg[g];
         for (int r = 1; r < kp1; ++r) P[r + 1] = ((2 * r + 1) * xg[g] * P[r] - r * P[r - 1]) / (r + 1);
-        for (int r = 0; r < kp1; ++r) B[g * kp1 + r] = std::sqrt(2.0 * r + 1.0) * P[r] / std::sqrt(h);
+        for (int r = 0; r < kp1; ++r) {
+            Q.P_host[g * kp1 + r] = std::sqrt(2.0 * r + 1.0) * P[r];
+            B[g * kp1 + r] = Q.P_host[g * kp1 + r] / std::sqrt(h);
+        }
         w1[g] = 0.5 * h * wg[g];
     }
-    Q.B_host = B;
     Q.w_host = w1;
     Q.B64.upload(B, ctx->stream);
     Q.w64.upload(w1, ctx->stream);

@@ -24,8 +24,9 @@ struct Quad {
     FiberPlan fwd[SGK_MAX_DIM][2], bwd[SGK_MAX_DIM][2];  // [direction][fp64, fp32]
     DevBuf<double> B64, w64;
     DevBuf<float> B32, w32;
-    std::vector<double> B_host, w_host;  // q x (k+1) and q
+    std::vector<double> P_host, w_host;  // q x (k+1) sqrt(2r+1) P_r(xi_g), and q weights h w_g / 2
     bool fused = false;                  // last direction runs in the pencil kernel
+    bool fused_df = false;               // and in double-float for the F passes of mixed mode
 };
 
 int reaction_degree(const ReactionDev& rx);

@@ -421,7 +421,7 @@ void cell_pass(sgk_solver* s, bool jac, T* const* u, T* const* w, T* const* out)
         a.w[sp] = jac ? w[sp] : nullptr;
         a.out[sp] = out[sp];
     }
-    pencil_launch<T>(s->ctx, a, Q.d, Q.kp1, Q.q, s->nspecies, jac, Q.B_host.data(), Q.w_host.data(),
+    pencil_launch<T>(s->ctx, a, Q.d, Q.kp1, Q.q, s->nspecies, jac, Q.P_host.data(), Q.w_host.data(),
                      Q.tab.two_scale.data(), s->rx);
 }
 
@@ -489,8 +489,8 @@ void evalF_df(sgk_solver* s, const double* U, double* F) {
 }
 
 // The reaction passes of every F that fixes the answer: FP64, or in mixed
-// mode double-float where the fused pencil kernel serves the shape.
-bool df_reaction(const sgk_solver* s) { return s->prec == SGK_MIXED && s->Q.fused; }
+// mode double-float for the shapes that have it in the fused pencil kernel.
+bool df_reaction(const sgk_solver* s) { return s->prec == SGK_MIXED && s->Q.fused_df; }
 
 // F(U, t^n + toff): the reaction passes (about 1e-14 relative accuracy in
 // both precision modes), then the source terms in FP64

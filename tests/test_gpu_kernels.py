@@ -12,6 +12,7 @@ torch = pytest.importorskip("torch")
 from oracle.index_set import IndexSet as OIndex  # noqa: E402
 from oracle.operator import (DIRICHLET0, PERIODIC, cross_blocks_1d, sipg_1d,  # noqa: E402
                              sparse_matvec_general)
+from oracle.reaction import Reaction  # noqa: E402
 from paper_1810_11111_gb300 import sgkiif  # noqa: E402
 
 pytestmark = [pytest.mark.gpu,
@@ -56,4 +57,43 @@ def test_mixed_derivative_rows(ctx, d, n, k, pairs, bc):
     want = sparse_matvec_general(OIndex(d, n, k), sipg_1d(n, k, bc), P, E, K, xd.double().cpu().numpy())
     assert rel(yd.double().cpu().numpy(), want) <= tol
     op.close()
+    idx.close()
+
+
+CUBIC = [[(-2.0, (3,)), (0.7, (2,)), (-0.3, (0,))]]
+QUADRATIC = [[(1.5, (2,)), (-0.4, (1,))]]
+PAIR = [[(0.1, (0, 0)), (-1.0, (1, 0)), (1.0, (2, 1)), (0.4, (0, 3))],
+        [(0.9, (0, 0)), (-1.0, (2, 1)), (0.6, (1, 2)), (-0.2, (0, 1))]]
+# every shape of the fused last-direction pass (d, k, reaction) with levels at
+# which its stages differ: one split only, partial and full subtrees, several
+# pencils and several stages per CTA, levels whose cells outnumber the threads
+FUSED = [(2, 1, CUBIC, (1, 2, 5, 9)), (2, 2, CUBIC, (1, 3, 6)), (2, 3, CUBIC, (1, 2, 4, 8)),
+         (2, 1, PAIR, (1, 4)), (2, 2, PAIR, (1, 3, 8)), (2, 3, PAIR, (1, 2, 5)),
+         (2, 1, QUADRATIC, (1, 6)), (2, 2, QUADRATIC, (1, 4, 7)), (2, 3, QUADRATIC, (2, 5)),
+         (3, 1, CUBIC, (1, 2, 5)), (3, 2, CUBIC, (1, 2, 3, 5)), (3, 3, CUBIC, (1, 3, 4)),
+         (3, 1, PAIR, (1, 4)), (3, 2, PAIR, (1, 2, 4)), (3, 3, PAIR, (1, 3)),
+         (3, 1, QUADRATIC, (1, 3)), (3, 2, QUADRATIC, (2, 4)),
+         (4, 1, CUBIC, (1, 2, 4)), (4, 2, CUBIC, (1, 3)), (4, 1, PAIR, (1, 3))]
+
+
+@pytest.mark.parametrize("d,k,rx,n", [(d, k, rx, n) for d, k, rx, levels in FUSED for n in levels])
+def test_fused_reaction_shapes(ctx, d, k, rx, n):
+    S = len(rx)
+    idx = sgkiif.IndexSet(ctx, d, n, k)
+    ops = [sgkiif.Operator(ctx, idx, [1.0] * d) for _ in range(S)]
+    sol = sgkiif.Solver(ctx, ops, rx, 5, 0.01)
+    rng = np.random.default_rng(n)
+    U = [0.5 * (np.arange(idx.dof) == 0) + 0.3 * rng.standard_normal(idx.dof) / np.sqrt(idx.dof) for _ in range(S)]
+    W = [rng.standard_normal(idx.dof) for _ in range(S)]
+    Ud, Wd = dev(np.concatenate(U)), dev(np.concatenate(W))
+    Fd, Jd = torch.empty_like(Ud), torch.empty_like(Ud)
+    sol.reaction_eval(Ud.data_ptr(), Fd.data_ptr())
+    sol.jacobian_apply(Ud.data_ptr(), Wd.data_ptr(), Jd.data_ptr())
+    torch.cuda.synchronize()
+    R = Reaction(OIndex(d, n, k), rx)
+    assert rel(Fd.cpu().numpy(), np.concatenate(R.F(U))) <= 1e-12
+    assert rel(Jd.cpu().numpy(), np.concatenate(R.J(U, W))) <= (1e-12 if ctx.precision == sgkiif.SGK_FP64 else 1e-5)
+    sol.close()
+    for o in ops:
+        o.close()
     idx.close()
