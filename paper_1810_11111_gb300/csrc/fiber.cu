@@ -17,10 +17,12 @@
 // two-scale pyramid on them.
 #include <algorithm>
 
-#include "sgk_dfloat.h"
 #include "sgk_internal.h"
+#include "sgk_twoscale.cuh"
 
 namespace {
+
+using namespace sgk_ts;
 
 __device__ __forceinline__ int level_of(int pos, int kp1) {
     int q = pos / kp1;
@@ -57,20 +59,11 @@ constexpr int PD = 3;
 template <typename T, int MODE, int KP1>
 __global__ void __launch_bounds__(256) pyr_kernel(const FiberItem* __restrict__ items, int nitems,
                                                   const FiberGroup* __restrict__ groups, const T* __restrict__ src,
-                                                  T* __restrict__ dst, const PyrFilt<T> flt, int H, int Nfull) {
+                                                  T* __restrict__ dst, const __grid_constant__ Filt<T, KP1> flt, int H,
+                                                  int Nfull) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     T* tile = reinterpret_cast<T*>(smem_raw);
     __shared__ FiberGroup sg;
-    T Hm[2][KP1][KP1], Gm[2][KP1][KP1];
-#pragma unroll
-    for (int h = 0; h < 2; ++h)
-#pragma unroll
-        for (int r = 0; r < KP1; ++r)
-#pragma unroll
-            for (int s = 0; s < KP1; ++s) {
-                Hm[h][r][s] = flt.H[h][r][s];
-                Gm[h][r][s] = flt.G[h][r][s];
-            }
     const int De = Nfull < PD ? Nfull : PD;  // levels expanded in registers
     const int t = Nfull - De;                // level of the subtree roots
     for (int it = blockIdx.x; it < nitems; it += gridDim.x) {
@@ -118,25 +111,15 @@ __global__ void __launch_bounds__(256) pyr_kernel(const FiberItem* __restrict__ 
                 for (int r = 0; r < KP1; ++r) cell[0][r] = X[r * st + c];
                 // ancestors of the subtree root, level 1..t
                 for (int n = 1; n <= t; ++n) {
-                    const int an = j >> (t - n), h = an & 1, par = an >> 1;
-                    T d[KP1], q[KP1];
+                    const int an = j >> (t - n), par = an >> 1;
+                    const bool h = an & 1;
+                    T d[KP1], A[KP1], B[KP1];
 #pragma unroll
-                    for (int r = 0; r < KP1; ++r) d[r] = n <= Np ? X[((KP1 << (n - 1)) + par * KP1 + r) * st + c] : T(0);
+                    for (int r = 0; r < KP1; ++r)
+                        d[r] = n <= Np ? X[((KP1 << (n - 1)) + par * KP1 + r) * st + c] : zero<T>();
+                    split_node<T, KP1>(cell[0], d, flt, A, B);
 #pragma unroll
-                    for (int s2 = 0; s2 < KP1; ++s2) {
-                        T acc = T(0);
-#pragma unroll
-                        for (int r = 0; r < KP1; ++r) {
-                            // select, not index: a runtime index would put the
-                            // filters in local memory
-                            const T hf = h ? Hm[1][r][s2] : Hm[0][r][s2];
-                            const T gf = h ? Gm[1][r][s2] : Gm[0][r][s2];
-                            acc += hf * cell[0][r] + gf * d[r];
-                        }
-                        q[s2] = acc;
-                    }
-#pragma unroll
-                    for (int r = 0; r < KP1; ++r) cell[0][r] = q[r];
+                    for (int r = 0; r < KP1; ++r) cell[0][r] = add_signed(A[r], B[r], h, h);
                 }
                 // expand the subtree (children written over consumed parents)
 #pragma unroll
@@ -146,21 +129,16 @@ __global__ void __launch_bounds__(256) pyr_kernel(const FiberItem* __restrict__ 
 #pragma unroll
                         for (int i = (1 << l) - 1; i >= 0; --i) {
                             const int par = (j << l) + i;
-                            T d[KP1], p[KP1];
+                            T d[KP1], A[KP1], B[KP1];
 #pragma unroll
-                            for (int r = 0; r < KP1; ++r) {
-                                p[r] = cell[i][r];
-                                d[r] = n <= Np ? X[((KP1 << (n - 1)) + par * KP1 + r) * st + c] : T(0);
+                            for (int r = 0; r < KP1; ++r)
+                                d[r] = n <= Np ? X[((KP1 << (n - 1)) + par * KP1 + r) * st + c] : zero<T>();
+                            split_node<T, KP1>(cell[i], d, flt, A, B);
+#pragma unroll
+                            for (int s2 = 0; s2 < KP1; ++s2) {
+                                cell[2 * i][s2] = add(A[s2], B[s2]);
+                                cell[2 * i + 1][s2] = sub(A[s2], B[s2]);
                             }
-#pragma unroll
-                            for (int h = 0; h < 2; ++h)
-#pragma unroll
-                                for (int s2 = 0; s2 < KP1; ++s2) {
-                                    T acc = T(0);
-#pragma unroll
-                                    for (int r = 0; r < KP1; ++r) acc += Hm[h][r][s2] * p[r] + Gm[h][r][s2] * d[r];
-                                    cell[2 * i + h][s2] = acc;
-                                }
                         }
                     }
                 }
@@ -189,24 +167,17 @@ __global__ void __launch_bounds__(256) pyr_kernel(const FiberItem* __restrict__ 
                         const bool keep = n <= Np;
 #pragma unroll
                         for (int i = 0; i < (1 << l); ++i) {
-                            T x0[KP1], x1[KP1];
+                            T sum[KP1], dif[KP1], d[KP1];
 #pragma unroll
                             for (int s2 = 0; s2 < KP1; ++s2) {
-                                x0[s2] = cell[2 * i][s2];
-                                x1[s2] = cell[2 * i + 1][s2];
+                                sum[s2] = add(cell[2 * i][s2], cell[2 * i + 1][s2]);
+                                dif[s2] = sub(cell[2 * i][s2], cell[2 * i + 1][s2]);
                             }
                             const int par = (j << l) + i;
+                            merge_node<T, KP1>(sum, dif, flt, cell[i], d);
+                            if (keep)
 #pragma unroll
-                            for (int r = 0; r < KP1; ++r) {
-                                T sp = T(0), sd = T(0);
-#pragma unroll
-                                for (int s2 = 0; s2 < KP1; ++s2) {
-                                    sp += Hm[0][r][s2] * x0[s2] + Hm[1][r][s2] * x1[s2];
-                                    sd += Gm[0][r][s2] * x0[s2] + Gm[1][r][s2] * x1[s2];
-                                }
-                                cell[i][r] = sp;
-                                if (keep) Y[((KP1 << (n - 1)) + par * KP1 + r) * st + c] = sd;
-                            }
+                                for (int r = 0; r < KP1; ++r) Y[((KP1 << (n - 1)) + par * KP1 + r) * st + c] = d[r];
                         }
                     }
                 }
@@ -222,22 +193,18 @@ __global__ void __launch_bounds__(256) pyr_kernel(const FiberItem* __restrict__ 
                 const bool keep = n <= Np;
                 for (int u = threadIdx.x; u < (nc << (n - 1)); u += blockDim.x) {
                     const int c = u % nc, par = u / nc;
-                    T x0[KP1], x1[KP1];
+                    T sum[KP1], dif[KP1], p[KP1], d[KP1];
 #pragma unroll
                     for (int s2 = 0; s2 < KP1; ++s2) {
-                        x0[s2] = cur[((2 * par) * KP1 + s2) * st + c];
-                        x1[s2] = cur[((2 * par + 1) * KP1 + s2) * st + c];
+                        const T x0 = cur[((2 * par) * KP1 + s2) * st + c], x1 = cur[((2 * par + 1) * KP1 + s2) * st + c];
+                        sum[s2] = add(x0, x1);
+                        dif[s2] = sub(x0, x1);
                     }
+                    merge_node<T, KP1>(sum, dif, flt, p, d);
 #pragma unroll
                     for (int r = 0; r < KP1; ++r) {
-                        T sp = T(0), sd = T(0);
-#pragma unroll
-                        for (int s2 = 0; s2 < KP1; ++s2) {
-                            sp += Hm[0][r][s2] * x0[s2] + Hm[1][r][s2] * x1[s2];
-                            sd += Gm[0][r][s2] * x0[s2] + Gm[1][r][s2] * x1[s2];
-                        }
-                        nxt[(par * KP1 + r) * st + c] = sp;
-                        if (keep) Y[((KP1 << (n - 1)) + par * KP1 + r) * st + c] = sd;
+                        nxt[(par * KP1 + r) * st + c] = p[r];
+                        if (keep) Y[((KP1 << (n - 1)) + par * KP1 + r) * st + c] = d[r];
                     }
                 }
                 __syncthreads();
@@ -262,13 +229,6 @@ template <typename T>
 void launch_pyr(sgk_ctx* ctx, const FiberPlan& plan, int mode, const T* src, T* dst, int H, int kp1,
                 const double* two_scale) {
     if (plan.nitems == 0) return;
-    PyrFilt<T> f{};
-    for (int h = 0; h < 2; ++h)
-        for (int r = 0; r < kp1; ++r)
-            for (int s = 0; s < kp1; ++s) {
-                f.H[h][r][s] = (T)two_scale[h * kp1 * kp1 + r * kp1 + s];
-                f.G[h][r][s] = (T)two_scale[(2 + h) * kp1 * kp1 + r * kp1 + s];
-            }
     int Nfull = 0;
     while ((kp1 << Nfull) < H) ++Nfull;
     const int grid = std::min(plan.nitems, ctx->num_sms * 8);
@@ -277,8 +237,8 @@ void launch_pyr(sgk_ctx* ctx, const FiberPlan& plan, int mode, const T* src, T* 
 #define SGK_PYR_CASE(M, K)                                                                                   \
     if (mode == M && kp1 == K) {                                                                             \
         allow_max_dynamic_smem(ctx->smem_optin, pyr_kernel<T, M, K>);          \
-        pyr_kernel<T, M, K><<<grid, 256, smem, ctx->stream>>>(plan.items.p, plan.nitems, plan.groups.p, src, dst, \
-                                                              f, H, Nfull);                                 \
+        pyr_kernel<T, M, K><<<grid, 256, smem, ctx->stream>>>(plan.items.p, plan.nitems, plan.groups.p, src,     \
+                                                                  dst, make_filt<T, K>(two_scale), H, Nfull);  \
     }
     SGK_PYR_CASE(FIBER_FWD, 2)
     SGK_PYR_CASE(FIBER_FWD, 3)

@@ -280,13 +280,6 @@ struct FiberPlan {
 void finalize_plan(FiberPlan& plan, std::vector<FiberGroup>& groups, int kp1, int H, int mode, size_t elem_bytes,
                    size_t smem_budget, long long src_size, long long dst_size, cudaStream_t s);
 
-// Two-scale filters for the pyramid kernels (entries beyond k+1 unused).
-template <typename T>
-struct PyrFilt {
-    T H[2][4][4];
-    T G[2][4][4];
-};
-
 // Change of basis along one direction (plan mode FIBER_FWD or FIBER_BWD) by
 // the two-scale pyramid; two_scale as in Tables1D.
 template <typename T>
