@@ -11,17 +11,27 @@
 // (the norm of w'' follows by Pythagoras; near breakdown a third barrier
 // sums it explicitly); with the double-float matvec one more barrier at the
 // start publishes the pairs of v / gamma for the first gathers (pairs of
-// FP32 numbers cannot hold an unnormalised v of tiny magnitude).  The
-// cross-CTA sums are exact: every CTA adds its
-// partials, as 128-bit fixed-point integers, into integer accumulators with
-// atomic adds, and after the barrier every CTA reads the same totals, so all
-// CTAs hold bitwise equal h1, h2 and beta and take the same breakdown
+// FP32 numbers cannot hold an unnormalised v of tiny magnitude).  The sums,
+// inside a CTA and across CTAs, are exact: partials become 128-bit
+// fixed-point integers, added by shuffles, then into integer accumulators
+// with atomic adds, and after the barrier every CTA reads the same totals, so
+// all CTAs hold bitwise equal h1, h2 and beta and take the same breakdown
 // decision without another barrier; the results do not depend on the order
 // in which CTAs arrive.  The next matvec gathers the unnormalised w' and
-// forms A v_{j+1} = (A w' - Z h2) / beta from the stored raw outputs Z; the
-// two w buffers alternate so that those gathers never race with the writes
-// of the next step.  Accumulator sets rotate over three buffers for the same
-// reason.
+// forms A v_{j+1} = (A w' - Z h2) / beta from the stored raw outputs Z; it
+// starts before 1 / beta is known.  The two w buffers alternate so that those
+// gathers never race with the writes of the next step.  Accumulator sets
+// rotate over three steps for the same reason.
+//
+// Bound: latency.  A step at 5 184 coefficients, 25 columns (24 000 clocks):
+// 2 x 4 950 for a barrier and the read of the sums behind it (additions to
+// arrive, release, poll, read, each an L2 round trip), 2 x 1 900 for inner
+// products, 2 x 1 750 for the updates, 2 500 for the gathers, 3 500 for
+// staging the gathered vector, the rest scalars.  Per exponential, before and
+// after sums by integers, updates over all four schedulers, scalars beside
+// the gathers and the staged vector: 350 -> 300 us there, 541 -> 505 at
+// 18 576 x 30, 684 -> 640 at 11 520 x 40, 449 -> 388 at 8 832 x 30, 1240 ->
+// 1184 at 44 032 x 30, 15.9 -> 13.5 ms at 850 176 x 30.
 //
 // Barriers are counters in global memory with a bounded wait: a CTA that
 // waits longer than the limit sets an error flag and returns, and every
@@ -59,8 +69,8 @@ int64_t arnoldi_persistent_max_n(const sgk_ctx* ctx) {
 
 size_t arnoldi_persistent_pbuf_size(const sgk_ctx* ctx, int M) {
     (void)M;
-    // per-CTA norm partials, then the three fixed-point accumulator sets
-    return (size_t)ctx->num_sms + 3 * sgk_arn::FX_SET;
+    // per-CTA norm partials, then (16-byte aligned) the fixed-point accumulator sets
+    return ((size_t)ctx->num_sms + 1) / 2 * 2 + sgk_arn::FX_SETS * sgk_arn::FX_SET;
 }
 
 static size_t smem_budget(const sgk_ctx* ctx) {
@@ -134,17 +144,18 @@ ArnPrep arnoldi_prepare(sgk_ctx* ctx, const sgk_op* op, const PersistentWork& pw
     a.Z = pw.Z;
     a.H = kw.H;
     a.pbuf = pw.pbuf;
-    a.acc = reinterpret_cast<unsigned long long*>(pw.pbuf + ctx->num_sms);
+    a.acc = reinterpret_cast<unsigned long long*>(pw.pbuf + (ctx->num_sms + 1) / 2 * 2);
     // fixed-point scales from the bound ||A v|| <= ||A|| for ||v|| = 1:
     // |partial| <= 2^(e - 1) with e = ceil(log2 ||A||) + 1, entered as
-    // floor(p 2^(110 - e)), so |P| < 2^110; the squared norm likewise with 2e
+    // trunc(p 2^(110 - e)), so |P| < 2^110; the squared norm likewise with 2e
     {
         const double an = op->anorm > 0.0 ? op->anorm : 1.0;
         const int e = std::min(400, std::max(-400, (int)std::ceil(std::log2(an)) + 1));
-        a.sc_h = std::ldexp(1.0, 46 - e);
-        a.isc_h = std::ldexp(1.0, e - 110);
-        a.sc_n = std::ldexp(1.0, 46 - 2 * e);
-        a.isc_n = std::ldexp(1.0, 2 * e - 110);
+        a.sh_h = 110 - e;
+        a.sh_n = 110 - 2 * e;
+        // H has at most M + 1 entries a column, and no column is longer than
+        // ||A v|| (twice, for rounding)
+        a.no_brk = std::ldexp(1e-24 * 2.0 * (M + 1), 2 * e);
     }
     a.bar = pw.bar;
     // failure injection on the host: with SGK_TEST_BARRIER_STALL set, every
@@ -178,20 +189,43 @@ ArnPrep arnoldi_prepare(sgk_ctx* ctx, const sgk_op* op, const PersistentWork& pw
     a.smem_vz = 0;
     a.smem_loc = 0;
     a.list_cap = 0;
-    if (has_list && ws + vz + lst <= budget) {
-        a.smem_vz = 1;
-        a.list_cap = (int)std::max<int64_t>(list_ent, 1);
-    } else if (has_list && ws + lst <= budget) {
-        a.list_cap = (int)std::max<int64_t>(list_ent, 1);
-    } else {
-        a.smem_vz = ws + vz <= budget;
-        a.smem_loc = ws + (a.smem_vz ? vz : 0) + lb <= budget;
-    }
-    const size_t smem = ws + (a.smem_vz ? vz : 0) + (a.list_cap ? lst : 0) + (a.smem_loc ? lb : 0);
-    // mixed precision: the matvec in double-float arithmetic (~1e-14
-    // relative; FP64 issue on this part is 1/64 of FP32), with the gather lists
     a.cvk2 = op->gmv_cvk2.p;
-    a.df = ctx->precision == SGK_MIXED && a.list_cap > 0 && op->gmv_cvk2.p != nullptr;
+    // The gathered vector staged in shared memory, where it fits beside the
+    // slices of w and the entries (10 bytes each): copied as a whole past L1,
+    // which is empty after every step's acquire, the gathers themselves take
+    // 2 800 to 4 200 clocks a step at 8 832 and 11 520 coefficients on 152
+    // CTAs (the whole process 650 and 423 us, 690 and 449 with gathers through
+    // L1).  The slices of V and Z go to shared memory next.  With the entries
+    // streamed from L2 beside a staged vector (18 576 coefficients) the copy
+    // and the stream cost more than they saved: 564 against 541 us.
+    const bool mixed = ctx->precision == SGK_MIXED;
+    const size_t xb = sizeof(double) * (size_t)((n + 1) / 2 * 2);
+    const size_t lst10 = sgk_arn::arn_eoff_bytes((int)E, d) + 10 * (size_t)std::max<int64_t>(list_ent, 1);
+    a.ei = op->gmv_ei.p;
+    a.ev = op->gmv_ev.p;
+    a.ev2 = op->gmv_ev2.p;
+    a.xs = a.ei != nullptr && (mixed ? a.ev2 != nullptr : a.ev != nullptr) && xb + ws + lst10 <= budget;
+    size_t smem;
+    if (a.xs) {
+        a.smem_vz = xb + ws + lst10 + vz <= budget;
+        a.list_cap = (int)std::max<int64_t>(list_ent, 1);
+        smem = xb + ws + lst10 + (a.smem_vz ? vz : 0);
+        a.df = mixed;
+    } else {
+        if (has_list && ws + vz + lst <= budget) {
+            a.smem_vz = 1;
+            a.list_cap = (int)std::max<int64_t>(list_ent, 1);
+        } else if (has_list && ws + lst <= budget) {
+            a.list_cap = (int)std::max<int64_t>(list_ent, 1);
+        } else {
+            a.smem_vz = ws + vz <= budget;
+            a.smem_loc = ws + (a.smem_vz ? vz : 0) + lb <= budget;
+        }
+        smem = ws + (a.smem_vz ? vz : 0) + (a.list_cap ? lst : 0) + (a.smem_loc ? lb : 0);
+        // mixed precision: the matvec in double-float arithmetic (~1e-14
+        // relative; FP64 issue on this part is 1/64 of FP32), with the gather lists
+        a.df = mixed && a.list_cap > 0 && op->gmv_cvk2.p != nullptr;
+    }
     ArnPrep out;
     out.a = a;
     out.smem = smem;

@@ -27,6 +27,14 @@ struct ArnArgs {
     // vectors (w0, w1) and Z then hold (hi, lo) pairs instead of doubles
     const float2* cvk2;
     int df;
+    // xs: the whole gathered vector (8 n bytes) is staged in shared memory
+    // before every matvec, and the gathers read it there; the entries (at
+    // most list_cap) then come with their own values (entry q: ei[q], and
+    // ev[q] or ev2[q]), staged in shared memory too
+    int xs;
+    const unsigned short* ei;
+    const double* ev;
+    const float2* ev2;
     const double* v;
     double* V;  // column c at V + c n
     double* w0;
@@ -34,11 +42,14 @@ struct ArnArgs {
     double* Z;     // raw matvec outputs A v_c, column c at Z + c n (own slices only)
     double* H;     // (M + 1) x M row-major
     double* pbuf;  // gridDim.x per-CTA partials of a norm (gamma, explicit fallback)
-    unsigned long long* acc;  // 3 rotating sets of FX_COLS fixed-point accumulators (FX_LIMBS words each)
+    unsigned long long* acc;  // FX_SETS rotating sets of FX_COLS fixed-point accumulators (FX_LIMBS words each)
     // fixed-point scales: a partial p of an inner product enters as
-    // floor(p sc 2^64), the sum is read back times isc; _h for the columns of
-    // V^T w (|p| <= ||A||), _n for ||w'||^2 (|p| <= ||A||^2)
-    double sc_h, isc_h, sc_n, isc_n;
+    // trunc(p 2^sh); _h for the columns of V^T w (|p| <= ||A||), _n for
+    // ||w'||^2 (|p| <= ||A||^2)
+    int sh_h, sh_n;
+    // a ||w''||^2 above this is no breakdown whatever H holds (its entries
+    // are bounded by ||A||): 1e-24 times a bound on ||H||_F^2
+    double no_brk;
     unsigned* bar;  // [0] barrier arrivals (zero at launch), [1] error flag
     unsigned bar_extra;  // added to every barrier target: 0, or 1 to make the waits run out (failure test)
     KrylovScalars* ks;
@@ -46,11 +57,12 @@ struct ArnArgs {
 };
 
 constexpr int FX_COLS = SGK_MAX_KRYLOV + 2;  // columns of one accumulator set
-constexpr int FX_LIMBS = 4;                   // three 56-bit limbs and a count of invalid partials
+constexpr int FX_LIMBS = 4;                   // words of a column, see fx_add
 // copies of every accumulator: CTA b adds into copy b % FX_COPIES, so that
 // the CTAs arriving together do not serialise on the same words
 constexpr int FX_COPIES = 8;
 constexpr int FX_SET = FX_COPIES * FX_COLS * FX_LIMBS;  // words of one set
+constexpr int FX_SETS = 6;                              // two phases a step, three steps in rotation
 
 // Bytes of the staged entry offsets of a slice of E outputs (D per output
 // and one end), rounded up to 16.
@@ -95,6 +107,101 @@ __device__ __forceinline__ bool grid_barrier(unsigned* bar, unsigned target, int
     __syncthreads();
     return *s_ok != 0;
 }
+
+// Gather of one output from the staged x: the entries q0 .. qe of its merged
+// row (all directions), entry q0 + i in virtual lane i mod 8 as in
+// gmv_accumulate, one chain each; a thread's 8 / G virtual lanes are
+// independent chains side by side.  The sum does not depend on G.
+template <int G>
+__device__ __forceinline__ double gather_staged(const unsigned short* ei, const double* ev, const double* xs, int q0,
+                                                int qe, int r, int ncorr, const double* hc, const double* zc,
+                                                int64_t zld) {
+    constexpr int VL = 8, PER = VL / G;
+    double b[PER];
+#pragma unroll
+    for (int k = 0; k < PER; ++k) b[k] = 0.0;
+#pragma unroll 2
+    for (int q = q0 + r; q < qe; q += VL)
+#pragma unroll
+        for (int k = 0; k < PER; ++k)
+            if (q + k * G < qe) b[k] += ev[q + k * G] * xs[ei[q + k * G]];
+    if (ncorr > 0) {
+        double c0[PER];
+#pragma unroll
+        for (int k = 0; k < PER; ++k) c0[k] = 0.0;
+        for (int c = r; c < ncorr; c += VL)
+#pragma unroll
+            for (int k = 0; k < PER; ++k)
+                if (c + k * G < ncorr) c0[k] += hc[c + k * G] * zc[(c + k * G) * zld];
+#pragma unroll
+        for (int k = 0; k < PER; ++k) b[k] -= c0[k];
+    }
+#pragma unroll
+    for (int o = 1; o < G; o <<= 1)
+#pragma unroll
+        for (int k = 0; k < PER; ++k) b[k] += __shfl_xor_sync(0xffffffffu, b[k], o);
+#pragma unroll
+    for (int m = 1; m < PER; m <<= 1)
+#pragma unroll
+        for (int k = 0; k + m < PER; k += 2 * m) b[k] += b[k + m];
+    return b[0];
+}
+template <int G>
+__device__ __forceinline__ df64 gather_staged(const unsigned short* ei, const float2* ev, const float2* xs, int q0,
+                                              int qe, int r, int ncorr, const float2* hc, const float2* zc,
+                                              int64_t zld) {
+    constexpr int VL = 8, PER = VL / G;
+    df64 b[PER];
+#pragma unroll
+    for (int k = 0; k < PER; ++k) b[k] = df_make(0.f, 0.f);
+#pragma unroll 2
+    for (int q = q0 + r; q < qe; q += VL)
+#pragma unroll
+        for (int k = 0; k < PER; ++k)
+            if (q + k * G < qe)
+                b[k] = df_add(b[k], df_mul(df_from_float2(ev[q + k * G]), df_from_float2(xs[ei[q + k * G]])));
+    if (ncorr > 0) {
+        df64 c0[PER];
+#pragma unroll
+        for (int k = 0; k < PER; ++k) c0[k] = df_make(0.f, 0.f);
+        for (int c = r; c < ncorr; c += VL)
+#pragma unroll
+            for (int k = 0; k < PER; ++k)
+                if (c + k * G < ncorr)
+                    c0[k] = df_add(c0[k], df_mul(df_from_float2(hc[c + k * G]), df_from_float2(zc[(c + k * G) * zld])));
+#pragma unroll
+        for (int k = 0; k < PER; ++k) b[k] = df_add(b[k], df_neg(c0[k]));
+    }
+#pragma unroll
+    for (int o = 1; o < G; o <<= 1)
+#pragma unroll
+        for (int k = 0; k < PER; ++k) b[k] = df_add(b[k], df_shfl_xor(b[k], o));
+#pragma unroll
+    for (int m = 1; m < PER; m <<= 1)
+#pragma unroll
+        for (int k = 0; k + m < PER; k += 2 * m) b[k] = df_add(b[k], b[k + m]);
+    return b[0];
+}
+
+// asynchronous copy of n 8-byte elements into shared memory by the CTA (16
+// bytes at a time, past L1, when the source is aligned)
+__device__ __forceinline__ void stage_vector(void* dst, const void* src, int64_t n) {
+    const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+    const char* s = static_cast<const char*>(src);
+    if ((reinterpret_cast<uintptr_t>(src) & 15) == 0) {
+        for (int i = threadIdx.x; i < (int)(n >> 1); i += PT)
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d + 16 * i), "l"(s + 16 * (size_t)i) : "memory");
+        if ((n & 1) && threadIdx.x == 0)
+            asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(d + 8 * (unsigned)(n - 1)),
+                         "l"(s + 8 * (size_t)(n - 1))
+                         : "memory");
+    } else {
+        for (int i = threadIdx.x; i < (int)n; i += PT)
+            asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(d + 8 * i), "l"(s + 8 * (size_t)i) : "memory");
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+}
+__device__ __forceinline__ void stage_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
 __device__ __forceinline__ double warp_sum(double a) {
 #pragma unroll
@@ -144,133 +251,233 @@ __device__ __forceinline__ void colsum(const double* P, int nb, int ncols, doubl
     }
 }
 
-// out[c] = sum_{u < ne} Vl[c vld + u] ws[u], c < ncols (this CTA's slice,
-// Vl/vld its basis columns in shared or global memory); with norm, also
-// out[ncols] = sum ws[u]^2; out in shared memory, complete on return.  CH
-// threads per column (a power of two, the most with nt CH <= PT, at most 32)
-// sum strided elements in two chains; the CH partials of a column are added
-// through shared memory in a fixed tree (quarters by four threads, then the
-// four by one), so the FP64 work is spread over every warp of the CTA (FP64
-// issue is slow on this part: spreading it, not shortening chains, is what
-// pays).  tmp holds PT doubles, tmp2 4 (SGK_MAX_KRYLOV + 2).
-__device__ __forceinline__ void slice_dots(const double* Vl, int64_t vld, int ncols, const double* ws, int ne,
-                                           double* out, bool norm, double* tmp, double* tmp2) {
-    const int nt = ncols + (norm ? 1 : 0);
-    int CH = 32;
-    while (CH > 1 && nt * CH > PT) CH >>= 1;
-    const int t = threadIdx.x;
-    if (t < nt * CH) {
-        const int c = t / CH, k = t - (t / CH) * CH;
-        const double* vc = c < ncols ? Vl + c * vld : ws;
-        double a = 0.0, b = 0.0;
-        int u = k;
-        for (; u + CH < ne; u += 2 * CH) {
-            a += vc[u] * ws[u];
-            b += vc[u + CH] * ws[u + CH];
-        }
-        if (u < ne) a += vc[u] * ws[u];
-        tmp[t] = a + b;
-    }
-    __syncthreads();
-    const int Q = CH < 4 ? CH : 4, per = CH / Q;
-    if (t < nt * Q) {
-        const double* p = tmp + t * per;  // column t / Q, quarter t % Q
-        double a = p[0];
-        for (int i = 1; i < per; ++i) a += p[i];
-        tmp2[t] = a;
-    }
-    __syncthreads();
-    if (t < nt) {
-        const double* p = tmp2 + t * Q;
-        out[t] = Q == 4 ? (p[0] + p[1]) + (p[2] + p[3]) : (Q == 2 ? p[0] + p[1] : p[0]);
-    }
-    __syncthreads();
-}
-
-// Exact sums across CTAs.  A partial p is taken as the 128-bit integer
-// P = trunc(p sc 2^64) (two's complement; sc a power of two chosen from a
-// bound on |p| so that |P| < 2^110) and added to per-column accumulators of
-// three 56-bit limbs with 64-bit integer atomic adds.  Integer addition is
+// Exact sums.  A partial p of an inner product is taken as the 128-bit
+// integer P = trunc(p 2^sh) (two's complement; sh from a bound on |p| such
+// that |P| < 2^110), formed and added by integer operations: the FP64 pipe
+// issues one warp instruction per 64 clocks, so a tree of FP64 additions and
+// its barriers cost more than the products they add.  Integer addition is
 // associative: the total is exact whatever the order of arrival, and every
-// CTA reads back the same value, in every run.  A partial that is not
-// finite or outside the range is counted in the fourth word and makes the
-// column NaN.
+// CTA reads back the same value, in every run.
+struct Fix {
+    unsigned long long lo, hi;
+    bool bad;  // not finite or outside the range
+};
+__device__ __forceinline__ Fix fx_fixed(double p, int sh) {
+    const unsigned long long bits = (unsigned long long)__double_as_longlong(p);
+    int e = (int)((bits >> 52) & 0x7ff);
+    unsigned long long m = bits & 0xfffffffffffffull;
+    Fix f;
+    f.bad = e == 0x7ff;
+    if (e) m |= 1ull << 52;
+    else e = 1;
+    const int s = e - 1075 + sh;  // P = m 2^s
+    f.bad = f.bad || s > 61;
+    if (s >= 0) {
+        f.lo = m << (s & 63);
+        f.hi = s ? m >> ((64 - s) & 63) : 0ull;
+    } else {
+        f.lo = s > -64 ? m >> (-s & 63) : 0ull;
+        f.hi = 0ull;
+    }
+    if (f.bad) f.lo = f.hi = 0ull;
+    if ((long long)bits < 0) {
+        f.lo = ~f.lo + 1ull;
+        f.hi = ~f.hi + (f.lo == 0ull ? 1ull : 0ull);
+    }
+    return f;
+}
+__device__ __forceinline__ void fx_sum(Fix& f, unsigned long long lo, unsigned long long hi) {
+    f.lo += lo;
+    f.hi += hi + (f.lo < lo ? 1ull : 0ull);
+}
+__device__ __forceinline__ Fix fx_warp_sum(Fix f) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+        fx_sum(f, __shfl_xor_sync(0xffffffffu, f.lo, o), __shfl_xor_sync(0xffffffffu, f.hi, o));
+    f.bad = __any_sync(0xffffffffu, f.bad);
+    return f;
+}
+// P 2^-sh rounded to FP64, and the same number as a double-float pair (its
+// leading 24 bits and the next 24) when df is not null
+__device__ __forceinline__ double fx_value(Fix f, int sh, float2* df = nullptr) {
+    const bool neg = (long long)f.hi < 0;
+    if (neg) {
+        f.lo = ~f.lo + 1ull;
+        f.hi = ~f.hi + (f.lo == 0ull ? 1ull : 0ull);
+    }
+    if (f.bad || (f.lo | f.hi) == 0ull) {
+        if (df) *df = f.bad ? make_float2(__int_as_float(0x7fc00000), 0.f) : make_float2(0.f, 0.f);
+        return f.bad ? __longlong_as_double(0x7ff8000000000000ll) : 0.0;
+    }
+    // leading bit to bit 127
+    if (f.hi == 0ull) {
+        f.hi = f.lo;
+        f.lo = 0ull;
+        sh += 64;
+    }
+    const int lz = __clzll((long long)f.hi);
+    if (lz) f.hi = (f.hi << lz) | (f.lo >> (64 - lz));
+    f.lo <<= lz;
+    const int ex = 127 - lz - sh;  // value = 1.xxx 2^ex
+    if (df) {
+        const float scale = ex > -100 && ex < 127 ? __int_as_float((ex + 127) << 23) : 0.f;
+        const float s = (neg ? -scale : scale) * 0x1p-23f;
+        const float h = (float)(unsigned)(f.hi >> 40), l = (float)(unsigned)((f.hi >> 16) & 0xffffffull);
+        *df = ex >= 127 ? make_float2(__int_as_float(neg ? 0xff800000 : 0x7f800000), 0.f)
+                        : make_float2(h * s, l * (s * 0x1p-24f));
+    }
+    unsigned long long m = f.hi >> 11;
+    const unsigned rem = (unsigned)(f.hi & 0x7ffull) | (f.lo ? 1u : 0u);
+    m += rem > 0x400u || (rem == 0x400u && (m & 1ull)) ? 1ull : 0ull;  // to nearest, ties to even
+    const unsigned long long bits = ((unsigned long long)(ex + 1022) << 52) + m;
+    return __longlong_as_double((long long)(bits | (neg ? 1ull << 63 : 0ull)));
+}
+// Adds a CTA's sum into its copy of a column: P in three words of 56, 56 and
+// 16 bits, whose sums over 255 CTAs fit 64; the fourth word counts invalid
+// partials.
 constexpr unsigned long long FX_M56 = (1ull << 56) - 1;
-
-__device__ __forceinline__ void fx_red(unsigned long long* a, double p, double sc) {
-    const double q = p * sc;  // |q| < 2^46 when the bound holds
-    const double aq = fabs(q);
-    if (!(aq < 1125899906842624.0)) {  // 2^50; false for NaN
+__device__ __forceinline__ void fx_add(unsigned long long* a, const Fix& f) {
+    if (f.bad) {
         atomicAdd(a + 3, 1ull);
         return;
     }
-    // |P| = H 2^64 + L: the integer part, and the fraction (exact for a
-    // non-negative double) scaled to 64 bits
-    const double hd = floor(aq);
-    unsigned long long H = __double2ull_rn(hd);
-    unsigned long long L = __double2ull_rd((aq - hd) * 18446744073709551616.0);
-    if (q < 0.0) {  // two's complement of the 128-bit magnitude
-        L = ~L + 1ull;
-        H = ~H + (L == 0ull ? 1ull : 0ull);
-    }
-    atomicAdd(a, L & FX_M56);
-    atomicAdd(a + 1, ((L >> 56) | (H << 8)) & FX_M56);
-    atomicAdd(a + 2, (unsigned long long)((long long)H >> 48));
+    atomicAdd(a, f.lo & FX_M56);
+    atomicAdd(a + 1, ((f.lo >> 56) | (f.hi << 8)) & FX_M56);
+    atomicAdd(a + 2, (unsigned long long)((long long)f.hi >> 48));
 }
 
-// The accumulated sum of one column (its FX_COPIES copies, FX_COLS
-// columns apart) times isc; L2 loads: the limbs were added by other CTAs.
-__device__ __forceinline__ double fx_value(const unsigned long long* a, double isc) {
-    unsigned long long s0 = 0ull, s1 = 0ull, s2 = 0ull, bad = 0ull;
-#pragma unroll
-    for (int k = 0; k < FX_COPIES; ++k) {
-        const unsigned long long* c = a + (size_t)k * FX_COLS * FX_LIMBS;
-        s0 += __ldcg(c);
-        s1 += __ldcg(c + 1);
-        s2 += __ldcg(c + 2);
-        bad += __ldcg(c + 3);
-    }
-    if (bad != 0ull) return __longlong_as_double(0x7ff8000000000000ll);
-    // s0 + s1 2^56 + s2 2^112 (s2 signed) as hi 2^64 + lo; the limb sums
-    // stay below 2^64: at most one term below 2^56 per CTA
-    unsigned long long lo = s0 + (s1 << 56);
-    unsigned long long hi = (s1 >> 8) + (s2 << 48) + (lo < s0 ? 1ull : 0ull);
-    const bool neg = (long long)hi < 0;
-    if (neg) {  // magnitude, so that the conversion below keeps full relative precision
-        lo = ~lo + 1ull;
-        hi = ~hi + (lo == 0ull ? 1ull : 0ull);
-    }
-    const double m = __ull2double_rn(hi) * 18446744073709551616.0 + __ull2double_rn(lo);
-    return (neg ? -m : m) * isc;
-}
-
-// w -= V[:, :ncols] h on this CTA's slice, one thread per element (four
-// independent chains).  Writes the staged slice ws, the global w when w is
-// not null (or its double-float pair to wdf when that is not null), and when
-// vg is not null the next basis column w * inv to vg (global, slice offset
-// included) and vs (shared, or null).
-__device__ __forceinline__ void slice_update(const double* Vl, int64_t vld, int ncols, const double* h, double* w,
-                                             double* ws, int64_t lo, int ne, double* vg, double* vs, double inv,
-                                             float2* wdf = nullptr) {
-    for (int u = threadIdx.x; u < ne; u += PT) {
-        const double* vi = Vl + u;
-        double a0 = 0.0, a1 = 0.0, a2 = 0.0, a3 = 0.0;
-        int c = 0;
-        for (; c + 3 < ncols; c += 4) {
-            a0 += vi[c * vld] * h[c];
-            a1 += vi[(c + 1) * vld] * h[c + 1];
-            a2 += vi[(c + 2) * vld] * h[c + 2];
-            a3 += vi[(c + 3) * vld] * h[c + 3];
+// out[c] (and its pair in outdf when that is not null) = the sum of column c
+// < nt (the last one scaled by sh_last), after the barrier that follows the
+// additions; by the whole CTA: one thread per column and copy loads the
+// copy's four words (two 16-byte L2 loads: other CTAs added them), the copies
+// are added by shuffles.  (One thread per column loading all 32 words takes
+// 1 900 clocks.  Words that count their own arrivals, polled by their readers
+// in place of the barrier, took 6 000 to 11 000 clocks a phase against 5 000:
+// the polls hold up the additions they wait for.)
+__device__ __forceinline__ void fx_columns(const unsigned long long* set, int nt, int sh, int sh_last, double* out,
+                                           float2* outdf) {
+    static_assert(FX_COPIES == 8, "eight lanes per column");
+    const int k = threadIdx.x & 7;
+    for (int base = 0; base < nt; base += PT / 8) {
+        const int c = base + (int)(threadIdx.x >> 3);
+        ulonglong2 u = make_ulonglong2(0ull, 0ull), v = u;
+        if (c < nt) {
+            const ulonglong2* p = reinterpret_cast<const ulonglong2*>(set + ((size_t)k * FX_COLS + c) * FX_LIMBS);
+            u = __ldcg(p);
+            v = __ldcg(p + 1);
         }
-        for (; c < ncols; ++c) a0 += vi[c * vld] * h[c];
-        const double x = ws[u] - ((a0 + a1) + (a2 + a3));
-        ws[u] = x;
-        if (w) w[lo + u] = x;
-        if (wdf) wdf[lo + u] = df_to_float2(df_from_double(x));
-        if (vg) {
-            const double y = x * inv;
-            vg[u] = y;
-            if (vs) vs[u] = y;
+        const bool bad = __any_sync(0xffu << (threadIdx.x & 24), v.y != 0ull);
+#pragma unroll
+        for (int o = 1; o < 8; o <<= 1) {
+            u.x += __shfl_xor_sync(0xffffffffu, u.x, o);
+            u.y += __shfl_xor_sync(0xffffffffu, u.y, o);
+            v.x += __shfl_xor_sync(0xffffffffu, v.x, o);
+        }
+        if (c < nt && k == 0) {
+            // u.x + u.y 2^56 + v.x 2^112 modulo 2^128
+            Fix f{u.x, 0ull, bad};
+            fx_sum(f, u.y << 56, (u.y >> 8) + (v.x << 48));
+            out[c] = fx_value(f, c == nt - 1 ? sh_last : sh, outdf ? outdf + c : nullptr);
+        }
+    }
+}
+
+// The inner products of the staged slice with its basis columns, sum_{u < ne}
+// Vl[c vld + u] ws[u] for c < ncols and with norm also sum ws[u]^2 as column
+// ncols: emit(c, sum) by one thread per column.  A warp per column; long
+// slices with few columns give a column several warps, whose sums meet in
+// part (16 entries of shared memory).
+template <typename Emit>
+__device__ __forceinline__ void slice_dots(const double* Vl, int64_t vld, int ncols, const double* ws, int ne,
+                                           bool norm, int sh, int sh_n, Fix* part, Emit&& emit) {
+    const int nt = ncols + (norm ? 1 : 0);
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    auto column = [&](int c, int first, int step) {
+        const double* vc = c < ncols ? Vl + c * vld : ws;
+        double a = 0.0, b = 0.0;
+        int u = first;
+        if (ne > 512) {
+            double a2 = 0.0, b2 = 0.0;
+            for (; u + 3 * step < ne; u += 4 * step) {
+                const double v0 = vc[u], v1 = vc[u + step], v2 = vc[u + 2 * step], v3 = vc[u + 3 * step];
+                a += v0 * ws[u];
+                b += v1 * ws[u + step];
+                a2 += v2 * ws[u + 2 * step];
+                b2 += v3 * ws[u + 3 * step];
+            }
+            a += a2;
+            b += b2;
+            for (; u < ne; u += step) a += vc[u] * ws[u];
+            a += b;
+        } else {
+            for (; u < ne; u += step) a += vc[u] * ws[u];
+        }
+        return fx_warp_sum(fx_fixed(a, c < ncols ? sh : sh_n));
+    };
+    if (ne > 512 && nt <= PNW / 2) {
+        int P = 2;
+        while (2 * P * nt <= PNW) P *= 2;
+        if (wid < nt * P) {
+            const Fix f = column(wid / P, (wid & (P - 1)) * 32 + lane, 32 * P);
+            if (lane == 0) part[wid] = f;
+        }
+        __syncthreads();
+        if ((int)threadIdx.x < nt) {
+            Fix f = part[threadIdx.x * P];
+            for (int i = 1; i < P; ++i) {
+                const Fix g = part[threadIdx.x * P + i];
+                fx_sum(f, g.lo, g.hi);
+                f.bad = f.bad || g.bad;
+            }
+            emit((int)threadIdx.x, f);
+        }
+    } else {
+        for (int c = wid; c < nt; c += PNW) {
+            const Fix f = column(c, lane, 32);
+            if (lane == 0) emit(c, f);
+        }
+    }
+}
+
+// sum_{c < ncols} Vl[c vld + u] h[c] for the elements u < ne of the slice:
+// use(u, sum).  Short slices split the columns over four warps, one per
+// scheduler (the FP64 pipe takes 64 clocks a warp instruction, so one warp's
+// chain of M products is M times that); the four sums meet in tmp (PT
+// doubles).  Contains CTA barriers; not complete on return.
+template <typename Use>
+__device__ __forceinline__ void slice_combine(const double* Vl, int64_t vld, int ncols, const double* h, int ne,
+                                              double* tmp, Use&& use) {
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    if (ne <= 2 * PT / 4) {
+        const int part = wid & 3, blk = (wid >> 2) * 32 + lane;
+        for (int base = 0; base < ne; base += PT / 4) {
+            const int u = base + blk;
+            if (u < ne) {
+                double a = 0.0;
+                for (int c = part; c < ncols; c += 4) a += Vl[c * vld + u] * h[c];
+                tmp[part * (PT / 4) + blk] = a;
+            }
+            __syncthreads();
+            if ((int)threadIdx.x < PT / 4 && base + (int)threadIdx.x < ne) {
+                const double* p = tmp + threadIdx.x;
+                use(base + (int)threadIdx.x, (p[0] + p[PT / 4]) + (p[2 * (PT / 4)] + p[3 * (PT / 4)]));
+            }
+            if (base + PT / 4 < ne) __syncthreads();
+        }
+    } else {
+        for (int u = threadIdx.x; u < ne; u += PT) {
+            const double* vi = Vl + u;
+            double a0 = 0.0, a1 = 0.0, a2 = 0.0, a3 = 0.0;
+            int c = 0;
+#pragma unroll 2
+            for (; c + 3 < ncols; c += 4) {
+                a0 += vi[c * vld] * h[c];
+                a1 += vi[(c + 1) * vld] * h[c + 1];
+                a2 += vi[(c + 2) * vld] * h[c + 2];
+                a3 += vi[(c + 3) * vld] * h[c + 3];
+            }
+            for (; c < ncols; ++c) a0 += vi[c * vld] * h[c];
+            use(u, (a0 + a1) + (a2 + a3));
         }
     }
 }
@@ -294,17 +501,16 @@ __device__ __forceinline__ void slice_norm2(const double* ws, int ne, double* re
 template <int D, int KP1, int G, bool DF>
 __device__ __forceinline__ void arnoldi_body(const GmvArgs<double, D>& ga, const ArnArgs& a, const int nb,
                                              const int b) {
-    // dynamic shared memory: [w slices: 2 E][Vs: (M+1) Es][Zs: (M+1) Es][located rows, or gather offsets
-    // and entries]
-    extern __shared__ __align__(16) double smem[];
+    // dynamic shared memory: [x: n, 16-byte multiple][w slices: 2 E][Vs: (M+1) Es][Zs: (M+1) Es][located rows,
+    // or gather offsets and entries (staged x: values, then indices)]
+    extern __shared__ __align__(16) double smem_dyn[];
     __shared__ double h1[SGK_MAX_KRYLOV + 2];
     __shared__ double h2[SGK_MAX_KRYLOV + 2];
-    __shared__ double sdot[SGK_MAX_KRYLOV + 2];  // this CTA's inner products
     __shared__ double red[PNW];
-    __shared__ double s_scal[4];
-    // column-sum and inner-product staging: <= max(PT, 4 (SGK_MAX_KRYLOV + 2))
+    __shared__ double s_scal[4], s_beta;
+    // column-sum and combination staging: <= max(PT, 4 (SGK_MAX_KRYLOV + 2))
     __shared__ double ctmp[PT > 4 * (SGK_MAX_KRYLOV + 2) ? PT : 4 * (SGK_MAX_KRYLOV + 2)];
-    __shared__ double ctmp2[4 * (SGK_MAX_KRYLOV + 2)];
+    __shared__ Fix s_part[PNW];
     __shared__ int s_ok, s_flag;
     // double-float matvec: the correction's coefficients and the step's scale
     __shared__ float2 h2df[DF ? SGK_MAX_KRYLOV + 2 : 1];
@@ -315,6 +521,8 @@ __device__ __forceinline__ void arnoldi_body(const GmvArgs<double, D>& ga, const
     const int ne = (int)((a.bounds ? a.bounds[b + 1] : std::min<int64_t>(n, lo + E)) - lo);
     // the staged slice of w, two buffers alternating by step: the update of
     // step j (v_{j+1} from w') runs during the matvec of step j + 1
+    double* const xstage = smem_dyn;
+    double* const smem = smem_dyn + (a.xs ? (n + 1) / 2 * 2 : 0);
     double* const wsb0 = smem;
     double* const wsb1 = smem + E;
     // shared columns of V and Z have an odd stride: the lanes of one output
@@ -328,7 +536,11 @@ __device__ __forceinline__ void arnoldi_body(const GmvArgs<double, D>& ga, const
     // pre-located gathers of the slice: offsets rebased to the slice's first
     // entry, then the entries
     int* const seoff = a.list_cap > 0 ? reinterpret_cast<int*>(tail) : nullptr;
-    int2* const sent = a.list_cap > 0 ? reinterpret_cast<int2*>(tail + arn_eoff_bytes(E, D)) : nullptr;
+    int2* const sent = a.list_cap > 0 && !a.xs ? reinterpret_cast<int2*>(tail + arn_eoff_bytes(E, D)) : nullptr;
+    // staged x: the entries' values and indices, in shared memory or (their
+    // offsets as they are) in the flat copies
+    double* const sev = a.list_cap > 0 && a.xs ? reinterpret_cast<double*>(tail + arn_eoff_bytes(E, D)) : nullptr;
+    unsigned short* const sei = sev ? reinterpret_cast<unsigned short*>(sev + a.list_cap) : nullptr;
     // this slice's basis and raw-output columns: shared copies or HBM
     const double* const Vl = a.smem_vz ? Vs : a.V + lo;
     const int64_t vld = a.smem_vz ? Es : n;
@@ -337,42 +549,45 @@ __device__ __forceinline__ void arnoldi_body(const GmvArgs<double, D>& ga, const
     float2* const Zdf = reinterpret_cast<float2*>(Zl);  // Z as (hi, lo) pairs (double-float matvec)
     double* const P2 = a.pbuf;  // norms
     unsigned epoch = 0;
+    const bool alone = nb == 1 && a.bar_extra == 0u;  // one CTA: nothing to wait for or to add up
     auto barrier = [&]() {
+        if (alone) {
+            __syncthreads();
+            return true;
+        }
         ++epoch;
-        return grid_barrier(a.bar, epoch * (unsigned)nb + a.bar_extra, &s_ok);
+        const bool ok = grid_barrier(a.bar, epoch * (unsigned)nb + a.bar_extra, &s_ok);
+        if (!ok) stage_wait();  // the CTA leaves: none of its copies may land later
+        return ok;
     };
-    // fixed-point reductions: phase p adds into set p % 3, read after its
-    // barrier; after the barrier of phase p every CTA is done reading set
-    // (p - 1) % 3, which CTA 0 then clears for phase p + 2 (its stores precede
-    // its arrival at the barrier before that phase's atomics)
-    unsigned fx_phase = 0;
-    auto fx_set = [&](unsigned p) { return a.acc + (size_t)(p % 3u) * FX_SET; };
-    // publish sdot[0..nt) (the last column with the norm scale when norm)
-    auto fx_publish = [&](int nt, bool norm) {
-        unsigned long long* set = fx_set(fx_phase) + (size_t)(b % FX_COPIES) * FX_COLS * FX_LIMBS;
-        if ((int)threadIdx.x < nt) {
-            const bool nc_col = norm && (int)threadIdx.x == nt - 1;
-            fx_red(set + (size_t)threadIdx.x * FX_LIMBS, sdot[threadIdx.x], nc_col ? a.sc_n : a.sc_h);
-        }
+    // Fixed-point reductions: the two phases of step j add into sets
+    // 2 (j % 3) and 2 (j % 3) + 1, each read after a barrier.  After step j's
+    // first barrier every CTA has left step j - 1, and CTA 0 clears that
+    // step's sets for step j + 2; its arrival at step j's second barrier, which
+    // every CTA waits for, orders the clearing before that use.
+    auto fx_set = [&](int j, int phase) { return a.acc + (size_t)(2 * (j % 3) + phase) * FX_SET; };
+    // inner products of the slice into a phase (or straight to out)
+    auto dots = [&](int j, int phase, double* out, float2* outdf) {
+        const int nc = j + 1;
+        unsigned long long* set = fx_set(j, phase) + (size_t)(b % FX_COPIES) * FX_COLS * FX_LIMBS;
+        slice_dots(Vl, vld, nc, (j & 1) ? wsb1 : wsb0, ne, phase == 1, a.sh_h, a.sh_n, s_part, [&](int c, const Fix& f) {
+            if (alone) out[c] = fx_value(f, c < nc ? a.sh_h : a.sh_n, outdf ? outdf + c : nullptr);
+            else fx_add(set + (size_t)c * FX_LIMBS, f);
+        });
     };
-    // after reading phase p: CTA 0 clears set (p + 2) % 3, next phase
-    auto fx_done = [&]() {
-        if (b == 0) {
-            unsigned long long* old = fx_set(fx_phase + 2u);
-            for (int i = threadIdx.x; i < FX_SET; i += PT) old[i] = 0ull;
+    // and their sums over the CTAs
+    auto collect = [&](int j, int phase, double* out, float2* outdf) {
+        if (!barrier()) return false;
+        if (!alone) {
+            fx_columns(fx_set(j, phase), j + 1 + phase, a.sh_h, phase ? a.sh_n : a.sh_h, out, outdf);
+            __syncthreads();
         }
-        ++fx_phase;
-    };
-    auto fx_read = [&](int nt, bool norm, double* out) {
-        const unsigned long long* set = fx_set(fx_phase);
-        if ((int)threadIdx.x < nt) {
-            const bool nc_col = norm && (int)threadIdx.x == nt - 1;
-            out[threadIdx.x] = fx_value(set + (size_t)threadIdx.x * FX_LIMBS, nc_col ? a.isc_n : a.isc_h);
-        }
-        fx_done();
+        return true;
     };
     const int r = threadIdx.x & (G - 1);
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    // the warps that form the step's scalars: those with the least to gather
+    constexpr int WNORM = PNW - 1, WCOL = PNW - 2;
     KrylovScalars* ks = a.ks;
     if (sloc)
         for (int u = threadIdx.x; u < ne; u += PT) gmv_locate<double, D, KP1>(ga, lo + u, sloc[u]);
@@ -383,13 +598,25 @@ __device__ __forceinline__ void arnoldi_body(const GmvArgs<double, D>& ga, const
             return;
         }
         for (int i = threadIdx.x; i <= ne * D; i += PT) seoff[i] = a.eoff[lo * D + i] - e0;
-        for (int i = threadIdx.x; i < ecount; i += PT) sent[i] = a.ent[e0 + i];
+        if (sev) {
+            const double* src = DF ? reinterpret_cast<const double*>(a.ev2) : a.ev;
+            for (int i = threadIdx.x; i < ecount; i += PT) {
+                sev[i] = src[e0 + i];
+                sei[i] = a.ei[e0 + i];
+            }
+        } else {
+            for (int i = threadIdx.x; i < ecount; i += PT) sent[i] = a.ent[e0 + i];
+        }
     }
+    if (!DF && a.xs) stage_vector(xstage, a.v, n);  // the first gathers read v
 
-    // the accumulator sets start cleared (before the first barrier; the
-    // first atomics follow the second)
-    if (b == 0)
-        for (int i = threadIdx.x; i < 3 * FX_SET; i += PT) a.acc[i] = 0ull;
+    // the accumulator sets start cleared (before the first barrier)
+    auto clear_set = [&](unsigned long long* set, int cols) {
+        for (int i = threadIdx.x; i < FX_COPIES * cols * FX_LIMBS; i += PT)
+            set[(size_t)(i / (cols * FX_LIMBS)) * FX_COLS * FX_LIMBS + i % (cols * FX_LIMBS)] = 0ull;
+    };
+    if (b == 0 && !alone)
+        for (int i = 0; i < FX_SETS; ++i) clear_set(a.acc + (size_t)i * FX_SET, a.M + 1);
     // gamma = ||v||
     for (int u = threadIdx.x; u < ne; u += PT) wsb0[u] = a.v[lo + u];
     __syncthreads();
@@ -414,7 +641,10 @@ __device__ __forceinline__ void arnoldi_body(const GmvArgs<double, D>& ga, const
         }
     }
     __syncthreads();
-    if (!(s_scal[1] > 0.0)) return;  // gamma = 0: the same decision in every CTA
+    if (!(s_scal[1] > 0.0)) {  // gamma = 0: the same decision in every CTA
+        stage_wait();
+        return;
+    }
     double scale = s_scal[1];
     for (int u = threadIdx.x; u < ne; u += PT) {
         const double y = wsb0[u] * scale;
@@ -431,191 +661,227 @@ __device__ __forceinline__ void arnoldi_body(const GmvArgs<double, D>& ga, const
         // one more barrier publishes the pairs; the first product is then
         // A v_0 itself (scale 1)
         if (!barrier()) return;
+        if (a.xs) stage_vector(xstage, a.w1, n);
         scale = 1.0;
         if (threadIdx.x == 0) s_scaldf = df_to_float2(df_from_double(1.0));
         __syncthreads();
     }
     // the next matvec gathers x (written by all CTAs) and forms
-    // A v_j = scale (A x - corr), corr = sum_c hp_c A v_c over the previous
+    // A v_j = scale (A x - corr), corr = sum_c h2_c A v_c over the previous
     // step's columns: with the norm taken by Pythagoras, x is w' (complete at
-    // the second barrier) and A v_j = (A w' - A V h2) / beta, A V being the
+    // the second phase) and A v_j = (A w' - A V h2) / beta, A V being the
     // stored raw matvec outputs of the slice; after an explicit norm x is w''
     const double* x = a.v;
     const float2* xdf = reinterpret_cast<const float2*>(a.w1);
     int ncorr = 0;                 // columns of the correction (0: none)
-    double fro2 = 0.0, sub = 0.0;  // kept alike by every lane of warp 0
+    // ||H||_F^2 without the last subdiagonal (warp WCOL), and that one's square
+    // (every thread)
+    double fro2 = 0.0, sub2 = 0.0;
     // the pending update of the previous step: v_{pj+1} on the slice from
     // that step's staged w (w' - V h2, or w'' after an explicit norm) times
-    // pscale, into column pj + 1 of V (global and shared)
-    int pj = -1, pnc = 0;
+    // its scale, into column pj + 1 of V (global and shared)
+    int pj = -1;
     bool pexpl = false;
-    double pscale = 0.0;
     auto pending_update = [&]() {
-        double* const wp = (pj & 1) ? wsb1 : wsb0;
+        const double* const wp = (pj & 1) ? wsb1 : wsb0;
         double* vg = a.V + (int64_t)(pj + 1) * n + lo;
         double* vs = Vs ? Vs + (int64_t)(pj + 1) * Es : nullptr;
+        const double pscale = s_scal[1];
+        auto put = [&](int u, double sum) {
+            const double y = (wp[u] - sum) * pscale;
+            vg[u] = y;
+            if (vs) vs[u] = y;
+        };
         if (pexpl) {
-            for (int u = threadIdx.x; u < ne; u += PT) {
-                const double y = wp[u] * pscale;
-                vg[u] = y;
-                if (vs) vs[u] = y;
-            }
+            for (int u = threadIdx.x; u < ne; u += PT) put(u, 0.0);
         } else {
-            slice_update(Vl, vld, pnc, h2, nullptr, wp, lo, ne, vg, vs, pscale);
+            slice_combine(Vl, vld, pj + 1, h2, ne, ctmp, put);
         }
     };
+    if (threadIdx.x == 0) s_scal[1] = scale;
     for (int j = 0; j < a.M; ++j) {
         double* w = (j & 1) ? a.w1 : a.w0;
         double* const ws = (j & 1) ? wsb1 : wsb0;
         const int nc = j + 1;
-        // A v_j on this slice, staged in shared memory and kept in Z
+        // A v_j on this slice before its scale, which one warp may still be
+        // forming: raw sums into the staged slice (a double, or a pair)
+        if (a.xs) {
+            stage_wait();
+            __syncthreads();
+        }
         for (int base = 0; base < ne; base += PT / G) {
             const int u = base + (int)threadIdx.x / G;
             const bool live = u < ne;
-            double acc;
+            const int uu = live ? u : 0;
             // the correction's columns are dealt over the virtual lanes like
             // the matrix rows (sum independent of G)
-            if (DF) {
-                df64 ad = gmv_accumulate_list_df<D, G>(seoff + (live ? u : 0) * D, sent, a.cvk2, xdf, r, live,
-                                                       ncorr, h2df, Zdf + (live ? u : 0), zld);
-                if (live && r == 0) {
-                    ad = df_mul(ad, df_from_float2(s_scaldf));
-                    ws[u] = df_to_double(ad);
-                    Zdf[(int64_t)j * zld + u] = df_to_float2(ad);
-                }
-                continue;
-            } else if (seoff) {
-                acc = gmv_accumulate_list<D, G>(seoff + (live ? u : 0) * D, sent, ga.cvk, x, r, live, ncorr, h2,
-                                                Zl + (live ? u : 0), zld);
-            } else if (sloc) {
-                acc = gmv_accumulate<double, D, G, 2>(ga, x, sloc[live ? u : 0], r, live, ncorr, h2,
-                                                         Zl + (live ? u : 0), zld);
+            if constexpr (DF) {
+                df64 ad;
+                if (a.xs)
+                    ad = gather_staged<G>(sei, reinterpret_cast<const float2*>(sev),
+                                          reinterpret_cast<const float2*>(xstage), seoff[uu * D],
+                                          live ? seoff[(uu + 1) * D] : 0, r, live ? ncorr : 0, h2df, Zdf + uu, zld);
+                else
+                    ad = gmv_accumulate_list_df<D, G>(seoff + uu * D, sent, a.cvk2, xdf, r, live, ncorr, h2df, Zdf + uu,
+                                                      zld);
+                if (live && r == 0) reinterpret_cast<float2*>(ws)[u] = df_to_float2(ad);
             } else {
-                GmvLoc<D> l1;
-                if (live) gmv_locate<double, D, KP1>(ga, lo + u, l1);
-                acc = gmv_accumulate<double, D, G, 2>(ga, x, l1, r, live, ncorr, h2, Zl + (live ? u : 0), zld);
+                double acc;
+                if (a.xs) {
+                    acc = gather_staged<G>(sei, sev, xstage, seoff[uu * D], live ? seoff[(uu + 1) * D] : 0, r,
+                                           live ? ncorr : 0, h2, Zl + uu, zld);
+                } else if (seoff) {
+                    acc = gmv_accumulate_list<D, G>(seoff + uu * D, sent, ga.cvk, x, r, live, ncorr, h2, Zl + uu, zld);
+                } else if (sloc) {
+                    acc = gmv_accumulate<double, D, G, 2>(ga, x, sloc[uu], r, live, ncorr, h2, Zl + uu, zld);
+                } else {
+                    GmvLoc<D> l1;
+                    if (live) gmv_locate<double, D, KP1>(ga, lo + u, l1);
+                    acc = gmv_accumulate<double, D, G, 2>(ga, x, l1, r, live, ncorr, h2, Zl + uu, zld);
+                }
+                if (live && r == 0) ws[u] = acc;
             }
-            if (live && r == 0) {
-                acc *= scale;
+        }
+        __syncthreads();
+        // the scale is there: A v_j staged and kept in Z, by the upper half of
+        // the CTA, which the combination's last sums leave idle
+        for (int u = (int)threadIdx.x - PT / 2; u < ne; u += PT / 2) {
+            if (u < 0) break;
+            if constexpr (DF) {
+                const df64 ad = df_mul(df_from_float2(reinterpret_cast<const float2*>(ws)[u]), df_from_float2(s_scaldf));
+                ws[u] = df_to_double(ad);
+                Zdf[(int64_t)j * zld + u] = df_to_float2(ad);
+            } else {
+                const double acc = ws[u] * s_scal[1];
                 ws[u] = acc;
                 Zl[(int64_t)j * zld + u] = acc;
             }
         }
         if (pj >= 0) pending_update();
         __syncthreads();
-        slice_dots(Vl, vld, nc, ws, ne, sdot, false, ctmp, ctmp2);
-        fx_publish(nc, false);
-        if (!barrier()) return;
-        fx_read(nc, false, h1);
-        __syncthreads();
+        dots(j, 0, h1, nullptr);
+        if (!collect(j, 0, h1, nullptr)) return;
+        if (b == 0 && j > 0 && !alone) {
+            clear_set(fx_set(j + 2, 0), nc);
+            clear_set(fx_set(j + 2, 1), nc + 1);
+        }
         // w' = w - V h1, published for the next matvec
-        slice_update(Vl, vld, nc, h1, DF ? nullptr : w, ws, lo, ne, nullptr, nullptr, 0.0,
-                     DF ? reinterpret_cast<float2*>(w) : nullptr);
+        slice_combine(Vl, vld, nc, h1, ne, ctmp, [&](int u, double sum) {
+            const double y = ws[u] - sum;
+            ws[u] = y;
+            if (DF) reinterpret_cast<float2*>(w)[lo + u] = df_to_float2(df_from_double(y));
+            else w[lo + u] = y;
+        });
         __syncthreads();
         // second pass: V^T w' and ||w'||^2 in one reduction
-        slice_dots(Vl, vld, nc, ws, ne, sdot, true, ctmp, ctmp2);
-        fx_publish(nc + 1, true);
-        if (!barrier()) return;
-        // column j of H and the breakdown test from ||w''||^2 = b2 and
-        // part = ||h1 + h2||^2: warp 0 of every CTA, every lane alike
-        auto hcol = [&](double b2, double part) {
-            const double f = fro2 + sub * sub + part;
-            // one reciprocal square root on two lanes: 1/beta and sqrt(f)
-            const double xin = lane == 0 ? b2 : f;
-            const double rs = xin > 0.0 ? rsqrt(xin) : 0.0;
-            const double inv = __shfl_sync(0xffffffffu, rs, 0);
-            const double sf = f > 0.0 ? f * __shfl_sync(0xffffffffu, rs, 1) : 0.0;
-            const double beta = b2 > 0.0 ? b2 * inv : 0.0;
-            fro2 = f;
-            sub = beta;
-            const bool brk = !(beta > 1e-12 * sf);
-            if (b == 0)
-                for (int i = lane; i < nc; i += 32) a.H[(int64_t)i * a.M + j] = h1[i] + h2[i];
+        dots(j, 1, h2, DF ? h2df : nullptr);
+        if (!collect(j, 1, h2, DF ? h2df : nullptr)) return;
+        // the next gathers' vector, copied while the scalars are formed (again
+        // after an explicit norm, which changes it)
+        if (a.xs && j + 1 < a.M) stage_vector(xstage, w, n);
+        // ||w''||^2 = ||w'||^2 - ||h2||^2 (V orthonormal, w'' = w' - V h2).
+        // As a rule h2 is rounding and its square below half a unit in the
+        // last place of ||w'||^2, which is then the norm as it stands, and far
+        // above a breakdown; integer comparisons of exponents tell, alike in
+        // every warp, and the next gathers start at once while one warp forms
+        // 1 / beta (scalar FP64 work is latency, 64 clocks an operation).
+        auto inverse_norm = [&](double b2) {  // one warp
+            const bool ok = b2 > 0.0 && b2 < 1.7976931348623157e308;
+            const double inv = ok ? rsqrt(b2) : 0.0;
             if (lane == 0) {
-                s_scal[1] = brk ? 0.0 : inv;
-                if (DF) s_scaldf = df_to_float2(df_from_double(brk ? 0.0 : inv));
-                if (b == 0) {
-                    a.H[(int64_t)(j + 1) * a.M + j] = beta;
-                    ks->fro2 = f;
-                    ks->m_eff = j + 1;
-                    if (brk) {
-                        ks->stop = 1;
-                        ks->breakdown = 1;
-                    }
-                }
+                s_scal[1] = inv;
+                s_scal[3] = ok ? b2 : 0.0;
+                if (DF) s_scaldf = df_to_float2(df_from_double(inv));
+                s_beta = b2 * inv;
+                if (b == 0) a.H[(int64_t)(j + 1) * a.M + j] = s_beta;
             }
         };
-        // ||w''||^2 = ||w'||^2 - ||h2||^2 (V orthonormal, w'' = w' - V h2);
-        // when the second pass removed more than 1e-3 of ||w'||^2 (near
-        // breakdown) the norm is summed explicitly instead.  With at most 32
-        // columns warp 0 reads h2 itself and, in the common case, finishes
-        // the column at once: one CTA barrier for the whole scalar part
-        auto pyth = [&](double part, double hh, double wn2) {
-            const double b2 = wn2 - hh;
-            const bool flag = !(hh <= 1e-3 * wn2) || !(b2 > 0.0);
-            if (lane == 0) {
-                s_flag = flag;
-                s_scal[0] = b2;
-                s_scal[2] = part;
+        auto column_of_h = [&]() {  // one warp: ||h1 + h2||^2, CTA 0 stores the column
+            double part = 0.0;
+            for (int i = lane; i < nc; i += 32) {
+                const double hv = h1[i] + h2[i];
+                part += hv * hv;
+                if (b == 0) a.H[(int64_t)i * a.M + j] = hv;
             }
-            if (!flag) hcol(b2, part);
+            fro2 += sub2 + warp_sum(part);
         };
-        if (nc + 1 <= 32) {
-            if (wid == 0) {
-                const unsigned long long* set = fx_set(fx_phase);
-                const double hv2 =
-                    lane <= nc ? fx_value(set + (size_t)lane * FX_LIMBS, lane == nc ? a.isc_n : a.isc_h) : 0.0;
-                if (lane <= nc) h2[lane] = hv2;
-                if (DF && lane < nc) h2df[lane] = df_to_float2(df_from_double(hv2));
-                __syncwarp();
-                const double hv = lane < nc ? h1[lane] + hv2 : 0.0;
-                const double part = warp_sum(hv * hv);
-                const double hh = warp_sum(lane < nc ? hv2 * hv2 : 0.0);
-                pyth(part, hh, __shfl_sync(0xffffffffu, hv2, nc));
-            }
-            fx_done();
+        unsigned hm = 0u;
+        for (int i = lane; i < nc; i += 32)
+            hm = max(hm, (unsigned)(__double_as_longlong(h2[i]) >> 32) & 0x7fffffffu);
+        hm = __reduce_max_sync(0xffffffffu, hm);
+        const long long wb = __double_as_longlong(h2[nc]);
+        const int eh = (int)(hm >> 20), ew = (int)(wb >> 52);
+        // h2_i^2 < 2^(2 (eh - 1022)), nc <= 2^7 of them, against 2^(ew - 1023 - 55)
+        const bool plain = wb > __double_as_longlong(a.no_brk) && ew < 0x7ff && eh < 0x7ff &&
+                           2 * (eh - 1022) + 7 <= ew - 1023 - 55;
+        bool explicit_norm = false;
+        if (plain) {
+            if (wid == WNORM) inverse_norm(h2[nc]);
+            else if (wid == WCOL) column_of_h();
+            sub2 = h2[nc];
         } else {
-            fx_read(nc + 1, true, h2);
+            // near breakdown: when the second pass removed more than 1e-3 of
+            // ||w'||^2 the norm is summed explicitly
+            if (wid == WNORM) {
+                double hh = 0.0;
+                for (int i = lane; i < nc; i += 32) hh += h2[i] * h2[i];
+                hh = warp_sum(hh);
+                const double wn2 = h2[nc], b2 = wn2 - hh;
+                if (lane == 0) s_flag = !(hh <= 1e-3 * wn2) || !(b2 > 0.0);
+                inverse_norm(b2);
+            } else if (wid == WCOL) {
+                column_of_h();
+                // the square of 1e-12 ||H||_F; no value of beta passes a NaN
+                if (lane == 0) s_scal[2] = fro2 == fro2 ? 1e-24 * fro2 : 1.7976931348623157e308;
+            }
             __syncthreads();
-            if (DF)
-                for (int i = threadIdx.x; i < nc; i += PT) h2df[i] = df_to_float2(df_from_double(h2[i]));
-            if (wid == 0) {
-                double part = 0.0, hh = 0.0;
-                for (int i = lane; i < nc; i += 32) {
-                    const double hv = h1[i] + h2[i];
-                    part += hv * hv;
-                    hh += h2[i] * h2[i];
+            explicit_norm = s_flag != 0;
+            if (explicit_norm) {
+                // w'' in place (published), its norm through a barrier
+                if (a.xs) {  // the first copy must not land over the second
+                    stage_wait();
+                    __syncthreads();
                 }
-                pyth(warp_sum(part), warp_sum(hh), h2[nc]);
+                slice_combine(Vl, vld, nc, h2, ne, ctmp, [&](int u, double sum) {
+                    const double y = ws[u] - sum;
+                    ws[u] = y;
+                    if (DF) reinterpret_cast<float2*>(w)[lo + u] = df_to_float2(df_from_double(y));
+                    else w[lo + u] = y;
+                });
+                __syncthreads();
+                slice_norm2(ws, ne, red, P2 + b);
+                if (!barrier()) return;
+                colsum(P2, nb, 1, s_scal, ctmp);
+                __syncthreads();
+                if (wid == WNORM) inverse_norm(s_scal[0]);
+                if (a.xs && j + 1 < a.M) stage_vector(xstage, w, n);
+                __syncthreads();
+            }
+            sub2 = s_scal[3];
+            // breakdown: beta not above 1e-12 ||H||_F, the same decision in
+            // every thread of every CTA (squares, which order like their bit
+            // patterns: neither is negative or a NaN)
+            if (!(__double_as_longlong(sub2) > __double_as_longlong(s_scal[2]))) {
+                if (b == 0 && threadIdx.x == 0) {
+                    ks->m_eff = j + 1;
+                    ks->stop = 1;
+                    ks->breakdown = 1;
+                }
+                stage_wait();
+                return;
             }
         }
-        __syncthreads();
-        const bool explicit_norm = s_flag != 0;
-        if (explicit_norm) {
-            // w'' in place (published), its norm through a third barrier
-            slice_update(Vl, vld, nc, h2, DF ? nullptr : w, ws, lo, ne, nullptr, nullptr, 0.0,
-                         DF ? reinterpret_cast<float2*>(w) : nullptr);
-            __syncthreads();
-            slice_norm2(ws, ne, red, P2 + b);
-            if (!barrier()) return;
-            colsum(P2, nb, 1, s_scal, ctmp);
-            __syncthreads();
-            if (wid == 0) hcol(s_scal[0], s_scal[2]);
-            __syncthreads();
-        }
-        if (!(s_scal[1] > 0.0)) return;  // breakdown: the same decision in every CTA
-        scale = s_scal[1];
-        // v_{j+1} is formed during the next step's matvec (which gathers w',
-        // published, and needs no column of V); the inner products after it
+        if (b == 0 && threadIdx.x == 0) ks->m_eff = j + 1;
+        // v_{j+1} is formed after the next step's gathers (which read w',
+        // published, and need no column of V); the inner products after it
         // read column j + 1
         pj = j;
-        pnc = nc;
         pexpl = explicit_norm;
-        pscale = scale;
         ncorr = explicit_norm ? 0 : nc;
         x = w;
         xdf = reinterpret_cast<const float2*>(w);
     }
+    __syncthreads();
     if (pj >= 0) pending_update();  // the last column, v_M
 }
 
