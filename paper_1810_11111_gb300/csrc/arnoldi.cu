@@ -110,12 +110,12 @@ std::vector<int64_t> arnoldi_balanced_bounds(const sgk_ctx* ctx, const sgk_op* o
 
 static size_t loc_bytes(int d) {
     switch (d) {
-        case 1: return sizeof(GmvLoc<1>);
-        case 2: return sizeof(GmvLoc<2>);
-        case 3: return sizeof(GmvLoc<3>);
-        case 4: return sizeof(GmvLoc<4>);
-        case 5: return sizeof(GmvLoc<5>);
-        default: return sizeof(GmvLoc<6>);
+        case 1: return sizeof(GmvLoc<1, int>);
+        case 2: return sizeof(GmvLoc<2, int>);
+        case 3: return sizeof(GmvLoc<3, int>);
+        case 4: return sizeof(GmvLoc<4, int>);
+        case 5: return sizeof(GmvLoc<5, int>);
+        default: return sizeof(GmvLoc<6, int>);
     }
 }
 

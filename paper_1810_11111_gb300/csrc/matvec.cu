@@ -4,8 +4,8 @@
 //
 // y is written once; x is gathered through L2 (the 1D rows overlap, so
 // neighbouring outputs share most of their loads).  The sums are taken in a
-// fixed order (per lane two accumulators per direction, directions in order,
-// then a fixed xor tree over the group), so results are deterministic.
+// fixed order (chains over the entries, directions in order, then a fixed
+// tree), so results are deterministic.
 #include <algorithm>
 #include <cmath>
 
@@ -26,7 +26,7 @@ __global__ void gmv_flat_kernel(int64_t count, const int2* __restrict__ ent, con
 }
 
 
-template <typename T, int D, int KP1, int G>
+template <typename T, int D, int KP1, int G, typename IX>
 __global__ void __launch_bounds__(256) gmv_kernel(const GmvArgs<T, D> a, const T* __restrict__ x,
                                                   T* __restrict__ y) {
     // G consecutive lanes share one output coefficient (more loads in flight
@@ -39,7 +39,7 @@ __global__ void __launch_bounds__(256) gmv_kernel(const GmvArgs<T, D> a, const T
          gg += (int64_t)gridDim.x * blockDim.x) {
         const int64_t g = gg / G;
         const bool live = g < a.n;
-        GmvLoc<D> L;
+        GmvLoc<D, IX> L;
         if (live) gmv_locate<T, D, KP1>(a, g, L);
         const T acc = gmv_accumulate<T, D, G, 0>(a, x, L, r, live);
         if (live && r == 0) y[g] = acc;
@@ -59,10 +59,13 @@ void gmv_dispatch(const sgk_op* op, const T* x, T* y) {
     const int64_t blocks = (idx->dof * G + threads - 1) / threads;
     const int grid = (int)std::min<int64_t>(blocks, (int64_t)ctx->num_sms * 8);
     KTimer kt(ctx, KC_MATVEC);
-#define SGK_GMV(K, GG) gmv_kernel<T, D, K, GG><<<grid, threads, 0, ctx->stream>>>(a, x, y)
+#define SGK_GMV(K, GG) gmv_kernel<T, D, K, GG, int><<<grid, threads, 0, ctx->stream>>>(a, x, y)
 #define SGK_GMV_K(K)                         \
     switch (G) {                             \
-        case 1: SGK_GMV(K, 1); break;        \
+        case 1:                              \
+            if (idx->dof < (int64_t(1) << 31)) SGK_GMV(K, 1);                                             \
+            else gmv_kernel<T, D, K, 1, int64_t><<<grid, threads, 0, ctx->stream>>>(a, x, y);              \
+            break;                           \
         case 2: SGK_GMV(K, 2); break;        \
         case 4: SGK_GMV(K, 4); break;        \
         default: SGK_GMV(K, 8); break;       \

@@ -532,7 +532,7 @@ __device__ __forceinline__ void arnoldi_body(const GmvArgs<double, D>& ga, const
     double* const Zs = a.smem_vz ? smem + 2 * E + (size_t)(a.M + 1) * Es : nullptr;
     unsigned char* const tail =
         reinterpret_cast<unsigned char*>(smem + 2 * E + (a.smem_vz ? 2 * (size_t)(a.M + 1) * Es : 0));
-    GmvLoc<D>* const sloc = a.smem_loc ? reinterpret_cast<GmvLoc<D>*>(tail) : nullptr;
+    GmvLoc<D, int>* const sloc = a.smem_loc ? reinterpret_cast<GmvLoc<D, int>*>(tail) : nullptr;
     // pre-located gathers of the slice: offsets rebased to the slice's first
     // entry, then the entries
     int* const seoff = a.list_cap > 0 ? reinterpret_cast<int*>(tail) : nullptr;
@@ -735,7 +735,7 @@ __device__ __forceinline__ void arnoldi_body(const GmvArgs<double, D>& ga, const
                 } else if (sloc) {
                     acc = gmv_accumulate<double, D, G, 2>(ga, x, sloc[uu], r, live, ncorr, h2, Zl + uu, zld);
                 } else {
-                    GmvLoc<D> l1;
+                    GmvLoc<D, int> l1;
                     if (live) gmv_locate<double, D, KP1>(ga, lo + u, l1);
                     acc = gmv_accumulate<double, D, G, 2>(ga, x, l1, r, live, ncorr, h2, Zl + uu, zld);
                 }

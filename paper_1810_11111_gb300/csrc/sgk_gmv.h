@@ -34,16 +34,19 @@ struct GmvArgs {
 
 // Where output g's rows live: per direction the row range [q0, qe) of the
 // 1D matrix and the terms of the source address base[lb] + (oI << (lb-1))
-// + p I + in (oI = o I (k+1), lb >= 1; oI itself for lb = 0).
-template <int D>
+// + p I + in (oI = o I (k+1), lb >= 1; oI itself for lb = 0).  IX: 32-bit
+// indices for vectors of less than 2^31 elements (half the registers and
+// integer operations: more warps per SM for a kernel that waits on its
+// gathers), else 64-bit.
+template <int D, typename IX>
 struct GmvLoc {
     int cbrow[D];  // offset of the (tuple, direction) row of the block-offset table
     int q0[D], qe[D];
-    int64_t oI[D], I[D], in[D];
+    IX oI[D], I[D], in[D];
 };
 
-template <typename T, int D, int KP1>
-__device__ __forceinline__ void gmv_locate(const GmvArgs<T, D>& a, int64_t g, GmvLoc<D>& L) {
+template <typename T, int D, int KP1, typename IX>
+__device__ __forceinline__ void gmv_locate(const GmvArgs<T, D>& a, int64_t g, GmvLoc<D, IX>& L) {
     const int nl = a.N + 1;
     // tuple of g: binary search between the tuples of the chunk's ends
     int lo = a.chunk[g >> 8], hi = a.chunk[(g >> 8) + 1];
@@ -53,7 +56,7 @@ __device__ __forceinline__ void gmv_locate(const GmvArgs<T, D>& a, int64_t g, Gm
         else hi = mid - 1;
     }
     const int t = lo;
-    int64_t e = g - a.offsets[t];
+    IX e = (IX)(g - a.offsets[t]);
     int lv[D], sh[D], c[D], cnt[D];
     int sum = 0;
 #pragma unroll
@@ -66,18 +69,18 @@ __device__ __forceinline__ void gmv_locate(const GmvArgs<T, D>& a, int64_t g, Gm
     // local multi-index, last direction fastest; cnt[m] = KP1 2^sh[m]
 #pragma unroll
     for (int m = D - 1; m >= 0; --m) {
-        const int64_t q = (e >> sh[m]) / KP1;
+        const IX q = (e >> sh[m]) / KP1;
         c[m] = (int)(e - q * cnt[m]);
         e = q;
     }
 #pragma unroll
     for (int i = 0; i < D; ++i) {
-        int64_t o = 0, in = 0, I = 1;
+        IX o = 0, in = 0, I = 1;
 #pragma unroll
         for (int m = 0; m < i; ++m) o = o * cnt[m] + c[m];
 #pragma unroll
         for (int m = D - 1; m > i; --m) {
-            in += (int64_t)c[m] * I;
+            in += (IX)c[m] * I;
             I *= cnt[m];
         }
         const int np = a.N - (sum - lv[i]);
@@ -93,57 +96,72 @@ __device__ __forceinline__ void gmv_locate(const GmvArgs<T, D>& a, int64_t g, Gm
 
 // y_g for a located output, computed by the G lanes of a group (lane r of
 // G; G divides 8, the group is G consecutive lanes of a warp, every lane of
-// the warp calls this).  The sum does not depend on G: the entries of every
-// row are dealt to 8 virtual lanes (entry q to virtual lane q mod 8, two
-// chains each, directions in order), optionally minus a correction
-// sum_c h_c z_c whose columns are dealt the same way, and the 8 virtual sums
-// are added in one fixed binary tree -- physical lanes hold 8/G virtual
-// lanes, the lower tree levels are shuffles, the upper ones local.  The
-// result is returned in every lane of the group.  LD selects the loads of
-// x: 0 plain (read-only for the kernel), 1 L2 only, 2 cached in L1 through
-// the coherent path (for vectors written by other CTAs of the same
+// the warp calls this).  For G > 1 the sum does not depend on G: the entries
+// of every row are dealt to 8 virtual lanes (entry q0 + i to virtual lane i
+// mod 8, two chains each by turns, directions in order), optionally minus a
+// correction sum_c h_c z_c whose columns are dealt the same way, and the 8
+// virtual sums are added in one fixed binary tree -- physical lanes hold 8/G
+// virtual lanes, the lower tree levels are shuffles, the upper ones local.  A
+// thread goes through its virtual lanes side by side, 16 / G loads in flight.
+// With one lane per output (long vectors) the row is taken in order by eight
+// chains.  The result is returned in every lane of the group.  LD selects the
+// loads of x: 0 plain (read-only for the kernel), 1 L2 only, 2 cached in L1
+// through the coherent path (for vectors written by other CTAs of the same
 // persistent kernel and published by a barrier whose acquire made L1
 // current).
-template <typename T, int D, int G, int LD>
-__device__ __forceinline__ T gmv_accumulate(const GmvArgs<T, D>& a, const T* __restrict__ x, const GmvLoc<D>& L,
+template <typename T, int D, int G, int LD, typename IX>
+__device__ __forceinline__ T gmv_accumulate(const GmvArgs<T, D>& a, const T* __restrict__ x, const GmvLoc<D, IX>& L,
                                             int r, bool live, int ncorr = 0, const T* hc = nullptr,
                                             const T* zc = nullptr, int64_t zld = 0) {
-    constexpr int VL = 8, PER = VL / G;
-    T b[PER];
+    constexpr int VL = 8, PER = VL / G, CH = G == 1 ? 1 : 2;  // chains of a virtual lane
+    T s[CH][PER];
 #pragma unroll
-    for (int k = 0; k < PER; ++k) b[k] = T(0);
+    for (int k = 0; k < PER; ++k)
+#pragma unroll
+        for (int h = 0; h < CH; ++h) s[h][k] = T(0);
     if (live) {
 #pragma unroll
-        for (int k = 0; k < PER; ++k) {
-            const int v = r + k * G;
-            T s0 = T(0), s1 = T(0);
+        for (int i = 0; i < D; ++i) {
+            const int64_t* __restrict__ base = a.cb + L.cbrow[i];
+            const T* __restrict__ cv = a.cvk + i * a.nnz;
+            const IX oI = L.oI[i], I = L.I[i];
+            const T* __restrict__ xi = x + L.in[i];
+            auto ld = [&](int pk) {
+                const int lb = pk >> 16, p = pk & 0xffff;
+                const T* px = xi + ((IX)base[lb] + (lb ? (oI << (lb - 1)) : oI) + (IX)p * I);
+                if constexpr (LD == 1) return __ldcg(px);
+                else if constexpr (LD == 2) return __ldca(px);
+                else return *px;
+            };
+            const int qe = L.qe[i];
+            int q = L.q0[i] + r;
+            // whole rounds (one entry for every chain) without tests, then the rest
+            for (; q - r + CH * VL <= qe; q += CH * VL) {
+                T xv[CH][PER];
 #pragma unroll
-            for (int i = 0; i < D; ++i) {
-                const int64_t* __restrict__ base = a.cb + L.cbrow[i];
-                const T* __restrict__ cv = a.cvk + i * a.nnz;
-                const int64_t oI = L.oI[i], I = L.I[i], in = L.in[i];
-                auto ld = [&](int pk) {
-                    const int lb = pk >> 16, p = pk & 0xffff;
-                    const int64_t ob = lb ? (oI << (lb - 1)) : oI;
-                    const T* px = x + base[lb] + ob + (int64_t)p * I + in;
-                    if constexpr (LD == 1) return __ldcg(px);
-                    else if constexpr (LD == 2) return __ldca(px);
-                    else return *px;
-                };
-                const int qe = L.qe[i];
-                int q = L.q0[i] + v;
-#pragma unroll 2
-                for (; q + VL < qe; q += 2 * VL) {
-                    const int p0 = a.ce[q], p1 = a.ce[q + VL];
-                    const T v0 = cv[q], v1 = cv[q + VL];
-                    s0 += v0 * ld(p0);
-                    s1 += v1 * ld(p1);
-                }
-                if (q < qe) s0 += cv[q] * ld(a.ce[q]);
+                for (int h = 0; h < CH; ++h)
+#pragma unroll
+                    for (int k = 0; k < PER; ++k) xv[h][k] = ld(a.ce[q + h * VL + k * G]);
+#pragma unroll
+                for (int h = 0; h < CH; ++h)
+#pragma unroll
+                    for (int k = 0; k < PER; ++k) s[h][k] += cv[q + h * VL + k * G] * xv[h][k];
             }
+#pragma unroll
+            for (int h = 0; h < CH; ++h)
+#pragma unroll
+                for (int k = 0; k < PER; ++k)
+                    if (q + h * VL + k * G < qe) s[h][k] += cv[q + h * VL + k * G] * ld(a.ce[q + h * VL + k * G]);
+        }
+    }
+    T b[PER];
+#pragma unroll
+    for (int k = 0; k < PER; ++k) {
+        b[k] = CH == 2 ? s[0][k] + s[CH - 1][k] : s[0][k];
+        if (live && ncorr > 0) {
             T c0 = T(0);
-            for (int c = v; c < ncorr; c += VL) c0 += hc[c] * zc[c * zld];
-            b[k] = (s0 + s1) - c0;
+            for (int c = r + k * G; c < ncorr; c += VL) c0 += hc[c] * zc[c * zld];
+            b[k] -= c0;
         }
     }
 #pragma unroll

@@ -10,8 +10,9 @@ import pytest
 torch = pytest.importorskip("torch")
 
 from oracle.index_set import IndexSet as OIndex  # noqa: E402
+from oracle.krylov import krylov_expv  # noqa: E402
 from oracle.operator import (DIRICHLET0, PERIODIC, cross_blocks_1d, sipg_1d,  # noqa: E402
-                             sparse_matvec_general)
+                             sparse_matvec, sparse_matvec_general)
 from oracle.reaction import Reaction  # noqa: E402
 from paper_1810_11111_gb300 import sgkiif  # noqa: E402
 
@@ -96,4 +97,33 @@ def test_fused_reaction_shapes(ctx, d, k, rx, n):
     sol.close()
     for o in ops:
         o.close()
+    idx.close()
+
+
+@pytest.mark.parametrize("d,n,k,M,skip", [
+    (2, 0, 2, 12, 0),   # one tuple of 9 coefficients: the projection ends in a breakdown
+    (2, 1, 2, 20, 1),   # 27 coefficients, the vector 8 bytes off a 16-byte boundary
+    (2, 3, 1, 31, 0), (2, 3, 1, 32, 1), (2, 4, 1, 33, 0),   # the columns of one warp, one more
+    (3, 3, 2, 70, 0),   # columns read in two rounds
+    (2, 9, 3, 3, 0),    # few columns on long slices
+])
+def test_krylov_projection_edges(ctx, d, n, k, M, skip):
+    # exp(dt A) v with dt small enough for the projection to be converged,
+    # where it does not depend on how the basis was rounded: 1e-10 as for the
+    # other exponentials, 1e-9 with the double-float matvec
+    idx = sgkiif.IndexSet(ctx, d, n, k)
+    kap = [1.0, 0.5, 0.1][:d]
+    op = sgkiif.Operator(ctx, idx, kap)
+    dt = 1e-9 if M < 10 else 1e-4
+    sol = sgkiif.Solver(ctx, [op], [[]], M, dt)
+    v = np.random.default_rng(M).standard_normal(idx.dof)
+    held = dev(np.concatenate([np.zeros(skip), v]))
+    vd = held[skip:]
+    wd = torch.empty(idx.dof, dtype=torch.float64, device="cuda")
+    sol.krylov_expv(0, vd.data_ptr(), wd.data_ptr())
+    ref, S = OIndex(d, n, k), sipg_1d(n, k)
+    want, _ = krylov_expv(lambda x: sparse_matvec(ref, S, kap, x), v, dt, M)
+    assert rel(wd.cpu().numpy(), want) <= (1e-10 if ctx.precision == sgkiif.SGK_FP64 else 1e-9)
+    sol.close()
+    op.close()
     idx.close()
