@@ -184,8 +184,9 @@ int sgk_operator_assemble(sgk_ctx* ctx, const sgk_index* idx, const double* kapp
  * trial value over the finest cells; E: test jump against trial average over
  * the faces), restricted to the index set.  sgk_matvec applies it in two
  * launches (the diagonal gather, then the mixed terms); solvers on such an
- * operator run the Arnoldi process as a sequence of launches instead of the
- * persistent kernel. */
+ * operator keep the FP64 matvec inside the Arnoldi process in both precision
+ * modes, in the persistent kernel when every output's entries of all terms
+ * fit one list (some 26 000 coefficients), else as a sequence of launches. */
 int sgk_operator_assemble_full(sgk_ctx* ctx, const sgk_index* idx, const double* K, int bc, double sigma,
                                sgk_op** out);
 /* Multiply-adds of one sgk_matvec: the entries of the 1D matrix rows each

@@ -92,6 +92,14 @@ std::vector<int64_t> arnoldi_balanced_bounds(const sgk_ctx* ctx, const sgk_op* o
     const size_t fixed = sizeof(double) * (2 * (size_t)cap_len + 2 * (size_t)(M + 1) * (size_t)(cap_len | 1)) +
                          sgk_arn::arn_eoff_bytes((int)cap_len, d);
     const size_t budget = smem_budget(ctx);
+    // one list per output (mixed derivatives): its entries stay in device memory
+    if (op->x1_off.p) {
+        std::vector<int64_t> b1 = arnoldi_slice_bounds(op, nb, 2 * M, cap_len, int64_t(1) << 40);
+        *E = 0;
+        *list_ent = 0;
+        for (size_t i = 0; i + 1 < b1.size(); ++i) *E = std::max<int64_t>(*E, b1[i + 1] - b1[i]);
+        return b1;
+    }
     int64_t cap_ent = (op->gmv_ecnt_host.empty() || fixed >= budget) ? (int64_t(1) << 40)
                                                                       : (int64_t)((budget - fixed) / sizeof(int2));
     std::vector<int64_t> b = arnoldi_slice_bounds(op, nb, 2 * M, cap_len, cap_ent);
@@ -106,6 +114,16 @@ std::vector<int64_t> arnoldi_balanced_bounds(const sgk_ctx* ctx, const sgk_op* o
         }
     }
     return b;
+}
+
+bool arnoldi_persistent_takes(const sgk_ctx* ctx, const sgk_op* op) {
+    const int64_t n = op->idx->dof, nb = persistent_ctas(ctx);
+    if (n > arnoldi_persistent_max_n(ctx)) return false;
+    if (op->npairs == 0) return true;
+    // the staged vector beside the longest slice that the bounds allow
+    const int64_t E = ((n + nb - 1) / nb + PT / 8 - 1) / (PT / 8) * (PT / 8);
+    return op->x1_off.p != nullptr &&
+           sizeof(double) * (size_t)(n + 2 + 2 * E) + sgk_arn::arn_eoff_bytes((int)E, 1) <= smem_budget(ctx);
 }
 
 static size_t loc_bytes(int d) {
@@ -206,7 +224,19 @@ ArnPrep arnoldi_prepare(sgk_ctx* ctx, const sgk_op* op, const PersistentWork& pw
     a.ev2 = op->gmv_ev2.p;
     a.xs = a.ei != nullptr && (mixed ? a.ev2 != nullptr : a.ev != nullptr) && xb + ws + lst10 <= budget;
     size_t smem;
-    if (a.xs) {
+    a.eo1 = nullptr;
+    if (op->npairs > 0) {
+        // mixed derivatives: one list per output, FP64 in both modes
+        const size_t off = sgk_arn::arn_eoff_bytes((int)E, 1);
+        SGK_REQUIRE(op->x1_off.p && xb + ws + off <= budget, SGK_EUNSUPPORTED, "persistent Arnoldi: no entry lists");
+        a.xs = 1;
+        a.eo1 = op->x1_off.p;
+        a.ei = op->x1_ei.p;
+        a.ev = op->x1_ev.p;
+        a.smem_vz = xb + ws + off + vz <= budget;
+        smem = xb + ws + off + (a.smem_vz ? vz : 0);
+        a.df = 0;
+    } else if (a.xs) {
         a.smem_vz = xb + ws + lst10 + vz <= budget;
         a.list_cap = (int)std::max<int64_t>(list_ent, 1);
         smem = xb + ws + lst10 + (a.smem_vz ? vz : 0);

@@ -37,6 +37,7 @@ namespace {
 
 constexpr int XT = 4;  // stored 1D matrices: Q, P^T, E^T, P
 
+constexpr int64_t X1_MAX_ENT = int64_t(1) << 25;  // 336 MB
 constexpr int64_t X2_MAX_ENT = int64_t(1) << 26;  // 1.3 GB of entries and values, FP64 and FP32
 
 // The entries of the 2D rows: CTA a_i, one warp per a_j, the lanes over the
@@ -86,6 +87,69 @@ __global__ void __launch_bounds__(256) cross_fill_kernel(int H, int N, int kp1, 
     }
 }
 
+// Where an output stands: its tuple, and for a pair of directions i < j its
+// position (((o n_i + t_i) mid + c) n_j + t_j) in + r in the block: o over the
+// directions before i, c between, r after j.
+struct CrossPlace {
+    int d, tuple, local, lsum;
+    struct Pair {
+        int in, mid, r, c, o, ai, aj, L;
+        // index of x for a column {t_i | t_j << 16, l_i | l_j << 8}
+        __device__ __forceinline__ int position(int2 en, const int64_t* offs, int kp1) const {
+            const int bi = en.x & 0xffff, bj = en.x >> 16;
+            const int mi = en.y & 0xff, mj = en.y >> 8;
+            const int ni = mi == 0 ? kp1 : kp1 << (mi - 1), nj = mj == 0 ? kp1 : kp1 << (mj - 1);
+            return (int)offs[mi * (L + 1) + mj] + (((o * ni + bi) * mid + c) * nj + bj) * in + r;
+        }
+    };
+    __device__ __forceinline__ CrossPlace(int g, int dim, int ntuples, const int32_t* levels, const int64_t* offsets)
+        : d(dim) {
+        int lo = 0, hi = ntuples;  // offsets[lo] <= g < offsets[hi]
+        while (hi - lo > 1) {
+            const int mid = (lo + hi) >> 1;
+            if (offsets[mid] <= g) lo = mid;
+            else hi = mid;
+        }
+        tuple = lo;
+        local = g - (int)offsets[lo];
+        lsum = 0;
+        for (int m = 0; m < d; ++m) lsum += levels[lo * d + m];
+    }
+    __device__ __forceinline__ Pair pair(int i, int j, int N, int kp1, const int32_t* levels) const {
+        Pair p;
+        p.in = p.mid = 1;
+        p.r = p.c = p.o = 0;
+        int rest = local, ti = 0, tj = 0, li = 0, lj = 0, mul = 1;
+        for (int m = d - 1; m >= 0; --m) {
+            const int l = levels[tuple * d + m], n_l = l == 0 ? kp1 : kp1 << (l - 1);
+            const int q = rest / n_l, t = rest - q * n_l;
+            rest = q;
+            if (m == j) {
+                tj = t;
+                lj = l;
+                mul = 1;
+            } else if (m == i) {
+                ti = t;
+                li = l;
+                mul = 1;
+            } else if (m > j) {
+                p.r += t * mul;
+                p.in = mul *= n_l;
+            } else if (m > i) {
+                p.c += t * mul;
+                p.mid = mul *= n_l;
+            } else {
+                p.o += t * mul;
+                mul *= n_l;
+            }
+        }
+        p.L = N - (lsum - li - lj);
+        p.ai = (li == 0 ? 0 : kp1 << (li - 1)) + ti;
+        p.aj = (lj == 0 ? 0 : kp1 << (lj - 1)) + tj;
+        return p;
+    }
+};
+
 // The mixed-derivative terms from the table of 2D rows.  cross_kernel spends
 // four FP64 multiply-adds and a block position (a loop over the directions)
 // on every column, in the order of its longest rows; the table leaves one
@@ -110,64 +174,56 @@ __global__ void __launch_bounds__(256) cross_rows_kernel(int dof, int d, int N, 
     const int lane = threadIdx.x & 31;
     const int warps = (int)((gridDim.x * blockDim.x) >> 5);
     for (int g = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5); g < dof; g += warps) {
-        int lo = 0, hi = ntuples;  // offsets[lo] <= g < offsets[hi]
-        while (hi - lo > 1) {
-            const int mid = (lo + hi) >> 1;
-            if (offsets[mid] <= g) lo = mid;
-            else hi = mid;
-        }
-        const int e0 = g - (int)offsets[lo];
-        int lsum = 0;
-        for (int m = 0; m < d; ++m) lsum += levels[lo * d + m];
+        CrossPlace pl(g, d, ntuples, levels, offsets);
         T acc_all = T(0);
         for (int p = 0; p < npairs; ++p) {
-            const int i = pair_ij[2 * p], j = pair_ij[2 * p + 1];
-            // the output's position is (((o n_i + t_i) mid + c) n_j + t_j) in + r:
-            // o over the directions before i, c between, r after j
-            int rest = e0, in = 1, mid = 1, r = 0, c = 0, o = 0, ti = 0, tj = 0, li = 0, lj = 0, mul = 1;
-            for (int m = d - 1; m >= 0; --m) {
-                const int l = levels[lo * d + m], n_l = l == 0 ? kp1 : kp1 << (l - 1);
-                const int q = rest / n_l, t = rest - q * n_l;
-                rest = q;
-                if (m == j) {
-                    tj = t;
-                    lj = l;
-                    mul = 1;
-                } else if (m == i) {
-                    ti = t;
-                    li = l;
-                    mul = 1;
-                } else if (m > j) {
-                    r += t * mul;
-                    in = mul *= n_l;
-                } else if (m > i) {
-                    c += t * mul;
-                    mid = mul *= n_l;
-                } else {
-                    o += t * mul;
-                    mul *= n_l;
-                }
-            }
-            const int L = N - (lsum - li - lj);
-            const int ai = (li == 0 ? 0 : kp1 << (li - 1)) + ti, aj = (lj == 0 ? 0 : kp1 << (lj - 1)) + tj;
-            const int row = row0[ai] + aj;
-            const int qe = ptr[row] + len[row * (N + 1) + L];
-            const int64_t* offs = xoff + grp[(int64_t)lo * npairs + p];
+            const CrossPlace::Pair pr = pl.pair(pair_ij[2 * p], pair_ij[2 * p + 1], N, kp1, levels);
+            const int row = row0[pr.ai] + pr.aj;
+            const int qe = ptr[row] + len[row * (N + 1) + pr.L];
+            const int64_t* offs = xoff + grp[(int64_t)pl.tuple * npairs + p];
             T acc = T(0);
 #pragma unroll 4
-            for (int q = ptr[row] + lane; q < qe; q += 32) {
-                const int2 en = ent[q];
-                const int bi = en.x & 0xffff, bj = en.x >> 16;
-                const int mi = en.y & 0xff, mj = en.y >> 8;
-                const int ni = mi == 0 ? kp1 : kp1 << (mi - 1), nj = mj == 0 ? kp1 : kp1 << (mj - 1);
-                const int pos = (((o * ni + bi) * mid + c) * nj + bj) * in + r;
-                acc += val[q] * x[(int)offs[mi * (L + 1) + mj] + pos];
-            }
+            for (int q = ptr[row] + lane; q < qe; q += 32) acc += val[q] * x[pr.position(ent[q], offs, kp1)];
             acc_all += (T)kij[p] * acc;
         }
 #pragma unroll
         for (int s = 16; s > 0; s >>= 1) acc_all += __shfl_xor_sync(0xffffffffu, acc_all, s);
         if (lane == 0) y[g] -= acc_all;
+    }
+}
+
+// Every output's entries of the whole operator, one after the other: the
+// diagonal gather's (ent, {index of x, index of the value}), then -K_ij times
+// the row prefix of every pair.  One warp per output.
+__global__ void __launch_bounds__(256) cross_merge_kernel(
+    int dof, int d, int N, int kp1, int ntuples, const int32_t* __restrict__ levels,
+    const int64_t* __restrict__ offsets, const int* __restrict__ eoff, const int2* __restrict__ dent,
+    const double* __restrict__ cvk, int npairs, const int* __restrict__ pair_ij, const double* __restrict__ kij,
+    const int* __restrict__ row0, const int* __restrict__ ptr, const int* __restrict__ len,
+    const int2* __restrict__ ent, const double* __restrict__ val, const int64_t* __restrict__ grp,
+    const int64_t* __restrict__ xoff, const int* __restrict__ out_off, unsigned short* __restrict__ ei,
+    double* __restrict__ ev) {
+    const int lane = threadIdx.x & 31;
+    const int g = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
+    if (g >= dof) return;
+    int at = out_off[g];
+    for (int q = eoff[g * d] + lane; q < eoff[(g + 1) * d]; q += 32) {
+        const int2 e = dent[q];
+        ei[at + q - eoff[g * d]] = (unsigned short)e.x;
+        ev[at + q - eoff[g * d]] = cvk[e.y];
+    }
+    at += eoff[(g + 1) * d] - eoff[g * d];
+    CrossPlace pl(g, d, ntuples, levels, offsets);
+    for (int p = 0; p < npairs; ++p) {
+        const CrossPlace::Pair pr = pl.pair(pair_ij[2 * p], pair_ij[2 * p + 1], N, kp1, levels);
+        const int row = row0[pr.ai] + pr.aj;
+        const int n = len[row * (N + 1) + pr.L];
+        const int64_t* offs = xoff + grp[(int64_t)pl.tuple * npairs + p];
+        for (int q = lane; q < n; q += 32) {
+            ei[at + q] = (unsigned short)pr.position(ent[ptr[row] + q], offs, kp1);
+            ev[at + q] = -(kij[p] * val[ptr[row] + q]);
+        }
+        at += n;
     }
 }
 
@@ -422,6 +478,65 @@ void build_cross_tables(sgk_op* op, const double* K) {
     op->x_rlen.upload(rl, s);
     op->x_grp.upload(grp, s);
     op->x_off.upload(off, s);
+    // one list per output for the persistent Arnoldi kernel, and the part of
+    // the mixed terms in the bound on ||A||_2 (its fixed-point scale):
+    // ||B_ij|| <= 2 (||Q|| ||P|| + ||E|| ||P||), each at most the larger of
+    // the row and column sums
+    double nrm[XT];
+    for (int X = 0; X < XT; ++X) {
+        std::vector<double> cs(H, 0.0);
+        nrm[X] = 0.0;
+        for (int a = 0; a < H; ++a) {
+            double rs = 0.0;
+            for (int e = ptr[(size_t)X * (H + 1) + a]; e < ptr[(size_t)X * (H + 1) + a + 1]; ++e) {
+                rs += std::abs(val[e]);
+                cs[col[e]] += std::abs(val[e]);
+            }
+            nrm[X] = std::max(nrm[X], rs);
+        }
+        for (double c : cs) nrm[X] = std::max(nrm[X], c);
+    }
+    for (int p = 0; p < op->npairs; ++p) op->anorm += 2.0 * std::abs(kij[p]) * (nrm[0] * nrm[1] + nrm[2] * nrm[3]);
+    std::vector<int> off1;
+    if (op->x2_ent.p && op->gmv_ent.p && idx->dof <= GMV_STAGED_MAX) {
+        op->x1_cnt = op->gmv_ecnt_host;
+        int64_t total1 = 0;
+        for (int64_t tu = 0; tu < nt; ++tu) {
+            const int32_t* lv = &idx->levels[tu * d];
+            int ls = 0;
+            for (int m = 0; m < d; ++m) ls += lv[m];
+            for (int p = 0; p < op->npairs; ++p) {
+                const int i = pij[2 * p], j = pij[2 * p + 1], L = N - (ls - lv[i] - lv[j]);
+                int64_t mj = 1, mi = 1;  // position strides of directions j and i
+                for (int m = d - 1; m > j; --m) mj *= level_count(lv[m], kp1);
+                for (int m = d - 1; m > i; --m) mi *= level_count(lv[m], kp1);
+                for (int64_t e = 0; e < idx->offsets[tu + 1] - idx->offsets[tu]; ++e) {
+                    const int ai = level_offset(lv[i], kp1) + (int)(e / mi % level_count(lv[i], kp1));
+                    const int aj = level_offset(lv[j], kp1) + (int)(e / mj % level_count(lv[j], kp1));
+                    op->x1_cnt[idx->offsets[tu] + e] += len2[(size_t)(row2[ai] + aj) * nl + L];
+                }
+            }
+        }
+        off1.push_back(0);
+        for (int32_t c : op->x1_cnt) {
+            total1 += c;
+            if (total1 > X1_MAX_ENT) break;
+            off1.push_back((int)total1);
+        }
+        if (total1 <= X1_MAX_ENT) {
+            op->x1_off.upload(off1, s);
+            op->x1_ei.alloc(total1);
+            op->x1_ev.alloc(total1);
+            cross_merge_kernel<<<(int)((idx->dof + 7) / 8), 256, 0, s>>>(
+                (int)idx->dof, d, N, kp1, (int)nt, idx->d_levels.p, idx->d_offsets.p, op->gmv_eoff.p, op->gmv_ent.p,
+                op->gmv_cvk.p, op->npairs, op->x_pairs.p, op->x_kij.p, op->x2_row.p, op->x2_ptr.p, op->x2_len.p,
+                op->x2_ent.p, op->x2_val.p, op->x_grp.p, op->x_off.p, op->x1_off.p, op->x1_ei.p, op->x1_ev.p);
+            check_launch("cross_merge_kernel");
+            count_launch(op->ctx);
+        } else {
+            op->x1_cnt.clear();
+        }
+    }
     // multiply-adds of one application: per output and pair, the four terms'
     // truncated row products (counted on the host for the benchmarks)
     SGK_CUDA_CHECK(cudaStreamSynchronize(s));

@@ -253,7 +253,7 @@ std::vector<int64_t> arnoldi_slice_bounds(const sgk_op* op, int nb, int extra, i
     const int d = idx->d, N = idx->n, kp1 = idx->k + 1, nl = N + 1;
     const int64_t n = idx->dof;
     // entries of every output (the per-output matvec work)
-    std::vector<int32_t> ecnt = op->gmv_ecnt_host;
+    std::vector<int32_t> ecnt = op->x1_cnt.empty() ? op->gmv_ecnt_host : op->x1_cnt;
     if ((int64_t)ecnt.size() != n) {
         const std::vector<int>& rl = op->rlen_host;
         ecnt.assign(n, 0);

@@ -32,6 +32,10 @@ struct ArnArgs {
     // most list_cap) then come with their own values (entry q: ei[q], and
     // ev[q] or ev2[q]), staged in shared memory too
     int xs;
+    // eo1: one list per output over all terms of an operator with mixed
+    // derivatives (offset of output g; ei, ev), read from L2 in order with x
+    // staged; else null
+    const int* eo1;
     const unsigned short* ei;
     const double* ev;
     const float2* ev2;
@@ -181,6 +185,34 @@ __device__ __forceinline__ df64 gather_staged(const unsigned short* ei, const fl
 #pragma unroll
         for (int k = 0; k + m < PER; k += 2 * m) b[k] = df_add(b[k], b[k + m]);
     return b[0];
+}
+
+// Gather of one output from the staged x by a warp: entries q0 .. qe in
+// device memory, lane l takes q0 + l, q0 + l + 32, ... in one chain, eight
+// loads in flight; returned in every lane.
+__device__ __forceinline__ double gather_row(const unsigned short* __restrict__ ei, const double* __restrict__ ev,
+                                             const double* xs, int q0, int qe, int lane, int ncorr, const double* hc,
+                                             const double* zc, int64_t zld) {
+    constexpr int U = 8;
+    double b = 0.0;
+    int q = q0 + lane;
+    for (; q + (U - 1) * 32 < qe; q += U * 32) {
+        double v[U];
+        unsigned short i[U];
+#pragma unroll
+        for (int k = 0; k < U; ++k) {
+            v[k] = ev[q + 32 * k];
+            i[k] = ei[q + 32 * k];
+        }
+#pragma unroll
+        for (int k = 0; k < U; ++k) b += v[k] * xs[i[k]];
+    }
+#pragma unroll 4
+    for (; q < qe; q += 32) b += ev[q] * xs[ei[q]];
+    for (int c = lane; c < ncorr; c += 32) b -= hc[c] * zc[c * zld];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) b += __shfl_xor_sync(0xffffffffu, b, o);
+    return b;
 }
 
 // asynchronous copy of n 8-byte elements into shared memory by the CTA (16
@@ -535,7 +567,7 @@ __device__ __forceinline__ void arnoldi_body(const GmvArgs<double, D>& ga, const
     GmvLoc<D, int>* const sloc = a.smem_loc ? reinterpret_cast<GmvLoc<D, int>*>(tail) : nullptr;
     // pre-located gathers of the slice: offsets rebased to the slice's first
     // entry, then the entries
-    int* const seoff = a.list_cap > 0 ? reinterpret_cast<int*>(tail) : nullptr;
+    int* const seoff = a.list_cap > 0 || a.eo1 ? reinterpret_cast<int*>(tail) : nullptr;
     int2* const sent = a.list_cap > 0 && !a.xs ? reinterpret_cast<int2*>(tail + arn_eoff_bytes(E, D)) : nullptr;
     // staged x: the entries' values and indices, in shared memory or (their
     // offsets as they are) in the flat copies
@@ -591,7 +623,9 @@ __device__ __forceinline__ void arnoldi_body(const GmvArgs<double, D>& ga, const
     KrylovScalars* ks = a.ks;
     if (sloc)
         for (int u = threadIdx.x; u < ne; u += PT) gmv_locate<double, D, KP1>(ga, lo + u, sloc[u]);
-    if (seoff) {
+    if (a.eo1) {
+        for (int i = threadIdx.x; i <= ne; i += PT) seoff[i] = a.eo1[lo + i];
+    } else if (seoff) {
         const int e0 = a.eoff[lo * D], ecount = a.eoff[(lo + ne) * D] - e0;
         if (ecount > a.list_cap) {  // the host sized the list for every slice; fail rather than overrun
             if (threadIdx.x == 0) atomicExch(a.bar + 1, 1u);
@@ -709,7 +743,15 @@ __device__ __forceinline__ void arnoldi_body(const GmvArgs<double, D>& ga, const
             stage_wait();
             __syncthreads();
         }
-        for (int base = 0; base < ne; base += PT / G) {
+        if (!DF && a.eo1) {
+            // a warp per output: the rows are long and uneven (hundreds of
+            // entries, thousands at low levels)
+            for (int u = wid; u < ne; u += PNW) {
+                const double acc = gather_row(a.ei, a.ev, xstage, seoff[u], seoff[u + 1], lane, ncorr, h2, Zl + u, zld);
+                if (lane == 0) ws[u] = acc;
+            }
+        }
+        for (int base = 0; base < (a.eo1 ? 0 : ne); base += PT / G) {
             const int u = base + (int)threadIdx.x / G;
             const bool live = u < ne;
             const int uu = live ? u : 0;

@@ -348,6 +348,14 @@ struct sgk_op {
     DevBuf<double> x2_val;
     DevBuf<float> x2_valf;
     DevBuf<int> x2_ptr, x2_len, x2_row;
+    // diagonal and mixed-derivative entries of every output as one list, for
+    // the persistent Arnoldi kernel (index sets of at most GMV_STAGED_MAX
+    // coefficients and X1_MAX_ENT entries): offsets per output, index of x,
+    // value; empty otherwise.  x1_cnt: the host's entries per output
+    DevBuf<int> x1_off;
+    DevBuf<unsigned short> x1_ei;
+    DevBuf<double> x1_ev;
+    std::vector<int32_t> x1_cnt;
 };
 constexpr int64_t GMV_LIST_MAX = int64_t(1) << 24;
 // 8 bytes a coefficient in at most 227 KB of shared memory

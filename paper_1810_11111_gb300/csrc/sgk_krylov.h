@@ -65,6 +65,9 @@ int arnoldi_persistent_ctas(const sgk_ctx* ctx);
 // this context's device.
 int64_t arnoldi_persistent_max_n(const sgk_ctx* ctx);
 size_t arnoldi_persistent_pbuf_size(const sgk_ctx* ctx, int M);
+// Whether the persistent kernel takes an operator: its vectors' size and,
+// with mixed derivatives, its entry lists and the staged vector.
+bool arnoldi_persistent_takes(const sgk_ctx* ctx, const sgk_op* op);
 // Work-balanced slices for the persistent kernel (arnoldi_slice_bounds with
 // the caps that keep the slice's pre-located gathers and Krylov columns in
 // shared memory); empty when no such partition exists.  E and list_ent

@@ -1483,11 +1483,14 @@ void solver_alloc(sgk_solver* s) {
     s->ctl.alloc(sizeof(StepCtl));
     SGK_CUDA_CHECK(cudaMallocHost(&s->hrec, SGK_ASYNC_SLOTS * sizeof(StepRecord)));
     SGK_CUDA_CHECK(cudaMemsetAsync(s->ctl.p, 0, sizeof(StepCtl), s->ctx->stream));
-    // the persistent kernel's gather holds the diagonal terms only: an
-    // operator with mixed-derivative terms takes the launch-sequence path
-    bool cross = false;
-    for (int sp = 0; sp < S; ++sp) cross = cross || s->ops[sp]->npairs > 0;
-    s->persistent = std::getenv("SGK_NO_PERSISTENT") == nullptr && !cross && n <= arnoldi_persistent_max_n(s->ctx);
+    // operators that the persistent kernel does not take (long vectors, large
+    // ones with mixed derivatives) have the launch-sequence path
+    bool cross = false, takes = true;
+    for (int sp = 0; sp < S; ++sp) {
+        cross = cross || s->ops[sp]->npairs > 0;
+        takes = takes && arnoldi_persistent_takes(s->ctx, s->ops[sp]);
+    }
+    s->persistent = std::getenv("SGK_NO_PERSISTENT") == nullptr && takes;
     if (s->persistent) {
         s->w64b.alloc(n);
         s->zbuf.alloc((size_t)(M + 1) * n);
@@ -1512,8 +1515,8 @@ void solver_alloc(sgk_solver* s) {
         pw.bounds = s->abounds.p;
         pw.E = s->aE;
         pw.list_ent = s->alist;
-        s->arn_G = s->ctx->arn_G_fixed > 0
-                       ? s->ctx->arn_G_fixed
+        s->arn_G = s->ctx->arn_G_fixed > 0 || cross  // mixed derivatives: a warp per output
+                       ? std::max(s->ctx->arn_G_fixed, cross ? 8 : 0)
                        : arnoldi_autotune(s->ctx, s->ops[0], pw, krylov_work<double>(s, 0), s->W.p, n, M);
         SGK_CUDA_CHECK(cudaMemsetAsync(s->pbar.p, 0, 2 * S * sizeof(unsigned), s->ctx->stream));
     }

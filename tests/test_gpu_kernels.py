@@ -127,3 +127,32 @@ def test_krylov_projection_edges(ctx, d, n, k, M, skip):
     sol.close()
     op.close()
     idx.close()
+
+
+@pytest.mark.parametrize("d,n,k,M,bc", [(2, 1, 1, 9, PERIODIC), (2, 6, 2, 12, DIRICHLET0), (3, 4, 2, 35, PERIODIC),
+                                        (4, 2, 1, 20, DIRICHLET0)])
+def test_krylov_projection_mixed_derivatives(ctx, d, n, k, M, bc, monkeypatch):
+    # one list of all entries per output in the persistent kernel, against the
+    # sequence of launches (the same sums in another order) and the oracle;
+    # FP64 matvecs in both modes
+    K = np.diag(np.linspace(1.0, 0.6, d)) + 0.1 * (np.eye(d, k=1) + np.eye(d, k=-1))
+    idx = sgkiif.IndexSet(ctx, d, n, k)
+    op = sgkiif.Operator(ctx, idx, K, bc)
+    v = np.random.default_rng(n).standard_normal(idx.dof)
+    vd = dev(v)
+    dt, got = 1e-5, []
+    for off in (False, True):
+        if off:
+            monkeypatch.setenv("SGK_NO_PERSISTENT", "1")
+        sol = sgkiif.Solver(ctx, [op], [[]], M, dt)
+        wd = torch.empty_like(vd)
+        sol.krylov_expv(0, vd.data_ptr(), wd.data_ptr())
+        got.append(wd.cpu().numpy())
+        sol.close()
+    P, E = cross_blocks_1d(n, k, bc)
+    ref, S = OIndex(d, n, k), sipg_1d(n, k, bc)
+    want, _ = krylov_expv(lambda x: sparse_matvec_general(ref, S, P, E, K, x), v, dt, M)
+    assert rel(got[0], want) <= 1e-10 and rel(got[1], want) <= 1e-10
+    assert rel(got[0], got[1]) <= 1e-12
+    op.close()
+    idx.close()
