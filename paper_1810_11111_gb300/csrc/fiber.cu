@@ -265,34 +265,26 @@ static long long chunk_addr_host(const FiberGroup& g, long long o, int pos, long
     return g.cbase[l] + o * nl * I + (long long)(pos - off) * I + in;
 }
 
-static void validate_item(const FiberGroup& g, const FiberItem& it, int kp1, int H, int mode, long long src_size,
-                          long long dst_size) {
+// Every address of a group's columns lies in its buffers: addresses increase
+// with the outer and the inner index and with the position within a level's
+// chunk, so the first column's first and the last column's last position of
+// every chunk bound them all.
+static void validate_group(const FiberGroup& g, int kp1, int H, int mode, long long src_size, long long dst_size) {
     const int F = kp1 << (g.nlev - 1);
     SGK_REQUIRE(g.nlev >= 1 && g.nlev <= SGK_MAX_LEVEL + 1, SGK_EINVAL, "plan: bad level count");
-    SGK_REQUIRE(it.col0 >= 0 && it.ncols >= 1 && (long long)it.col0 + it.ncols <= (long long)g.O * g.I, SGK_EINVAL,
-                "plan: column range outside the group");
+    SGK_REQUIRE(g.O >= 1 && g.I >= 1, SGK_EINVAL, "plan: empty group");
     for (int side = 0; side < 2; ++side) {
         const bool full = (side == 0) ? mode == FIBER_BWD : mode == FIBER_FWD;
         const int len = full ? H : F;
         const long long size = side == 0 ? src_size : dst_size;
-        for (int c = 0; c < it.ncols; ++c) {
-            const long long col = it.col0 + c;
-            const long long o = col / g.I, in = col % g.I;
-            // addresses are increasing in pos within a level chunk: check the
-            // first and last position of every chunk
-            for (int l = 0; l < (full ? 1 : g.nlev); ++l) {
-                int p0, p1;
-                if (full) {
-                    p0 = 0;
-                    p1 = len - 1;
-                } else {
-                    p0 = l ? (kp1 << (l - 1)) : 0;
-                    p1 = p0 + (l ? (kp1 << (l - 1)) : kp1) - 1;
-                }
-                for (int pos : {p0, p1}) {
-                    const long long a = full ? g.fbase + (o * H + pos) * g.I + in : chunk_addr_host(g, o, pos, in, kp1, g.I);
-                    SGK_REQUIRE(a >= 0 && a < size, SGK_EINVAL, "plan: address outside its buffer");
-                }
+        for (int l = 0; l < (full ? 1 : g.nlev); ++l) {
+            const int p0 = full || l == 0 ? 0 : kp1 << (l - 1);
+            const int p1 = full ? len - 1 : p0 + (l ? (kp1 << (l - 1)) : kp1) - 1;
+            for (int last = 0; last < 2; ++last) {
+                const long long o = last ? g.O - 1 : 0, in = last ? g.I - 1 : 0;
+                const int pos = last ? p1 : p0;
+                const long long a = full ? g.fbase + (o * H + pos) * g.I + in : chunk_addr_host(g, o, pos, in, kp1, g.I);
+                SGK_REQUIRE(a >= 0 && a < size, SGK_EINVAL, "plan: address outside its buffer");
             }
         }
     }
@@ -316,6 +308,7 @@ void finalize_plan(FiberPlan& plan, std::vector<FiberGroup>& groups, int kp1, in
         const int src_len = mode == FIBER_BWD ? H : F;
         const int dst_len = mode == FIBER_FWD ? H : F;
         long long cols = (long long)g.O * g.I;
+        validate_group(g, kp1, H, mode, src_size, dst_size);
         SGK_REQUIRE(cols < (1LL << 31), SGK_EUNSUPPORTED, "plan: too many fibers in one group");
         // the pyramid kernel stages the source and destination fibers, and
         // for BWD the subtree roots (k+1 rows per subtree of 8 finest cells)
@@ -333,7 +326,8 @@ void finalize_plan(FiberPlan& plan, std::vector<FiberGroup>& groups, int kp1, in
             // an item computes whole fibers
             it.row0 = 0;
             it.nrows = dst_len;
-            validate_item(g, it, kp1, H, mode, src_size, dst_size);
+            SGK_REQUIRE(it.ncols >= 1 && (long long)it.col0 + it.ncols <= cols, SGK_EINVAL,
+                        "plan: column range outside the group");
             items.push_back(it);
             cost.push_back((long long)src_len * it.ncols + (long long)it.nrows * it.ncols * 8);
             smem = std::max(smem, (size_t)tile_rows * it.stride * elem_bytes);

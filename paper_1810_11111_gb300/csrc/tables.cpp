@@ -62,23 +62,37 @@ void gauss_legendre_ld(int q, std::vector<ld>& x, std::vector<ld>& w) {
     }
 }
 
-// Value of the hierarchical function (level n, cell j, degree p) of V_N^k at
-// x = (cell + (xi+1)/2) h on the piece belonging to finest cell `cell`.
-ld hier_value(int N, int k, const std::vector<ld>& alp, int n, int j, int p, int cell, ld xi) {
-    std::vector<ld> P(k + 1), dP(k + 1);
+// Values of the hierarchical functions (level n, cell j, degrees p = 0..k) of
+// V_N^k at x = (cell + (xi+1)/2) h on the piece belonging to finest cell `cell`.
+void hier_values(int N, int k, const std::vector<ld>& alp, int n, int j, int cell, ld xi, ld* out) {
+    ld P[8], dP[8];
     ld h = std::ldexp((ld)1, -N);
     ld x = (cell + (xi + 1) / 2) * h;
     if (n == 0) {
-        legendre_eval(k, 2 * x - 1, P.data(), dP.data());
-        return std::sqrt((ld)(2 * p + 1)) * P[p];
+        legendre_eval(k, 2 * x - 1, P, dP);
+        for (int p = 0; p <= k; ++p) out[p] = std::sqrt((ld)(2 * p + 1)) * P[p];
+        return;
     }
     int half = (cell >> (N - n)) & 1;
     ld y = std::ldexp(x, n) - (2 * j + 1);
     ld t = half == 0 ? 2 * y + 1 : 2 * y - 1;
-    legendre_eval(k, t, P.data(), dP.data());
-    ld v = 0;
-    for (int r = 0; r <= k; ++r) v += alp[p * 2 * (k + 1) + half * (k + 1) + r] * std::sqrt((ld)(2 * r + 1)) * P[r];
-    return std::ldexp(v, 0) * std::pow((ld)2, (ld)n / 2);
+    legendre_eval(k, t, P, dP);
+    // 2^{n/2}
+    const ld scale = std::ldexp(n % 2 ? std::sqrt((ld)2) : (ld)1, n / 2);
+    ld s[8];
+    for (int r = 0; r <= k; ++r) s[r] = std::sqrt((ld)(2 * r + 1));
+    for (int p = 0; p <= k; ++p) {
+        ld v = 0;
+        for (int r = 0; r <= k; ++r) v += alp[p * 2 * (k + 1) + half * (k + 1) + r] * s[r] * P[r];
+        out[p] = v * scale;
+    }
+}
+
+// one degree of them
+ld hier_value(int N, int k, const std::vector<ld>& alp, int n, int j, int p, int cell, ld xi) {
+    ld v[8];
+    hier_values(N, k, alp, n, j, cell, xi, v);
+    return v[p];
 }
 
 std::vector<ld> alpert_ld(int k) {
@@ -207,18 +221,30 @@ void build_transform_tables(int N, int k, Tables1D& out) {
     T.ptr.assign(H + 1, 0);
     T.col.clear();
     T.val.clear();
+    // a cell's row block takes K = k + 1 functions of every level; their values
+    // at the cell's points serve all rows (long double is software on some
+    // hosts: evaluated per entry this was 12.6 ms at level 6, degree 2)
+    const int per = kp1 * (N + 1);
+    std::vector<ld> v(kp1), acc((size_t)kp1 * per);
+    std::vector<int> cols(per);
+    T.col.reserve((size_t)H * per);
+    T.val.reserve((size_t)H * per);
     for (int c = 0; c < ncell; ++c) {
+        std::fill(acc.begin(), acc.end(), (ld)0);
+        for (int n = 0; n <= N; ++n) {
+            const int j = n == 0 ? 0 : (c >> (N - n + 1));
+            for (int p = 0; p < kp1; ++p) cols[n * kp1 + p] = level_offset(n, kp1) + j * kp1 + p;
+            for (int g = 0; g < kp1; ++g) {
+                hier_values(N, k, alp, n, j, c, xi[g], v.data());
+                for (int r = 0; r < kp1; ++r)
+                    for (int p = 0; p < kp1; ++p)
+                        acc[(size_t)r * per + n * kp1 + p] += h * w[g] / 2 * v[p] * Lg[g * kp1 + r];
+            }
+        }
         for (int r = 0; r < kp1; ++r) {
-            for (int n = 0; n <= N; ++n) {
-                int j = n == 0 ? 0 : (c >> (N - n + 1));
-                for (int p = 0; p < kp1; ++p) {
-                    int a = level_offset(n, kp1) + j * kp1 + p;
-                    ld acc = 0;
-                    for (int g = 0; g < kp1; ++g)
-                        acc += h * w[g] / 2 * hier_value(N, k, alp, n, j, p, c, xi[g]) * Lg[g * kp1 + r];
-                    T.col.push_back(a);
-                    T.val.push_back((double)acc);
-                }
+            for (int e = 0; e < per; ++e) {
+                T.col.push_back(cols[e]);
+                T.val.push_back((double)acc[(size_t)r * per + e]);
             }
             T.ptr[c * kp1 + r + 1] = (int)T.col.size();
         }
