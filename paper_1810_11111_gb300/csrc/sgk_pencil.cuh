@@ -90,6 +90,13 @@ struct Poly {
 // ceil((p k + k + 1) / 2).
 __host__ __device__ constexpr int max_degree(int K, int Q) { return (2 * Q - K) / (K - 1); }
 
+// One species in FP64: the polynomial is divided by its leading coefficient,
+// which goes into the outermost table of the moments (one multiplication less
+// at every point: -c u^3 takes two).  Not in the narrower types, whose range
+// would not hold the bare powers of a decayed state.
+template <typename T, int S>
+constexpr bool MONIC = std::is_same<T, double>::value && S == 1;
+
 // Horner's rule over total degree <= PM.  FP64 and double-float skip the zero
 // coefficients (the reactions are sparse polynomials, e.g. -c u^3; the tests
 // are uniform over the grid and cheaper than the multiply-adds); in FP32 a
@@ -98,13 +105,22 @@ template <typename T, int PM, int NP>
 __device__ __forceinline__ T poly_value(const Poly<T, 1, NP>& P, int i, const T (&u)[1]) {
     constexpr bool SKIP = !std::is_same<T, float>::value;
     T f = zero<T>();
-    bool started = false;
+    int state = 0;  // 0 above the leading term, 1 at it (monic: f stands for 1), 2 below
 #pragma unroll
     for (int e = PM < PDEG ? PM : PDEG - 1; e >= 0; --e) {
-        if (started) f = mul(f, u[0]);
+        if (state == 2) {
+            f = mul(f, u[0]);
+        } else if (state == 1) {
+            f = u[0];
+            state = 2;
+        }
         if (!SKIP || ((P.rows[i] >> e) & 1)) {
-            f = started ? add(f, cvalue(P.c[i][e])) : cvalue(P.c[i][e]);
-            started = true;
+            if (state == 0) {
+                f = cvalue(P.c[i][e]);
+                state = MONIC<T, 1> ? 1 : 2;
+            } else {
+                f = add(f, cvalue(P.c[i][e]));
+            }
         }
     }
     return f;
@@ -664,8 +680,9 @@ __global__ void __maxnreg__(MAX_REGS<T>)
 
 // Reaction coefficients by exponents, scaled for the basis without h^{-1/2}
 // (u = s u~ with s = h^{-d/2} at the points, the moments times s): c s^{deg+1}.
+// lead: the leading coefficient that a monic polynomial leaves out (else 1).
 template <typename T, int S, bool JAC>
-Poly<T, S, (JAC ? S * S : S)> make_poly(const ReactionDev& rx, double s) {
+Poly<T, S, (JAC ? S * S : S)> make_poly(const ReactionDev& rx, double s, double* lead) {
     constexpr int NP = JAC ? S * S : S, NCOEF = Pow<PDEG, S>::v;
     double c[NP][NCOEF] = {};
     for (int m = 0; m < rx.nmono; ++m) {
@@ -686,6 +703,15 @@ Poly<T, S, (JAC ? S * S : S)> make_poly(const ReactionDev& rx, double s) {
             }
         }
     }
+    *lead = 1.0;
+    if (MONIC<T, S>)
+        for (int j = NCOEF - 1; j >= 0; --j)
+            if (c[0][j] != 0.0) {
+                *lead = c[0][j];
+                for (int l = 0; l < j; ++l) c[0][l] /= *lead;
+                c[0][j] = 1.0;
+                break;
+            }
     Poly<T, S, NP> p{};
     for (int i = 0; i < NP; ++i)
         for (int j = 0; j < NCOEF; ++j) {
@@ -700,9 +726,10 @@ Poly<T, S, (JAC ? S * S : S)> make_poly(const ReactionDev& rx, double s) {
     return p;
 }
 
-// B: q x (k+1), sqrt(2r+1) P_r(xi_g) at ascending points; w: h w_g / 2
+// B: q x (k+1), sqrt(2r+1) P_r(xi_g) at ascending points; w: h w_g / 2; lead:
+// see make_poly
 template <typename T, int K, int Q>
-QuadTab<T, K, Q> make_tab(const double* B, const double* w) {
+QuadTab<T, K, Q> make_tab(const double* B, const double* w, double lead) {
     QuadTab<T, K, Q> t{};
     auto fill = [&](int g, int src) {
         for (int r = 0; r < K; ++r) {
@@ -720,7 +747,7 @@ QuadTab<T, K, Q> make_tab(const double* B, const double* w) {
         for (int r = 0; r < K; ++r) {
             const double sr = (r & 1) ? sign : 1.0;
             cst_set(t.TB[it][r], sr * B[src * K + r]);
-            cst_set(t.TWB[it][r], sr * w[src] * B[src * K + r]);
+            cst_set(t.TWB[it][r], sr * w[src] * B[src * K + r] * lead);
         }
     }
     return t;
@@ -731,8 +758,9 @@ void launch_one(sgk_ctx* ctx, const PencilArgs& a, const double* B, const double
                 const ReactionDev& rx, double scale) {
     using Sh = PencilShape<T, D, K, S, JAC>;
     const Filt<T, K> F = make_filt<T, K>(two_scale);
-    const auto poly = make_poly<T, S, JAC>(rx, scale);
-    const auto tab = make_tab<T, K, Q>(B, w);
+    double lead = 1.0;
+    const auto poly = make_poly<T, S, JAC>(rx, scale, &lead);
+    const auto tab = make_tab<T, K, Q>(B, w, lead);
     const size_t smem1 = Sh::bytes(a.H);
     SGK_REQUIRE(smem1 <= ctx->smem_optin, SGK_EUNSUPPORTED, "pencil exceeds shared memory");
     // Pencils per CTA: as many cells (pairs of cells) as threads, two a
