@@ -59,8 +59,10 @@ constexpr int PD = 3;
 template <typename T, int MODE, int KP1>
 __global__ void __launch_bounds__(256) pyr_kernel(const FiberItem* __restrict__ items, int nitems,
                                                   const FiberGroup* __restrict__ groups, const T* __restrict__ src,
-                                                  T* __restrict__ dst, const __grid_constant__ Filt<T, KP1> flt, int H,
-                                                  int Nfull) {
+                                                  T* __restrict__ dst, long long sstride, long long dstride,
+                                                  const __grid_constant__ Filt<T, KP1> flt, int H, int Nfull) {
+    src += blockIdx.y * sstride;  // one species per row of the grid
+    dst += blockIdx.y * dstride;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     T* tile = reinterpret_cast<T*>(smem_raw);
     __shared__ FiberGroup sg;
@@ -227,18 +229,18 @@ __global__ void __launch_bounds__(256) pyr_kernel(const FiberItem* __restrict__ 
 
 template <typename T>
 void launch_pyr(sgk_ctx* ctx, const FiberPlan& plan, int mode, const T* src, T* dst, int H, int kp1,
-                const double* two_scale) {
+                const double* two_scale, int count, long long sstride, long long dstride) {
     if (plan.nitems == 0) return;
     int Nfull = 0;
     while ((kp1 << Nfull) < H) ++Nfull;
-    const int grid = std::min(plan.nitems, ctx->num_sms * 8);
+    const dim3 grid(std::min(plan.nitems, ctx->num_sms * 8), count);
     const size_t smem = plan.smem_bytes;
     KTimer kt(ctx, mode);
 #define SGK_PYR_CASE(M, K)                                                                                   \
     if (mode == M && kp1 == K) {                                                                             \
         allow_max_dynamic_smem(ctx->smem_optin, pyr_kernel<T, M, K>);          \
         pyr_kernel<T, M, K><<<grid, 256, smem, ctx->stream>>>(plan.items.p, plan.nitems, plan.groups.p, src,     \
-                                                                  dst, make_filt<T, K>(two_scale), H, Nfull);  \
+                                                                  dst, sstride, dstride, make_filt<T, K>(two_scale), H, Nfull);  \
     }
     SGK_PYR_CASE(FIBER_FWD, 2)
     SGK_PYR_CASE(FIBER_FWD, 3)
@@ -251,9 +253,12 @@ void launch_pyr(sgk_ctx* ctx, const FiberPlan& plan, int mode, const T* src, T* 
     count_launch(ctx);
 }
 
-template void launch_pyr<double>(sgk_ctx*, const FiberPlan&, int, const double*, double*, int, int, const double*);
-template void launch_pyr<float>(sgk_ctx*, const FiberPlan&, int, const float*, float*, int, int, const double*);
-template void launch_pyr<dfloat>(sgk_ctx*, const FiberPlan&, int, const dfloat*, dfloat*, int, int, const double*);
+template void launch_pyr<double>(sgk_ctx*, const FiberPlan&, int, const double*, double*, int, int, const double*, int,
+                                 long long, long long);
+template void launch_pyr<float>(sgk_ctx*, const FiberPlan&, int, const float*, float*, int, int, const double*, int,
+                                 long long, long long);
+template void launch_pyr<dfloat>(sgk_ctx*, const FiberPlan&, int, const dfloat*, dfloat*, int, int, const double*, int,
+                                 long long, long long);
 
 // Host mirror of the kernel's address arithmetic, for plan validation.
 static long long chunk_addr_host(const FiberGroup& g, long long o, int pos, long long in, int kp1, int I) {

@@ -48,58 +48,6 @@ __global__ void reduce_final_kernel(const double* __restrict__ partials, int nb,
     if (threadIdx.x == 0) out[0] = mode == 1 ? sqrt(acc) : acc;
 }
 
-// partials[block][c] = sum_e V[c][e] w[e] over the block's elements, c < ncols
-template <typename T>
-__global__ void mdot_partial_kernel(const T* __restrict__ V, long long ldv, int ncols, const T* __restrict__ w,
-                                    long long n, double* __restrict__ partials, const int* __restrict__ stop) {
-    if (stop && *stop) return;
-    __shared__ double sh[32];
-    constexpr int CH = 8;
-    for (int c0 = 0; c0 < ncols; c0 += CH) {
-        double acc[CH];
-#pragma unroll
-        for (int c = 0; c < CH; ++c) acc[c] = 0.0;
-        for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
-             i += (long long)gridDim.x * blockDim.x) {
-            const double wv = (double)w[i];
-#pragma unroll
-            for (int c = 0; c < CH; ++c)
-                if (c0 + c < ncols) acc[c] += (double)V[(c0 + c) * ldv + i] * wv;
-        }
-#pragma unroll
-        for (int c = 0; c < CH; ++c) {
-            if (c0 + c >= ncols) break;
-            const double s = block_sum(acc[c], sh);
-            if (threadIdx.x == 0) partials[(long long)blockIdx.x * ncols + c0 + c] = s;
-        }
-    }
-}
-
-__global__ void mdot_final_kernel(const double* __restrict__ partials, int nb, int ncols, double* __restrict__ out,
-                                  const int* __restrict__ stop) {
-    if (stop && *stop) return;
-    for (int c = threadIdx.x; c < ncols; c += blockDim.x) {
-        double acc = 0.0;
-        for (int b = 0; b < nb; ++b) acc += partials[(long long)b * ncols + c];
-        out[c] = acc;
-    }
-}
-
-// w -= V[:, :ncols] h  (arithmetic in T)
-template <typename T>
-__global__ void gs_update_kernel(const T* __restrict__ V, long long ldv, int ncols, const double* __restrict__ h,
-                                 T* __restrict__ w, long long n, const int* __restrict__ stop) {
-    if (stop && *stop) return;
-    __shared__ T hs[SGK_MAX_KRYLOV + 1];
-    for (int c = threadIdx.x; c < ncols; c += blockDim.x) hs[c] = (T)h[c];
-    __syncthreads();
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-        T acc = T(0);
-        for (int c = 0; c < ncols; ++c) acc += V[c * ldv + i] * hs[c];
-        w[i] -= acc;
-    }
-}
-
 // Start of an Arnoldi process: gamma = ||v||, flags reset, breakdown if v = 0.
 __global__ void krylov_init_kernel(const double* __restrict__ gamma2, KrylovScalars* __restrict__ ks) {
     const double g = sqrt(*gamma2);
@@ -148,7 +96,7 @@ constexpr int GS_E = 128;
 // FMAs and shuffle reductions interleave instead of waiting on one another.
 template <typename T>
 __device__ __forceinline__ void warp_column_dots(const T* __restrict__ V, long long ldv, int ncols, const T* ws,
-                                                 long long i0, double* __restrict__ partials) {
+                                                 long long n, long long i0, double* __restrict__ partials) {
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
     double wl[GS_E / 32];
 #pragma unroll
@@ -162,7 +110,8 @@ __device__ __forceinline__ void warp_column_dots(const T* __restrict__ V, long l
             if (c < ncols) {
                 const T* vc = V + c * ldv + i0;
 #pragma unroll
-                for (int k = 0; k < GS_E / 32; ++k) a[u] += (double)vc[lane + 32 * k] * wl[k];
+                for (int k = 0; k < GS_E / 32; ++k)
+                    if (i0 + lane + 32 * k < n) a[u] += (double)vc[lane + 32 * k] * wl[k];
             }
         }
 #pragma unroll
@@ -244,13 +193,11 @@ template <typename T>
 __global__ void __launch_bounds__(GS_E) arn_dots_kernel(const T* __restrict__ V, long long ldv, int ncols, T* w,
                                                         long long n, double* __restrict__ partials, unsigned* counter,
                                                         double* __restrict__ h, const int* __restrict__ stop) {
-    if (*stop) return;
+    if (stop && *stop) return;
     __shared__ T ws[GS_E];
     const long long i0 = (long long)blockIdx.x * GS_E;
     slice_update<T>(V, ldv, ncols, nullptr, w, n, i0, ws, false);
-    // the last slice reads V beyond n only where ws is zero; V has M + 1
-    // full columns, so the reads stay inside the basis allocation
-    warp_column_dots<T>(V, ldv, ncols, ws, i0, partials);
+    warp_column_dots<T>(V, ldv, ncols, ws, n, i0, partials);
     if (last_block(counter)) final_columns(partials, gridDim.x, ncols, h);
 }
 
@@ -260,27 +207,23 @@ __global__ void __launch_bounds__(GS_E) arn_update_dots_kernel(const T* __restri
                                                                const double* __restrict__ h1, T* w, long long n,
                                                                double* __restrict__ partials, unsigned* counter,
                                                                double* __restrict__ h2, const int* __restrict__ stop) {
-    if (*stop) return;
+    if (stop && *stop) return;
     __shared__ T ws[GS_E];
     __shared__ T hs[SGK_MAX_KRYLOV + 1];
     for (int c = threadIdx.x; c < ncols; c += blockDim.x) hs[c] = (T)h1[c];
     __syncthreads();
     const long long i0 = (long long)blockIdx.x * GS_E;
     slice_update<T>(V, ldv, ncols, hs, w, n, i0, ws, true);
-    warp_column_dots<T>(V, ldv, ncols, ws, i0, partials);
+    warp_column_dots<T>(V, ldv, ncols, ws, n, i0, partials);
     if (last_block(counter)) final_columns(partials, gridDim.x, ncols, h2);
 }
 
-// w -= V h2, ||w||^2, and in the last block: column j of H, the breakdown
-// test and 1 / h_{j+1,j}
+// w -= V h2 and ||w||^2; true in the last block, which has the sum in *beta2
+// (shared memory)
 template <typename T>
-__global__ void __launch_bounds__(GS_E) arn_update_norm_kernel(const T* __restrict__ V, long long ldv, int ncols,
-                                                               const double* __restrict__ h1,
-                                                               const double* __restrict__ h2, T* w, long long n,
-                                                               double* __restrict__ partials, unsigned* counter,
-                                                               double* __restrict__ H, int j, int M,
-                                                               KrylovScalars* __restrict__ ks) {
-    if (ks->stop) return;
+__device__ __forceinline__ bool update_norm(const T* __restrict__ V, long long ldv, int ncols,
+                                            const double* __restrict__ h2, T* w, long long n,
+                                            double* __restrict__ partials, unsigned* counter, double* beta2) {
     __shared__ T ws[GS_E];
     __shared__ T hs[SGK_MAX_KRYLOV + 1];
     __shared__ double wsum[GS_E / 32];
@@ -297,11 +240,24 @@ __global__ void __launch_bounds__(GS_E) arn_update_norm_kernel(const T* __restri
         for (int k = 0; k < GS_E / 32; ++k) t += wsum[k];
         partials[blockIdx.x] = t;
     }
-    if (!last_block(counter)) return;
-    __shared__ double beta2;
-    final_columns(partials, gridDim.x, 1, &beta2);
+    if (!last_block(counter)) return false;
+    final_columns(partials, gridDim.x, 1, beta2);
     __syncthreads();
-    if (threadIdx.x != 0) return;
+    return true;
+}
+
+// w -= V h2, ||w||^2, and in the last block: column j of H, the breakdown
+// test and 1 / h_{j+1,j}
+template <typename T>
+__global__ void __launch_bounds__(GS_E) arn_update_norm_kernel(const T* __restrict__ V, long long ldv, int ncols,
+                                                               const double* __restrict__ h1,
+                                                               const double* __restrict__ h2, T* w, long long n,
+                                                               double* __restrict__ partials, unsigned* counter,
+                                                               double* __restrict__ H, int j, int M,
+                                                               KrylovScalars* __restrict__ ks) {
+    if (ks->stop) return;
+    __shared__ double beta2;
+    if (!update_norm<T>(V, ldv, ncols, h2, w, n, partials, counter, &beta2) || threadIdx.x != 0) return;
     double f = ks->fro2;
     if (j >= 1) {
         const double sub = H[(long long)j * M + (j - 1)];
@@ -909,22 +865,20 @@ __global__ void basis_accumulate_kernel(const double* __restrict__ V, long long 
 // GMRES: Givens rotations on column j of the (restart+1) x restart matrix
 // Hg (row-major, ld = restart), update of g; reports |g_{j+1}|, h_{j+1,j}
 // and the rotated diagonal to the host.
-__global__ void gmres_givens_kernel(int j, int ld, double* __restrict__ Hg, double* __restrict__ cs,
-                                    double* __restrict__ sn, double* __restrict__ g, const double* __restrict__ h1,
-                                    const double* __restrict__ h2, const double* __restrict__ hn2,
-                                    double* __restrict__ report) {
-    if (threadIdx.x != 0) return;
-    for (int i = 0; i <= j; ++i) Hg[i * ld + j] = h1[i] + h2[i];
-    const double hn = sqrt(*hn2);
-    Hg[(j + 1) * ld + j] = hn;
+__device__ __forceinline__ void gmres_givens(int j, int ld, double* __restrict__ Hg, double* __restrict__ cs,
+                                             double* __restrict__ sn, double* __restrict__ g,
+                                             const double* __restrict__ h1, const double* __restrict__ h2, double hn2,
+                                             double* __restrict__ report) {
+    const double hn = sqrt(hn2);
+    double top = h1[0] + h2[0];  // the entry that the next rotation turns
     for (int i = 0; i < j; ++i) {
-        const double t = cs[i] * Hg[i * ld + j] + sn[i] * Hg[(i + 1) * ld + j];
-        Hg[(i + 1) * ld + j] = -sn[i] * Hg[i * ld + j] + cs[i] * Hg[(i + 1) * ld + j];
-        Hg[i * ld + j] = t;
+        const double low = h1[i + 1] + h2[i + 1];
+        Hg[i * ld + j] = cs[i] * top + sn[i] * low;
+        top = -sn[i] * top + cs[i] * low;
     }
-    const double den = hypot(Hg[j * ld + j], Hg[(j + 1) * ld + j]);
-    cs[j] = Hg[j * ld + j] / den;
-    sn[j] = Hg[(j + 1) * ld + j] / den;
+    const double den = hypot(top, hn);
+    cs[j] = top / den;
+    sn[j] = hn / den;
     Hg[j * ld + j] = den;
     Hg[(j + 1) * ld + j] = 0.0;
     g[j + 1] = -sn[j] * g[j];
@@ -933,6 +887,20 @@ __global__ void gmres_givens_kernel(int j, int ld, double* __restrict__ Hg, doub
     report[1] = hn;
     report[2] = den;
     report[3] = hn > 0.0 ? 1.0 / hn : 0.0;
+}
+
+// w -= V h2 and its norm, and in the last block the new column of the GMRES
+// system
+__global__ void __launch_bounds__(GS_E) gmres_update_norm_kernel(const double* __restrict__ V, long long ldv, int j,
+                                                                 const double* __restrict__ h1,
+                                                                 const double* __restrict__ h2, double* w, long long n,
+                                                                 double* __restrict__ partials, unsigned* counter,
+                                                                 int ld, double* __restrict__ Hg,
+                                                                 double* __restrict__ cs, double* __restrict__ sn,
+                                                                 double* __restrict__ g, double* __restrict__ report) {
+    __shared__ double hn2;
+    if (update_norm<double>(V, ldv, j + 1, h2, w, n, partials, counter, &hn2) && threadIdx.x == 0)
+        gmres_givens(j, ld, Hg, cs, sn, g, h1, h2, hn2, report);
 }
 
 // GMRES: solve the triangular system H[:m,:m] y = g[:m]
@@ -1002,26 +970,6 @@ void vk_dotT(sgk_ctx* ctx, const T* a, const T* b, long long n, double* partials
     reduce_final_kernel<<<1, RED_THREADS, 0, ctx->stream>>>(partials, nb, out, mode, stop);
     check_launch("dotT");
     count_launch(ctx, 2);
-}
-
-template <typename T>
-void vk_mdot(sgk_ctx* ctx, const T* V, long long ldv, int ncols, const T* w, long long n, double* partials,
-             double* out, const int* stop) {
-    KTimer kt(ctx, KC_REDUCE);
-    const int nb = reduction_blocks(ctx, n);
-    mdot_partial_kernel<T><<<nb, RED_THREADS, 0, ctx->stream>>>(V, ldv, ncols, w, n, partials, stop);
-    mdot_final_kernel<<<1, 256, 0, ctx->stream>>>(partials, nb, ncols, out, stop);
-    check_launch("mdot");
-    count_launch(ctx, 2);
-}
-
-template <typename T>
-void vk_gs_update(sgk_ctx* ctx, const T* V, long long ldv, int ncols, const double* h, T* w, long long n,
-                  const int* stop) {
-    KTimer kt(ctx, KC_REDUCE);
-    gs_update_kernel<T><<<grid_for(ctx, n), 256, 0, ctx->stream>>>(V, ldv, ncols, h, w, n, stop);
-    check_launch("gs_update");
-    count_launch(ctx);
 }
 
 void vk_convert(sgk_ctx* ctx, const double* x, float* y, long long n) {
@@ -1119,12 +1067,17 @@ void vk_scale_from(sgk_ctx* ctx, const double* x, double* y, long long n, const 
     check_launch("scale");
     count_launch(ctx);
 }
-void gmres_givens(sgk_ctx* ctx, int j, int ld, double* Hg, double* cs, double* sn, double* g, const double* h1,
-                  const double* h2, const double* hn2, double* report) {
-    KTimer kt(ctx, KC_VECTOR);
-    gmres_givens_kernel<<<1, 32, 0, ctx->stream>>>(j, ld, Hg, cs, sn, g, h1, h2, hn2, report);
-    check_launch("gmres_givens");
-    count_launch(ctx);
+void gmres_orthogonalise(sgk_ctx* ctx, const double* V, long long n, int j, double* w, double* partials,
+                         unsigned* counter, double* h1, double* h2, int ld, double* Hg, double* cs, double* sn,
+                         double* g, double* report) {
+    KTimer kt(ctx, KC_REDUCE);
+    const int nb = (int)((n + GS_E - 1) / GS_E);
+    arn_dots_kernel<double><<<nb, GS_E, 0, ctx->stream>>>(V, n, j + 1, w, n, partials, counter, h1, nullptr);
+    arn_update_dots_kernel<double><<<nb, GS_E, 0, ctx->stream>>>(V, n, j + 1, h1, w, n, partials, counter, h2, nullptr);
+    gmres_update_norm_kernel<<<nb, GS_E, 0, ctx->stream>>>(V, n, j, h1, h2, w, n, partials, counter, ld, Hg, cs, sn, g,
+                                                          report);
+    check_launch("gmres_orthogonalise");
+    count_launch(ctx, 3);
 }
 void gmres_solve(sgk_ctx* ctx, int m, int ld, const double* Hg, const double* g, double* y) {
     KTimer kt(ctx, KC_VECTOR);
@@ -1337,9 +1290,5 @@ template void krylov_expv_dev<double>(sgk_ctx*, const KrylovWork<double>&,
 template void krylov_expv_dev<float>(sgk_ctx*, const KrylovWork<float>&,
                                      const std::function<void(const float*, float*)>&, const double*, double*,
                                      long long, int, double);
-template void vk_mdot<double>(sgk_ctx*, const double*, long long, int, const double*, long long, double*, double*,
-                              const int*);
-template void vk_gs_update<double>(sgk_ctx*, const double*, long long, int, const double*, double*, long long,
-                                   const int*);
 template void vk_jac_finish<double>(sgk_ctx*, const double*, const double*, double, double*, long long);
 template void vk_jac_finish<float>(sgk_ctx*, const double*, const float*, double, double*, long long);

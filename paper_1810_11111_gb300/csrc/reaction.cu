@@ -468,6 +468,20 @@ void quad_backward(sgk_ctx* ctx, const Quad& Q, T* moments, T* tmp, T* out, int 
 }
 
 template <typename T>
+void quad_forward_one(sgk_ctx* ctx, const Quad& Q, const T* in, long long istride, T* nodal, long long nstride,
+                      int count) {
+    launch_pyr<T>(ctx, Q.fwd[0][sizeof(T) == 8 ? 0 : 1], FIBER_FWD, in, nodal, Q.H, Q.kp1, Q.tab.two_scale.data(), count,
+                  istride, nstride);
+}
+
+template <typename T>
+void quad_backward_one(sgk_ctx* ctx, const Quad& Q, const T* moments, long long mstride, T* out, long long ostride,
+                       int count) {
+    launch_pyr<T>(ctx, Q.bwd[0][sizeof(T) == 8 ? 0 : 1], FIBER_BWD, moments, out, Q.H, Q.kp1, Q.tab.two_scale.data(),
+                  count, mstride, ostride);
+}
+
+template <typename T>
 void quad_cells(sgk_ctx* ctx, const Quad& Q, const ReactionDev& rx, bool jac, const T* const* u, const T* const* w,
                 T* const* out) {
     CellParams<T> p{};
@@ -519,6 +533,12 @@ template void quad_backward<double>(sgk_ctx*, const Quad&, double*, double*, dou
 template void quad_backward<float>(sgk_ctx*, const Quad&, float*, float*, float*, int);
 template void quad_forward<dfloat>(sgk_ctx*, const Quad&, const dfloat*, dfloat*, dfloat*, int);
 template void quad_backward<dfloat>(sgk_ctx*, const Quad&, dfloat*, dfloat*, dfloat*, int);
+template void quad_forward_one<double>(sgk_ctx*, const Quad&, const double*, long long, double*, long long, int);
+template void quad_backward_one<double>(sgk_ctx*, const Quad&, const double*, long long, double*, long long, int);
+template void quad_forward_one<float>(sgk_ctx*, const Quad&, const float*, long long, float*, long long, int);
+template void quad_backward_one<float>(sgk_ctx*, const Quad&, const float*, long long, float*, long long, int);
+template void quad_forward_one<dfloat>(sgk_ctx*, const Quad&, const dfloat*, long long, dfloat*, long long, int);
+template void quad_backward_one<dfloat>(sgk_ctx*, const Quad&, const dfloat*, long long, dfloat*, long long, int);
 template void quad_cells<double>(sgk_ctx*, const Quad&, const ReactionDev&, bool, const double* const*,
                                  const double* const*, double* const*);
 template void quad_cells<float>(sgk_ctx*, const Quad&, const ReactionDev&, bool, const float* const*,

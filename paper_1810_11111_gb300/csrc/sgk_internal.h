@@ -281,10 +281,11 @@ void finalize_plan(FiberPlan& plan, std::vector<FiberGroup>& groups, int kp1, in
                    size_t smem_budget, long long src_size, long long dst_size, cudaStream_t s);
 
 // Change of basis along one direction (plan mode FIBER_FWD or FIBER_BWD) by
-// the two-scale pyramid; two_scale as in Tables1D.
+// the two-scale pyramid; two_scale as in Tables1D.  count arrays (species) at
+// sstride and dstride elements from each other in one launch.
 template <typename T>
 void launch_pyr(sgk_ctx* ctx, const FiberPlan& plan, int mode, const T* src, T* dst, int H, int kp1,
-                const double* two_scale);
+                const double* two_scale, int count = 1, long long sstride = 0, long long dstride = 0);
 
 // ------------------------------------------------------------- operator ---
 

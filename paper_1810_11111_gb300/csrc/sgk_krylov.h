@@ -118,12 +118,6 @@ void krylov_expv_persistent(sgk_ctx* ctx, const sgk_op* op, const PersistentWork
 PadeCoef pade13_coefficients();
 void vk_dot(sgk_ctx* ctx, const double* a, const double* b, long long n, double* partials, double* out, int mode,
             const int* stop);
-template <typename T>
-void vk_mdot(sgk_ctx* ctx, const T* V, long long ldv, int ncols, const T* w, long long n, double* partials,
-             double* out, const int* stop);
-template <typename T>
-void vk_gs_update(sgk_ctx* ctx, const T* V, long long ldv, int ncols, const double* h, T* w, long long n,
-                  const int* stop);
 void vk_convert(sgk_ctx* ctx, const double* x, float* y, long long n);
 void vk_convert(sgk_ctx* ctx, const float* x, double* y, long long n);
 void vk_convert(sgk_ctx* ctx, const double* x, dfloat* y, long long n);
@@ -141,8 +135,12 @@ void vk_copy_scalar(sgk_ctx* ctx, double* dst, const double* src);
 void vk_basis_accumulate(sgk_ctx* ctx, const double* V, long long ldv, int m, const double* y, double* x,
                          long long n);
 void vk_scale_from(sgk_ctx* ctx, const double* x, double* y, long long n, const double* s, const int* stop);
-void gmres_givens(sgk_ctx* ctx, int j, int ld, double* Hg, double* cs, double* sn, double* g, const double* h1,
-                  const double* h2, const double* hn2, double* report);
+// One GMRES step after w = A v_j: w orthogonalised twice against the j + 1
+// columns of V and its norm, and the new column of H with its rotations
+// (report: |residual|, ||w||, diagonal entry, 1 / ||w||), in three launches.
+void gmres_orthogonalise(sgk_ctx* ctx, const double* V, long long n, int j, double* w, double* partials,
+                         unsigned* counter, double* h1, double* h2, int ld, double* Hg, double* cs, double* sn,
+                         double* g, double* report);
 void gmres_solve(sgk_ctx* ctx, int m, int ld, const double* Hg, const double* g, double* y);
 void gmres_init(sgk_ctx* ctx, double* g, int len, const double* beta, double* inv_beta);
 void expm_e1(sgk_ctx* ctx, const double* H, int M, const int* m_dev, int m_fixed, double tau, double* ws, double* y);

@@ -38,6 +38,14 @@ template <typename T>
 void quad_forward(sgk_ctx* ctx, const Quad& Q, const T* in, T* final_nodal, T* tmp, int ndims);
 template <typename T>
 void quad_backward(sgk_ctx* ctx, const Quad& Q, T* moments, T* tmp, T* out, int ndims);
+// The same for count species in one launch where one direction changes (no
+// work array): arrays at the given strides.
+template <typename T>
+void quad_forward_one(sgk_ctx* ctx, const Quad& Q, const T* in, long long istride, T* nodal, long long nstride,
+                      int count);
+template <typename T>
+void quad_backward_one(sgk_ctx* ctx, const Quad& Q, const T* moments, long long mstride, T* out, long long ostride,
+                       int count);
 template <typename T>
 void quad_cells(sgk_ctx* ctx, const Quad& Q, const ReactionDev& rx, bool jac, const T* const* u, const T* const* w,
                 T* const* out);

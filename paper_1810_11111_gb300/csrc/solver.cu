@@ -381,24 +381,44 @@ QuadPtrs<T> qptrs(sgk_solver* s) {
 // last one is fused with the cell quadrature in the pencil kernel).
 int fiber_dims(const sgk_solver* s) { return s->Q.fused ? s->Q.d - 1 : s->Q.d; }
 
+// Change of basis of every species: src at stride n to dst at stride F.  With
+// one direction to change (d = 2, fused) the species share one launch: those
+// launches are a wave or less and cost their latency (two species at level 8:
+// 10.7 us each, 12 for both).
 template <typename T>
 void forward_species(sgk_solver* s, const T* src, T* dst, T* tmp) {
     const int nd = fiber_dims(s);
-    if (nd == 0) {
-        SGK_CUDA_CHECK(cudaMemcpyAsync(dst, src, s->n * sizeof(T), cudaMemcpyDeviceToDevice, s->ctx->stream));
+    const long long n = s->n, F = s->Q.full_size;
+    if (nd == 1) {
+        quad_forward_one<T>(s->ctx, s->Q, src, n, dst, F, s->nspecies);
         return;
     }
-    quad_forward<T>(s->ctx, s->Q, src, dst, tmp, nd);
+    for (int sp = 0; sp < s->nspecies; ++sp, src += n, dst += F) {
+        if (nd > 1) {
+            quad_forward<T>(s->ctx, s->Q, src, dst, tmp, nd);
+            continue;
+        }
+
+        SGK_CUDA_CHECK(cudaMemcpyAsync(dst, src, n * sizeof(T), cudaMemcpyDeviceToDevice, s->ctx->stream));
+    }
 }
 
+// and its transpose: mom at stride F to out at stride n
 template <typename T>
 void backward_species(sgk_solver* s, T* mom, T* tmp, T* out) {
     const int nd = fiber_dims(s);
-    if (nd == 0) {
-        SGK_CUDA_CHECK(cudaMemcpyAsync(out, mom, s->n * sizeof(T), cudaMemcpyDeviceToDevice, s->ctx->stream));
+    const long long n = s->n, F = s->Q.full_size;
+    if (nd == 1) {
+        quad_backward_one<T>(s->ctx, s->Q, mom, F, out, n, s->nspecies);
         return;
     }
-    quad_backward<T>(s->ctx, s->Q, mom, tmp, out, nd);
+    for (int sp = 0; sp < s->nspecies; ++sp, mom += F, out += n) {
+        if (nd > 1) {
+            quad_backward<T>(s->ctx, s->Q, mom, tmp, out, nd);
+            continue;
+        }
+        SGK_CUDA_CHECK(cudaMemcpyAsync(out, mom, n * sizeof(T), cudaMemcpyDeviceToDevice, s->ctx->stream));
+    }
 }
 
 template <typename T>
@@ -430,24 +450,19 @@ void cell_pass(sgk_solver* s, bool jac, T* const* u, T* const* w, T* const* out)
 template <typename T>
 void evalF_T(sgk_solver* s, const double* U, double* F) {
     QuadPtrs<T> p = qptrs<T>(s);
-    const long long n = s->n;
-    for (int sp = 0; sp < s->nspecies; ++sp) {
-        const T* src;
-        if (sizeof(T) == 8) src = reinterpret_cast<const T*>(U + sp * n);
-        else {
-            vk_convert(s->ctx, U + sp * n, reinterpret_cast<float*>(p.spin[sp]), n);
-            src = p.spin[sp];
-        }
-        forward_species<T>(s, src, p.unod[sp], p.tmp);
+    const long long N = s->n * s->nspecies;
+    const T* src = reinterpret_cast<const T*>(U);
+    if (sizeof(T) == 4) {
+        vk_convert(s->ctx, U, reinterpret_cast<float*>(p.spin[0]), N);
+        src = p.spin[0];
     }
+    forward_species<T>(s, src, p.unod[0], p.tmp);
     cell_pass<T>(s, false, p.unod, nullptr, p.wnod);
-    for (int sp = 0; sp < s->nspecies; ++sp) {
-        if (sizeof(T) == 8) {
-            backward_species<T>(s, p.wnod[sp], p.tmp, reinterpret_cast<T*>(F + sp * n));
-        } else {
-            backward_species<T>(s, p.wnod[sp], p.tmp, p.spout[sp]);
-            vk_convert(s->ctx, reinterpret_cast<const float*>(p.spout[sp]), F + sp * n, n);
-        }
+    if (sizeof(T) == 8) {
+        backward_species<T>(s, p.wnod[0], p.tmp, reinterpret_cast<T*>(F));
+    } else {
+        backward_species<T>(s, p.wnod[0], p.tmp, p.spout[0]);
+        vk_convert(s->ctx, reinterpret_cast<const float*>(p.spout[0]), F, N);
     }
     s->unod_valid = true;
 }
@@ -456,18 +471,14 @@ void evalF_T(sgk_solver* s, const double* U, double* F) {
 template <typename T>
 void evalJ_T(sgk_solver* s, const double* w, T* out) {
     QuadPtrs<T> p = qptrs<T>(s);
-    const long long n = s->n;
-    for (int sp = 0; sp < s->nspecies; ++sp) {
-        const T* src;
-        if (sizeof(T) == 8) src = reinterpret_cast<const T*>(w + sp * n);
-        else {
-            vk_convert(s->ctx, w + sp * n, reinterpret_cast<float*>(p.spin[sp]), n);
-            src = p.spin[sp];
-        }
-        forward_species<T>(s, src, p.wnod[sp], p.tmp);
+    const T* src = reinterpret_cast<const T*>(w);
+    if (sizeof(T) == 4) {
+        vk_convert(s->ctx, w, reinterpret_cast<float*>(p.spin[0]), s->n * s->nspecies);
+        src = p.spin[0];
     }
+    forward_species<T>(s, src, p.wnod[0], p.tmp);
     cell_pass<T>(s, true, p.unod, p.wnod, p.wnod);
-    for (int sp = 0; sp < s->nspecies; ++sp) backward_species<T>(s, p.wnod[sp], p.tmp, out + sp * n);
+    backward_species<T>(s, p.wnod[0], p.tmp, out);
 }
 
 // F(U) in double-float arithmetic (the fused pencil path): U split into
@@ -475,16 +486,12 @@ void evalJ_T(sgk_solver* s, const double* w, T* out) {
 // result summed back to FP64; caches the transformed U (pairs) in unod.
 void evalF_df(sgk_solver* s, const double* U, double* F) {
     QuadPtrs<dfloat> p = qptrs<dfloat>(s);
-    const long long n = s->n;
-    for (int sp = 0; sp < s->nspecies; ++sp) {
-        vk_convert(s->ctx, U + sp * n, p.spin[sp], n);
-        forward_species<dfloat>(s, p.spin[sp], p.unod[sp], p.tmp);
-    }
+    const long long N = s->n * s->nspecies;
+    vk_convert(s->ctx, U, p.spin[0], N);
+    forward_species<dfloat>(s, p.spin[0], p.unod[0], p.tmp);
     cell_pass<dfloat>(s, false, p.unod, nullptr, p.wnod);
-    for (int sp = 0; sp < s->nspecies; ++sp) {
-        backward_species<dfloat>(s, p.wnod[sp], p.tmp, p.spout[sp]);
-        vk_convert(s->ctx, p.spout[sp], F + sp * n, n);
-    }
+    backward_species<dfloat>(s, p.wnod[0], p.tmp, p.spout[0]);
+    vk_convert(s->ctx, p.spout[0], F, N);
     s->unod_valid = true;
 }
 
@@ -632,7 +639,6 @@ void gmres_solve_host(sgk_solver* s, const double* G, double* x, int& iters) {
     double* w = s->cg_q.p;
     double* V = s->gm_V.p;
     double* beta = s->scal.p + 2;
-    double* hn2 = s->scal.p + 3;
     double* rep = s->gm_report.p;
     vk_axpby(ctx, -1.0, G, 0.0, G, b, N);
     SGK_CUDA_CHECK(cudaMemsetAsync(x, 0, N * sizeof(double), ctx->stream));
@@ -658,12 +664,8 @@ void gmres_solve_host(sgk_solver* s, const double* G, double* x, int& iters) {
         double last_g = beta_h;
         for (int j = 0; j < m; ++j) {
             apply_newton_matrix(s, V + (long long)j * N, w);
-            vk_mdot<double>(ctx, V, N, j + 1, w, N, s->partials.p, s->h1.p, nullptr);
-            vk_gs_update<double>(ctx, V, N, j + 1, s->h1.p, w, N, nullptr);
-            vk_mdot<double>(ctx, V, N, j + 1, w, N, s->partials.p, s->h2.p, nullptr);
-            vk_gs_update<double>(ctx, V, N, j + 1, s->h2.p, w, N, nullptr);
-            vk_dot(ctx, w, w, N, s->partials.p, hn2, 0, nullptr);
-            gmres_givens(ctx, j, restart, s->gm_H.p, s->gm_cs.p, s->gm_sn.p, s->gm_g.p, s->h1.p, s->h2.p, hn2, rep);
+            gmres_orthogonalise(ctx, V, N, j, w, s->partials.p, s->counters.p, s->h1.p, s->h2.p, restart, s->gm_H.p,
+                                s->gm_cs.p, s->gm_sn.p, s->gm_g.p, rep);
             SGK_CUDA_CHECK(cudaMemcpyAsync(s->ctx->hscal, rep, 4 * sizeof(double), cudaMemcpyDeviceToHost, ctx->stream));
             SGK_CUDA_CHECK(cudaStreamSynchronize(ctx->stream));
             used = j + 1;
@@ -770,14 +772,12 @@ void solver_jacobian_apply(sgk_solver* s, const double* U, const double* w, doub
     const long long n = s->n;
     if (s->prec == SGK_FP64) {
         QuadPtrs<double> p = qptrs<double>(s);
-        for (int sp = 0; sp < s->nspecies; ++sp) forward_species<double>(s, U + sp * n, p.unod[sp], p.tmp);
+        forward_species<double>(s, U, p.unod[0], p.tmp);
         evalJ_T<double>(s, w, jw);
     } else {
         QuadPtrs<float> p = qptrs<float>(s);
-        for (int sp = 0; sp < s->nspecies; ++sp) {
-            vk_convert(s->ctx, U + sp * n, p.spin[sp], n);
-            forward_species<float>(s, p.spin[sp], p.unod[sp], p.tmp);
-        }
+        vk_convert(s->ctx, U, p.spin[0], n * s->nspecies);
+        forward_species<float>(s, p.spin[0], p.unod[0], p.tmp);
         evalJ_T<float>(s, w, s->jw32.p);
         vk_convert(s->ctx, s->jw32.p, jw, n * s->nspecies);
     }
@@ -1473,7 +1473,7 @@ void solver_alloc(sgk_solver* s) {
     s->h2.alloc(std::max(M, s->opts.gmres_restart) + 1);
     s->ky.alloc(M + 1);
     s->scal.alloc(16);
-    const size_t nblk = std::max<size_t>(reduction_blocks(s->ctx, N), (size_t)((n + 127) / 128));
+    const size_t nblk = std::max<size_t>(reduction_blocks(s->ctx, N), (size_t)((N + 127) / 128));
     s->partials.alloc(nblk * (std::max(M, s->opts.gmres_restart) + 1) + 16);
     s->expm_ws.alloc(8 * (size_t)M * M);
     s->ks.alloc(S);
