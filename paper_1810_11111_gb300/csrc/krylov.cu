@@ -984,7 +984,7 @@ void vk_convert(sgk_ctx* ctx, const float* x, double* y, long long n) {
     check_launch("convert");
     count_launch(ctx);
 }
-// double-float conversions (split, pair sum in FP64, pair sum in FP32)
+// double-float conversions (split, pair sum in FP64)
 __global__ void df_split_kernel(const double* __restrict__ x, dfloat* __restrict__ y, long long n) {
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
         y[i] = df_split(x[i]);
@@ -992,10 +992,6 @@ __global__ void df_split_kernel(const double* __restrict__ x, dfloat* __restrict
 __global__ void df_value_kernel(const dfloat* __restrict__ x, double* __restrict__ y, long long n) {
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
         y[i] = df_value(x[i]);
-}
-__global__ void df_float_kernel(const dfloat* __restrict__ x, float* __restrict__ y, long long n) {
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-        y[i] = df_float(x[i]);
 }
 void vk_convert(sgk_ctx* ctx, const double* x, dfloat* y, long long n) {
     KTimer kt(ctx, KC_VECTOR);
@@ -1007,12 +1003,6 @@ void vk_convert(sgk_ctx* ctx, const dfloat* x, double* y, long long n) {
     KTimer kt(ctx, KC_VECTOR);
     df_value_kernel<<<grid_for(ctx, n), 256, 0, ctx->stream>>>(x, y, n);
     check_launch("df_value");
-    count_launch(ctx);
-}
-void vk_convert(sgk_ctx* ctx, const dfloat* x, float* y, long long n) {
-    KTimer kt(ctx, KC_VECTOR);
-    df_float_kernel<<<grid_for(ctx, n), 256, 0, ctx->stream>>>(x, y, n);
-    check_launch("df_float");
     count_launch(ctx);
 }
 void vk_axpby(sgk_ctx* ctx, double a, const double* x, double b, const double* y, double* z, long long n) {

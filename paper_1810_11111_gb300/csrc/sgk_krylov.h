@@ -122,7 +122,6 @@ void vk_convert(sgk_ctx* ctx, const double* x, float* y, long long n);
 void vk_convert(sgk_ctx* ctx, const float* x, double* y, long long n);
 void vk_convert(sgk_ctx* ctx, const double* x, dfloat* y, long long n);
 void vk_convert(sgk_ctx* ctx, const dfloat* x, double* y, long long n);
-void vk_convert(sgk_ctx* ctx, const dfloat* x, float* y, long long n);
 void vk_axpby(sgk_ctx* ctx, double a, const double* x, double b, const double* y, double* z, long long n);
 void vk_residual(sgk_ctx* ctx, const double* U, const double* F, const double* W, double c, double* G, long long n);
 template <typename T>

@@ -221,9 +221,10 @@ __global__ void residual_norm_kernel(const double* __restrict__ U, const double*
     });
 }
 
-// CG start: x = 0, r = p = -G, rr = r.r and the first CG decision
+// CG start: x = 0, r = p = -G, rr = r.r and the first CG decision; with p32
+// also p in FP32, the input of mixed mode's Jacobian pass
 __global__ void cg_start_kernel(const double* __restrict__ G, double* __restrict__ x, double* __restrict__ r,
-                                double* __restrict__ p, long long n, double* partials, unsigned* cnt, double* rr,
+                                double* __restrict__ p, float* __restrict__ p32, long long n, double* partials, unsigned* cnt, double* rr,
                                 StepCtl* ctl, double inner_tol, int inner_max, cudaGraphConditionalHandle h) {
     double acc = 0.0;
     SGK_GRID_STRIDE(i, n) {
@@ -232,6 +233,7 @@ __global__ void cg_start_kernel(const double* __restrict__ G, double* __restrict
         x[i] = 0.0;
         r[i] = v;
         p[i] = v;
+        if (p32) p32[i] = (float)v;
         acc += v * v;
     }
     finish_sum(acc, partials, cnt, [&](double t) {
@@ -269,13 +271,17 @@ __global__ void cg_update_dot_kernel(double* __restrict__ x, double* __restrict_
     finish_sum(acc, partials, cnt, [&](double t) { *rr_new = t; });
 }
 
-// p = r + (rr_new / rr) p; then rr = rr_new (after every block has read rr)
-// and the next CG decision
-__global__ void cg_direction_kernel(double* __restrict__ p, const double* __restrict__ r, const double* rr_new,
-                                    double* rr, long long n, unsigned* cnt, StepCtl* ctl, int inner_max,
+// p = r + (rr_new / rr) p (with p32 also in FP32); then rr = rr_new (after
+// every block has read rr) and the next CG decision
+__global__ void cg_direction_kernel(double* __restrict__ p, float* __restrict__ p32, const double* __restrict__ r,
+                                    const double* rr_new, double* rr, long long n, unsigned* cnt, StepCtl* ctl, int inner_max,
                                     cudaGraphConditionalHandle h) {
     const double beta = *rr_new / *rr;
-    SGK_GRID_STRIDE(i, n) p[i] = r[i] + beta * p[i];
+    SGK_GRID_STRIDE(i, n) {
+        const double v = r[i] + beta * p[i];
+        p[i] = v;
+        if (p32) p32[i] = (float)v;
+    }
     finish_last(cnt, [&]() {
         const double v = *rr_new;
         *rr = v;
@@ -290,6 +296,31 @@ __global__ void newton_step_kernel(double* __restrict__ U, const double* __restr
     finish_last(cnt, [&]() {
         if (ctl) newton_advance(ctl);
     });
+}
+
+// The transformed U of an accurate F (FP64 or double-float) rounded to FP32
+// for the Jacobian products of a mixed-mode correction.  Launched where a
+// correction begins, not with every F: the last F of a step and the
+// predictor's are followed by no correction.  With the FP32 copy of CG's
+// direction written by the CG kernels instead of a launch of its own: two 4D
+// steps on 16.8 M points 5385 -> 5277 us, four 2D IIF3 steps 5272 -> 5156 us.
+// A step graph's first correction (it = 0) follows the FP32 residual, whose
+// transform is already in place: nothing to do.  Two values per thread and
+// round, 16-byte loads (both buffers start an allocation).  Bound by memory.
+__device__ __forceinline__ float2 jac_state_round(const double2 v) { return make_float2((float)v.x, (float)v.y); }
+__device__ __forceinline__ float2 jac_state_round(const float4 v) {
+    return make_float2(df_float(dfloat(v.x, v.y)), df_float(dfloat(v.z, v.w)));
+}
+__device__ __forceinline__ float jac_state_one(const double v) { return (float)v; }
+__device__ __forceinline__ float jac_state_one(const dfloat v) { return df_float(v); }
+
+template <typename T, typename V>
+__global__ void __launch_bounds__(256)
+    jac_state_kernel(const T* __restrict__ x, float* __restrict__ y, long long n, const StepCtl* ctl) {
+    if (ctl && ctl->it == 0) return;
+    SGK_GRID_STRIDE(i, n / 2)
+        reinterpret_cast<float2*>(y)[i] = jac_state_round(__ldcs(reinterpret_cast<const V*>(x) + i));
+    if ((n & 1) && blockIdx.x == 0 && threadIdx.x == 0) y[n - 1] = jac_state_one(x[n - 1]);
 }
 
 #undef SGK_GRID_STRIDE
@@ -467,13 +498,14 @@ void evalF_T(sgk_solver* s, const double* U, double* F) {
     s->unod_valid = true;
 }
 
-// J_F(U) w for the U cached in unod; output in T.
+// J_F(U) w for the U cached in unod; output in T.  staged: the FP32 w is in
+// spin already (the CG kernels write their direction there).
 template <typename T>
-void evalJ_T(sgk_solver* s, const double* w, T* out) {
+void evalJ_T(sgk_solver* s, const double* w, T* out, bool staged = false) {
     QuadPtrs<T> p = qptrs<T>(s);
     const T* src = reinterpret_cast<const T*>(w);
     if (sizeof(T) == 4) {
-        vk_convert(s->ctx, w, reinterpret_cast<float*>(p.spin[0]), s->n * s->nspecies);
+        if (!staged) vk_convert(s->ctx, w, reinterpret_cast<float*>(p.spin[0]), s->n * s->nspecies);
         src = p.spin[0];
     }
     forward_species<T>(s, src, p.wnod[0], p.tmp);
@@ -502,9 +534,9 @@ bool df_reaction(const sgk_solver* s) { return s->prec == SGK_MIXED && s->Q.fuse
 // F(U, t^n + toff): the reaction passes (about 1e-14 relative accuracy in
 // both precision modes), then the source terms in FP64
 //
-// In mixed mode the FP32 Jacobian passes that follow read an FP32 copy of
-// the transformed U, made here.  lo: a mixed-mode F that only seeds a
-// Newton correction and never decides acceptance runs in FP32 (and leaves
+// In mixed mode the FP32 Jacobian passes that may follow read an FP32 copy
+// of the transformed U (jacobian_state).  lo: a mixed-mode F that only seeds
+// a Newton correction and never decides acceptance runs in FP32 (and leaves
 // its FP32 transform for the Jacobian passes directly).
 // F += sum_m e^{lambda_m (t^n + toff)} S_m per species (FP64)
 void add_sources(sgk_solver* s, double* F, double toff) {
@@ -535,13 +567,27 @@ void evalF(sgk_solver* s, const double* U, double* F, double toff, bool lo = fal
     } else {
         evalF_T<double>(s, U, F);
     }
-    if (s->prec == SGK_MIXED && !lo) {
-        const long long m = (long long)s->nspecies * s->Q.full_size;
-        if (df_reaction(s)) vk_convert(s->ctx, reinterpret_cast<const dfloat*>(s->q64.p), s->q32.p, m);
-        else vk_convert(s->ctx, s->q64.p, s->q32.p, m);
-    }
     add_sources(s, F, toff);
 }
+
+// Mixed mode, before a correction's Jacobian products: the FP32 copy of the
+// accurate residual's transformed U (jac_state_kernel).
+void jacobian_state(sgk_solver* s, const StepCtl* ctl) {
+    if (s->prec != SGK_MIXED) return;
+    const long long m = (long long)s->nspecies * s->Q.full_size;
+    const int grid = (int)std::min<long long>((m / 2 + 256) / 256, 8LL * s->ctx->num_sms);
+    KTimer kt(s->ctx, KC_VECTOR);
+    if (df_reaction(s))
+        jac_state_kernel<dfloat, float4><<<grid, 256, 0, s->ctx->stream>>>(
+            reinterpret_cast<const dfloat*>(s->q64.p), s->q32.p, m, ctl);
+    else
+        jac_state_kernel<double, double2><<<grid, 256, 0, s->ctx->stream>>>(s->q64.p, s->q32.p, m, ctl);
+    check_launch("jac_state");
+    count_launch(s->ctx);
+}
+
+// where CG leaves its direction in FP32 (mixed mode), else null
+float* cg_direction32(sgk_solver* s) { return s->prec == SGK_MIXED ? qptrs<float>(s).spin[0] : nullptr; }
 
 // writes t^n to the device before a step (or a stand-alone F) reads it
 void write_time(sgk_solver* s) {
@@ -568,7 +614,8 @@ void drop_graphs(sgk_solver* s) {
     }
 }
 
-// q = p - dt/2 J_F(U) p (stacked FP64); with pq also pq = p.q
+// q = p - dt/2 J_F(U) p (stacked FP64); with pq (CG, whose direction is in
+// FP32 beside p in mixed mode) also pq = p.q
 void apply_newton_matrix(sgk_solver* s, const double* pv, double* q, double* pq = nullptr) {
     const long long N = s->n * s->nspecies;
     const double c = s->newton_c;
@@ -580,7 +627,7 @@ void apply_newton_matrix(sgk_solver* s, const double* pv, double* q, double* pq 
                              N, part, cnt, pq);
         else vk_jac_finish<double>(s->ctx, pv, s->jw64.p, c, q, N);
     } else {
-        evalJ_T<float>(s, pv, s->jw32.p);
+        evalJ_T<float>(s, pv, s->jw32.p, pq != nullptr);
         if (pq) launch_fused(s, N, "jac_finish_dot", jac_finish_dot_kernel<float>, pv, (const float*)s->jw32.p, c, q,
                              N, part, cnt, pq);
         else vk_jac_finish<float>(s->ctx, pv, s->jw32.p, c, q, N);
@@ -612,8 +659,8 @@ void cg_solve(sgk_solver* s, const double* G, double* x, int& iters) {
     double* const rr = s->scal.p + 2;
     double* const rr_new = s->scal.p + 3;
     double* const pq = s->scal.p + 4;
-    launch_fused(s, N, "cg_start", cg_start_kernel, G, x, r, pv, N, s->partials.p, s->fcnt.p + FC_CGSTART, rr,
-                 (StepCtl*)nullptr, 0.0, 0, cudaGraphConditionalHandle{});
+    launch_fused(s, N, "cg_start", cg_start_kernel, G, x, r, pv, cg_direction32(s), N, s->partials.p,
+                 s->fcnt.p + FC_CGSTART, rr, (StepCtl*)nullptr, 0.0, 0, cudaGraphConditionalHandle{});
     double rr_h = read_scalar(s, rr);
     const double stop = s->opts.inner_tol * s->opts.inner_tol * rr_h;
     iters = 0;
@@ -622,8 +669,8 @@ void cg_solve(sgk_solver* s, const double* G, double* x, int& iters) {
             apply_newton_matrix(s, pv, q, pq);
             launch_fused(s, N, "cg_update", cg_update_dot_kernel, x, r, (const double*)pv, (const double*)q,
                          (const double*)rr, (const double*)pq, N, s->partials.p, s->fcnt.p + FC_CGUPD, rr_new);
-            launch_fused(s, N, "cg_direction", cg_direction_kernel, pv, (const double*)r, (const double*)rr_new, rr,
-                         N, s->fcnt.p + FC_CGDIR, (StepCtl*)nullptr, 0, cudaGraphConditionalHandle{});
+            launch_fused(s, N, "cg_direction", cg_direction_kernel, pv, cg_direction32(s), (const double*)r,
+                         (const double*)rr_new, rr, N, s->fcnt.p + FC_CGDIR, (StepCtl*)nullptr, 0, cudaGraphConditionalHandle{});
         });
         rr_h = read_scalar(s, rr);
         ++iters;
@@ -743,6 +790,7 @@ int newton(sgk_solver* s) {
         if (!lo && g <= stop) return SGK_OK;
         if (it == s->opts.max_iter) break;
         int inner = 0;
+        if (!lo) jacobian_state(s, nullptr);
         if (s->nspecies == 1) cg_solve(s, s->G.p, s->cg_x.p, inner);
         else gmres_solve_host(s, s->G.p, s->cg_x.p, inner);
         s->stats.inner_iters += inner;
@@ -1000,8 +1048,9 @@ void build_step_graph(sgk_solver* s, int part = STEP_WHOLE) {
                     capture_while(
                         ctx, s->aux[1],
                         [&](cudaGraphConditionalHandle hc) {
-                            launch_fused(s, N, "cg_start", cg_start_kernel, (const double*)s->G.p, x, r, pv, N,
-                                         s->partials.p, s->fcnt.p + FC_CGSTART, rr, ctl, s->opts.inner_tol,
+                            jacobian_state(s, ctl);
+                            launch_fused(s, N, "cg_start", cg_start_kernel, (const double*)s->G.p, x, r, pv,
+                                         cg_direction32(s), N, s->partials.p, s->fcnt.p + FC_CGSTART, rr, ctl, s->opts.inner_tol,
                                          s->opts.inner_max, hc);
                             s->n_cgpre = ctx->launches - mark;
                         },
@@ -1011,8 +1060,8 @@ void build_step_graph(sgk_solver* s, int part = STEP_WHOLE) {
                             launch_fused(s, N, "cg_update", cg_update_dot_kernel, x, r, (const double*)pv,
                                          (const double*)q, (const double*)rr, (const double*)pq, N, s->partials.p,
                                          s->fcnt.p + FC_CGUPD, rr_new);
-                            launch_fused(s, N, "cg_direction", cg_direction_kernel, pv, (const double*)r,
-                                         (const double*)rr_new, rr, N, s->fcnt.p + FC_CGDIR, ctl,
+                            launch_fused(s, N, "cg_direction", cg_direction_kernel, pv, cg_direction32(s),
+                                         (const double*)r, (const double*)rr_new, rr, N, s->fcnt.p + FC_CGDIR, ctl,
                                          s->opts.inner_max, hc);
                             s->n_cgbody = ctx->launches - mark;
                         });

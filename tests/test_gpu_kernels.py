@@ -14,7 +14,8 @@ from oracle.krylov import krylov_expv  # noqa: E402
 from oracle.operator import (DIRICHLET0, PERIODIC, cross_blocks_1d, sipg_1d,  # noqa: E402
                              sparse_matvec, sparse_matvec_general)
 from oracle.reaction import Reaction  # noqa: E402
-from paper_1810_11111_gb300 import sgkiif  # noqa: E402
+from paper_1810_11111_gb300 import sgkiif, workloads  # noqa: E402
+from paper_1810_11111_gb300.runner import Problem  # noqa: E402
 
 pytestmark = [pytest.mark.gpu,
               pytest.mark.skipif(not torch.cuda.is_available(), reason="needs a CUDA device")]
@@ -156,3 +157,25 @@ def test_krylov_projection_mixed_derivatives(ctx, d, n, k, M, bc, monkeypatch):
     assert rel(got[0], got[1]) <= 1e-12
     op.close()
     idx.close()
+
+
+@pytest.mark.parametrize("n,k", [(0, 2), (1, 2), (3, 1), (3, 2)])  # n = 0: 27 values, an odd count
+@pytest.mark.parametrize("scheme", [sgkiif.SGK_IIF2, sgkiif.SGK_IIF3], ids=["graph", "host"])
+def test_mixed_corrections_use_the_current_state(n, k, scheme):
+    # the FP32 copy of the transformed state behind a mixed correction: a
+    # stale one only costs corrections.  Both modes stop at 1e-12 of the
+    # stage's scale; against FP64 the FP32 first residual may cost one
+    # correction a step and the inner tolerance of 1e-6 one more.
+    cfg = dict(workloads.cubic3d(n=n, k=k), scheme=scheme)
+    steps, out, its = 3, {}, {}
+    for prec in (sgkiif.SGK_FP64, sgkiif.SGK_MIXED):
+        prob = Problem(cfg, prec)
+        prob.reset()
+        U0 = np.random.default_rng(5).standard_normal(prob.U0[0].numel())
+        prob.solver.set_state(0, U0 / np.linalg.norm(U0))
+        prob.solver.step(steps)
+        out[prec] = prob.state()[0]
+        its[prec] = prob.solver.stats()["newton_iters"]
+        prob.close()
+    assert rel(out[sgkiif.SGK_MIXED], out[sgkiif.SGK_FP64]) <= 1e-10
+    assert its[sgkiif.SGK_MIXED] <= its[sgkiif.SGK_FP64] + 2 * steps
