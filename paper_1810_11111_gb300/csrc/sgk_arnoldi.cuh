@@ -112,24 +112,35 @@ __device__ __forceinline__ bool grid_barrier(unsigned* bar, unsigned target, int
     return *s_ok != 0;
 }
 
-// Gather of one output from the staged x: the entries q0 .. qe of its merged
-// row (all directions), entry q0 + i in virtual lane i mod 8 as in
-// gmv_accumulate, one chain each; a thread's 8 / G virtual lanes are
-// independent chains side by side.  The sum does not depend on G.
-template <int G>
-__device__ __forceinline__ double gather_staged(const unsigned short* ei, const double* ev, const double* xs, int q0,
-                                                int qe, int r, int ncorr, const double* hc, const double* zc,
-                                                int64_t zld) {
+// Gather of one output from the staged x, with the virtual lanes of
+// gmv_accumulate_list (entry q of a direction's row in lane q mod 8): a
+// thread's 8 / G virtual lanes are independent chains side by side, and the
+// sum does not depend on G.
+//
+// FP64: the directions one after another in two chains per virtual lane, the
+// order of gmv_accumulate_list, so that staging x changes no bit.  A rounding
+// is not harmless here: ten decaying heat steps of 192 coefficients amplify
+// one to more than 1e-9 of the result for a quarter of the initial data.
+template <int D, int G>
+__device__ __forceinline__ double gather_staged(const unsigned short* ei, const double* ev, const double* xs,
+                                                const int* eo, bool live, int r, int ncorr, const double* hc,
+                                                const double* zc, int64_t zld) {
     constexpr int VL = 8, PER = VL / G;
-    double b[PER];
+    double b[PER], s1[PER];
 #pragma unroll
-    for (int k = 0; k < PER; ++k) b[k] = 0.0;
-#pragma unroll 2
-    for (int q = q0 + r; q < qe; q += VL)
+    for (int k = 0; k < PER; ++k) b[k] = s1[k] = 0.0;
+    if (live) {
 #pragma unroll
-        for (int k = 0; k < PER; ++k)
-            if (q + k * G < qe) b[k] += ev[q + k * G] * xs[ei[q + k * G]];
-    if (ncorr > 0) {
+        for (int i = 0; i < D; ++i) {
+            const int qe = eo[i + 1];
+            for (int q = eo[i] + r; q < qe; q += 2 * VL)
+#pragma unroll
+                for (int k = 0; k < PER; ++k) {
+                    const int qk = q + k * G;
+                    if (qk < qe) b[k] += ev[qk] * xs[ei[qk]];
+                    if (qk + VL < qe) s1[k] += ev[qk + VL] * xs[ei[qk + VL]];
+                }
+        }
         double c0[PER];
 #pragma unroll
         for (int k = 0; k < PER; ++k) c0[k] = 0.0;
@@ -138,7 +149,7 @@ __device__ __forceinline__ double gather_staged(const unsigned short* ei, const 
             for (int k = 0; k < PER; ++k)
                 if (c + k * G < ncorr) c0[k] += hc[c + k * G] * zc[(c + k * G) * zld];
 #pragma unroll
-        for (int k = 0; k < PER; ++k) b[k] -= c0[k];
+        for (int k = 0; k < PER; ++k) b[k] = (b[k] + s1[k]) - c0[k];
     }
 #pragma unroll
     for (int o = 1; o < G; o <<= 1)
@@ -150,6 +161,7 @@ __device__ __forceinline__ double gather_staged(const unsigned short* ei, const 
         for (int k = 0; k + m < PER; k += 2 * m) b[k] += b[k + m];
     return b[0];
 }
+// Double-float: one chain per virtual lane over the merged row q0 .. qe.
 template <int G>
 __device__ __forceinline__ df64 gather_staged(const unsigned short* ei, const float2* ev, const float2* xs, int q0,
                                               int qe, int r, int ncorr, const float2* hc, const float2* zc,
@@ -418,7 +430,8 @@ __device__ __forceinline__ void fx_columns(const unsigned long long* set, int nt
 // Vl[c vld + u] ws[u] for c < ncols and with norm also sum ws[u]^2 as column
 // ncols: emit(c, sum) by one thread per column.  A warp per column; long
 // slices with few columns give a column several warps, whose sums meet in
-// part (16 entries of shared memory).
+// part (16 entries of shared memory).  A slice of up to four elements (the
+// smallest problems) takes one thread per column, summed in FP64.
 template <typename Emit>
 __device__ __forceinline__ void slice_dots(const double* Vl, int64_t vld, int ncols, const double* ws, int ne,
                                            bool norm, int sh, int sh_n, Fix* part, Emit&& emit) {
@@ -446,7 +459,14 @@ __device__ __forceinline__ void slice_dots(const double* Vl, int64_t vld, int nc
         }
         return fx_warp_sum(fx_fixed(a, c < ncols ? sh : sh_n));
     };
-    if (ne > 512 && nt <= PNW / 2) {
+    if (ne <= 4) {
+        for (int c = threadIdx.x; c < nt; c += PT) {
+            const double* vc = c < ncols ? Vl + c * vld : ws;
+            double a = 0.0;
+            for (int u = 0; u < ne; ++u) a = __dadd_rn(a, __dmul_rn(vc[u], ws[u]));
+            emit(c, fx_fixed(a, c < ncols ? sh : sh_n));
+        }
+    } else if (ne > 512 && nt <= PNW / 2) {
         int P = 2;
         while (2 * P * nt <= PNW) P *= 2;
         if (wid < nt * P) {
@@ -475,8 +495,12 @@ __device__ __forceinline__ void slice_dots(const double* Vl, int64_t vld, int nc
 // use(u, sum).  Short slices split the columns over four warps, one per
 // scheduler (the FP64 pipe takes 64 clocks a warp instruction, so one warp's
 // chain of M products is M times that); the four sums meet in tmp (PT
-// doubles).  Contains CTA barriers; not complete on return.
-template <typename Use>
+// doubles).  TAIL (FP64 solves): the columns beyond a multiple of four go to
+// the first sum, as in the one-thread form for long slices, so that the
+// slicing changes no bit; in mixed mode they stay one to a warp (about 1% of a
+// step of two species at 11 520 coefficients).
+// Contains CTA barriers; not complete on return.
+template <bool TAIL, typename Use>
 __device__ __forceinline__ void slice_combine(const double* Vl, int64_t vld, int ncols, const double* h, int ne,
                                               double* tmp, Use&& use) {
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -486,7 +510,10 @@ __device__ __forceinline__ void slice_combine(const double* Vl, int64_t vld, int
             const int u = base + blk;
             if (u < ne) {
                 double a = 0.0;
-                for (int c = part; c < ncols; c += 4) a += Vl[c * vld + u] * h[c];
+                const int full = TAIL ? ncols & ~3 : ncols;
+                for (int c = part; c < full; c += 4) a += Vl[c * vld + u] * h[c];
+                if (part == 0)
+                    for (int c = full; c < ncols; ++c) a += Vl[c * vld + u] * h[c];
                 tmp[part * (PT / 4) + blk] = a;
             }
             __syncthreads();
@@ -729,7 +756,7 @@ __device__ __forceinline__ void arnoldi_body(const GmvArgs<double, D>& ga, const
         if (pexpl) {
             for (int u = threadIdx.x; u < ne; u += PT) put(u, 0.0);
         } else {
-            slice_combine(Vl, vld, pj + 1, h2, ne, ctmp, put);
+            slice_combine<!DF>(Vl, vld, pj + 1, h2, ne, ctmp, put);
         }
     };
     if (threadIdx.x == 0) s_scal[1] = scale;
@@ -770,8 +797,7 @@ __device__ __forceinline__ void arnoldi_body(const GmvArgs<double, D>& ga, const
             } else {
                 double acc;
                 if (a.xs) {
-                    acc = gather_staged<G>(sei, sev, xstage, seoff[uu * D], live ? seoff[(uu + 1) * D] : 0, r,
-                                           live ? ncorr : 0, h2, Zl + uu, zld);
+                    acc = gather_staged<D, G>(sei, sev, xstage, seoff + uu * D, live, r, ncorr, h2, Zl + uu, zld);
                 } else if (seoff) {
                     acc = gmv_accumulate_list<D, G>(seoff + uu * D, sent, ga.cvk, x, r, live, ncorr, h2, Zl + uu, zld);
                 } else if (sloc) {
@@ -808,7 +834,7 @@ __device__ __forceinline__ void arnoldi_body(const GmvArgs<double, D>& ga, const
             clear_set(fx_set(j + 2, 1), nc + 1);
         }
         // w' = w - V h1, published for the next matvec
-        slice_combine(Vl, vld, nc, h1, ne, ctmp, [&](int u, double sum) {
+        slice_combine<!DF>(Vl, vld, nc, h1, ne, ctmp, [&](int u, double sum) {
             const double y = ws[u] - sum;
             ws[u] = y;
             if (DF) reinterpret_cast<float2*>(w)[lo + u] = df_to_float2(df_from_double(y));
@@ -884,7 +910,7 @@ __device__ __forceinline__ void arnoldi_body(const GmvArgs<double, D>& ga, const
                     stage_wait();
                     __syncthreads();
                 }
-                slice_combine(Vl, vld, nc, h2, ne, ctmp, [&](int u, double sum) {
+                slice_combine<!DF>(Vl, vld, nc, h2, ne, ctmp, [&](int u, double sum) {
                     const double y = ws[u] - sum;
                     ws[u] = y;
                     if (DF) reinterpret_cast<float2*>(w)[lo + u] = df_to_float2(df_from_double(y));
