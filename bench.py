@@ -146,11 +146,11 @@ def layout_sizes(d, n, k):
 # removed when the kernel changes.  Double-float F pencil launch (the
 # dominant kernel of the cell-quadrature class in mixed mode), keyed by (d,
 # level, degree, precision): profiles/pencil_kernel_cubic3d_l6k2_dfloat.md
-PENCIL_TRAFFIC = {(3, 6, 2, "mixed"): 57394944 + 13584896}
+PENCIL_TRAFFIC = {(3, 6, 2, "mixed"): 56705536 + 9454336}
 # one persistent Arnoldi launch (one exponential), keyed by (d, level,
 # degree, M, precision): profiles/arnoldi_kernel_cubic3d_l6k2_m30.md (the
 # mixed-precision variant, double-float gather)
-ARNOLDI_TRAFFIC = {(3, 6, 2, 30, "mixed"): 6501376 + 54016}
+ARNOLDI_TRAFFIC = {(3, 6, 2, 30, "mixed"): 6505728 + 105216}
 
 
 def pencil_q(cfg):
@@ -427,7 +427,7 @@ def native(args, rank, world, local_rank):
                             work_model="FP32-pipe flops: 2 per FP32 multiply-add, 24 per double-float "
                                        "multiply-add (12 FP32 operations); algorithmic multiply-adds of the "
                                        "sum-factorised quadrature and the two-scale pyramids of the last "
-                                       "direction" if mixed else "FP64 flops, 2 per multiply-add",
+                                       "direction (the kernel's even and odd sums do about half of them)" if mixed else "FP64 flops, 2 per multiply-add",
                             peak_source="derived: 152 SMs x 128 FP32 lanes x 2 flop x max SM clock" if mixed
                             else "nominal FP64 rate of the part (1.25 TFLOP/s)",
                             algorithmic_flops_per_launch=flops_algo / nl,

@@ -58,8 +58,8 @@ extern "C" {
                         in FP32; the Krylov matvec and every other F(U) (the
                         predictor's and each accepting Newton residual's) in
                         double-float arithmetic (pairs of FP32 numbers, about
-                        48 significand bits; F in FP64 where the fused
-                        reaction kernel does not serve the shape); the
+                        48 significand bits; F in FP64 for shapes without
+                        a double-float reaction pass); the
                         Gram-Schmidt inner products and norms, exp(tau H), the
                         state and the Newton residual vector in FP64.  The
                         interpolation form of F (SGK_REACTION_INTERP) runs in

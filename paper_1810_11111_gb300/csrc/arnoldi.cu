@@ -12,8 +12,8 @@
 // sums it explicitly); with the double-float matvec one more barrier at the
 // start publishes the pairs of v / gamma for the first gathers (pairs of
 // FP32 numbers cannot hold an unnormalised v of tiny magnitude).  The sums,
-// inside a CTA and across CTAs, are exact: partials become 128-bit
-// fixed-point integers, added by shuffles, then into integer accumulators
+// inside a CTA and across CTAs, are exact: partials (a lane's, or a whole
+// slice's of up to four elements) become 128-bit fixed-point integers, added by shuffles, then into integer accumulators
 // with atomic adds, and after the barrier every CTA reads the same totals, so
 // all CTAs hold bitwise equal h1, h2 and beta and take the same breakdown
 // decision without another barrier; the results do not depend on the order
@@ -31,7 +31,8 @@
 // after sums by integers, updates over all four schedulers, scalars beside
 // the gathers and the staged vector: 350 -> 300 us there, 541 -> 505 at
 // 18 576 x 30, 684 -> 640 at 11 520 x 40, 449 -> 388 at 8 832 x 30, 1240 ->
-// 1184 at 44 032 x 30, 15.9 -> 13.5 ms at 850 176 x 30.
+// 1184 at 44 032 x 30, 15.9 -> 13.5 ms at 850 176 x 30 (1116 us and 12.6 ms
+// with the 32-bit gathers of sgk_gmv.h).
 //
 // Barriers are counters in global memory with a bounded wait: a CTA that
 // waits longer than the limit sets an error flag and returns, and every

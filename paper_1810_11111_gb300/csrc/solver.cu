@@ -19,8 +19,8 @@
 // FP32 copy of the transformed U), and so does the first residual of a step,
 // which only seeds the first correction and never accepts; every other F
 // that fixes the answer -- the predictor's F(U^n) and each Newton residual's
-// F(U) -- runs in double-float arithmetic (about 1e-14 relative, FP64 where
-// the fused pencil kernel does not serve the shape), so Newton's fixed point
+// F(U) -- runs in double-float arithmetic (about 1e-14 relative, FP64 for the
+// shapes without a double-float pencil kernel), so Newton's fixed point
 // is that of the FP64 path and the outer stop is the same ||G||_2 <= tol
 // max(||W||_2, ||G(W)||_2) in both modes (an inexact Jacobian only changes
 // the convergence rate).  With the interpolation form of F (interp.cu) the
