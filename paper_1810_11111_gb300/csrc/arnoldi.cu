@@ -11,28 +11,37 @@
 // (the norm of w'' follows by Pythagoras; near breakdown a third barrier
 // sums it explicitly); with the double-float matvec one more barrier at the
 // start publishes the pairs of v / gamma for the first gathers (pairs of
-// FP32 numbers cannot hold an unnormalised v of tiny magnitude).  The sums,
-// inside a CTA and across CTAs, are exact: partials (a lane's, or a whole
-// slice's of up to four elements) become 128-bit fixed-point integers, added by shuffles, then into integer accumulators
-// with atomic adds, and after the barrier every CTA reads the same totals, so
-// all CTAs hold bitwise equal h1, h2 and beta and take the same breakdown
-// decision without another barrier; the results do not depend on the order
-// in which CTAs arrive.  The next matvec gathers the unnormalised w' and
-// forms A v_{j+1} = (A w' - Z h2) / beta from the stored raw outputs Z; it
-// starts before 1 / beta is known.  The two w buffers alternate so that those
-// gathers never race with the writes of the next step.  Accumulator sets
-// rotate over three steps for the same reason.
+// FP32 numbers cannot hold an unnormalised v of tiny magnitude).  The
+// cross-CTA sums are exact: every CTA's partial becomes a 128-bit fixed-point
+// integer and is added to integer accumulators with atomic adds, and after
+// the barrier every CTA reads the same totals, so all CTAs hold bitwise equal
+// h1, h2 and beta and take the same breakdown decision without another
+// barrier; the results do not depend on the order in which CTAs arrive.  The
+// next matvec gathers the unnormalised w' and forms A v_{j+1} =
+// (A w' - Z h2) / beta from the stored raw outputs Z; it starts before
+// 1 / beta is known.  The two w buffers alternate so that those gathers never
+// race with the writes of the next step.  Accumulator sets rotate over three
+// steps for the same reason.
 //
-// Bound: latency.  A step at 5 184 coefficients, 25 columns (24 000 clocks):
-// 2 x 4 950 for a barrier and the read of the sums behind it (additions to
-// arrive, release, poll, read, each an L2 round trip), 2 x 1 900 for inner
-// products, 2 x 1 750 for the updates, 2 500 for the gathers, 3 500 for
-// staging the gathered vector, the rest scalars.  Per exponential, before and
-// after sums by integers, updates over all four schedulers, scalars beside
-// the gathers and the staged vector: 350 -> 300 us there, 541 -> 505 at
-// 18 576 x 30, 684 -> 640 at 11 520 x 40, 449 -> 388 at 8 832 x 30, 1240 ->
-// 1184 at 44 032 x 30, 15.9 -> 13.5 ms at 850 176 x 30 (1116 us and 12.6 ms
-// with the 32-bit gathers of sgk_gmv.h).
+// The order of every sum is fixed, in both arithmetics, whatever the lanes per
+// output and the memory that holds a slice, and a change of layout keeps it to
+// the bit: the method's unconverged projections amplify a rounding by up to
+// ten orders of magnitude for some initial data (one heat step at d = 4, level
+// 4, degree 1, M = 30 moves by 1e-5 of its result).
+//
+// Bound: latency.  A step is a chain of two barriers with the reads of the
+// sums behind them (arrive, release, poll, read: about 5 000 clocks each at
+// 152 CTAs), two inner products, two updates and the gathers.  1 / beta is
+// formed beside the gathers, the updates use all four schedulers, and the
+// column sums that need no scale run while long rows are gathered.  Per
+// exponential, FP64 (double-float matvec), without and with these: 192 x 20
+// 333 -> 306 us (351 -> 307), 5 504 x 25 453 -> 428 (469 -> 430), 11 520 x 40
+// 876 -> 826 (861 -> 782), 17 408 x 20 443 -> 427 (441 -> 423), 18 576 x 30
+// 681 -> 667 (665 -> 643), 32 768 x 20 543 -> 538 (529 -> 509), 44 712 x 30
+// 1214 -> 1135 (1157 -> 1079).  Staging the gathered vector in shared memory
+// costs more than the gathers through L1 that it saves (11 520 x 40: 888
+// against 826 us, 8 832 x 30: 590 and 531), except where the entries come from
+// L2 anyway (eo1).
 //
 // Barriers are counters in global memory with a bounded wait: a CTA that
 // waits longer than the limit sets an error flag and returns, and every
@@ -209,39 +218,22 @@ ArnPrep arnoldi_prepare(sgk_ctx* ctx, const sgk_op* op, const PersistentWork& pw
     a.smem_loc = 0;
     a.list_cap = 0;
     a.cvk2 = op->gmv_cvk2.p;
-    // The gathered vector staged in shared memory, where it fits beside the
-    // slices of w and the entries (10 bytes each): copied as a whole past L1,
-    // which is empty after every step's acquire, the gathers themselves take
-    // 2 800 to 4 200 clocks a step at 8 832 and 11 520 coefficients on 152
-    // CTAs (the whole process 650 and 423 us, 690 and 449 with gathers through
-    // L1).  The slices of V and Z go to shared memory next.  With the entries
-    // streamed from L2 beside a staged vector (18 576 coefficients) the copy
-    // and the stream cost more than they saved: 564 against 541 us.
     const bool mixed = ctx->precision == SGK_MIXED;
-    const size_t xb = sizeof(double) * (size_t)((n + 1) / 2 * 2);
-    const size_t lst10 = sgk_arn::arn_eoff_bytes((int)E, d) + 10 * (size_t)std::max<int64_t>(list_ent, 1);
-    a.ei = op->gmv_ei.p;
-    a.ev = op->gmv_ev.p;
-    a.ev2 = op->gmv_ev2.p;
-    a.xs = a.ei != nullptr && (mixed ? a.ev2 != nullptr : a.ev != nullptr) && xb + ws + lst10 <= budget;
     size_t smem;
     a.eo1 = nullptr;
+    a.ei = nullptr;
+    a.ev = nullptr;
     if (op->npairs > 0) {
         // mixed derivatives: one list per output, FP64 in both modes
         const size_t off = sgk_arn::arn_eoff_bytes((int)E, 1);
+        const size_t xb = sizeof(double) * (size_t)((n + 1) / 2 * 2);
         SGK_REQUIRE(op->x1_off.p && xb + ws + off <= budget, SGK_EUNSUPPORTED, "persistent Arnoldi: no entry lists");
-        a.xs = 1;
         a.eo1 = op->x1_off.p;
         a.ei = op->x1_ei.p;
         a.ev = op->x1_ev.p;
         a.smem_vz = xb + ws + off + vz <= budget;
         smem = xb + ws + off + (a.smem_vz ? vz : 0);
         a.df = 0;
-    } else if (a.xs) {
-        a.smem_vz = xb + ws + lst10 + vz <= budget;
-        a.list_cap = (int)std::max<int64_t>(list_ent, 1);
-        smem = xb + ws + lst10 + (a.smem_vz ? vz : 0);
-        a.df = mixed;
     } else {
         if (has_list && ws + vz + lst <= budget) {
             a.smem_vz = 1;

@@ -13,19 +13,6 @@
 
 namespace {
 
-// pre-located entries {index of x, index of the value} -> index and value
-__global__ void gmv_flat_kernel(int64_t count, const int2* __restrict__ ent, const double* __restrict__ cvk,
-                                const float2* __restrict__ cvk2, unsigned short* __restrict__ ei,
-                                double* __restrict__ ev, float2* __restrict__ ev2) {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < count; i += (int64_t)gridDim.x * blockDim.x) {
-        const int2 e = ent[i];
-        ei[i] = (unsigned short)e.x;
-        if (ev) ev[i] = cvk[e.y];
-        if (ev2) ev2[i] = cvk2[e.y];
-    }
-}
-
-
 template <typename T, int D, int KP1, int G, typename IX>
 __global__ void __launch_bounds__(256) gmv_kernel(const GmvArgs<T, D> a, const T* __restrict__ x,
                                                   T* __restrict__ y) {
@@ -231,17 +218,6 @@ void build_gmv_tables(sgk_op* op) {
     op->gmv_cvk.upload(cvk, op->ctx->stream);
     op->gmv_cvkf.upload(cvkf, op->ctx->stream);
     op->gmv_cvk2.upload(cvk2, op->ctx->stream);
-    if (!ent.empty() && idx->dof <= GMV_STAGED_MAX) {
-        const bool mixed = op->ctx->precision == SGK_MIXED;
-        const int64_t count = (int64_t)ent.size();
-        op->gmv_ei.alloc(count);
-        if (mixed) op->gmv_ev2.alloc(count);
-        else op->gmv_ev.alloc(count);
-        gmv_flat_kernel<<<(int)std::min<int64_t>((count + 255) / 256, 1024), 256, 0, op->ctx->stream>>>(
-            count, op->gmv_ent.p, op->gmv_cvk.p, op->gmv_cvk2.p, op->gmv_ei.p, op->gmv_ev.p, op->gmv_ev2.p);
-        check_launch("gmv_flat_kernel");
-        count_launch(op->ctx);
-    }
     op->gmv_ce.upload(ce, op->ctx->stream);
     op->gmv_cb.upload(cb, op->ctx->stream);
     op->gmv_chunk.upload(chunk, op->ctx->stream);

@@ -27,18 +27,13 @@ struct ArnArgs {
     // vectors (w0, w1) and Z then hold (hi, lo) pairs instead of doubles
     const float2* cvk2;
     int df;
-    // xs: the whole gathered vector (8 n bytes) is staged in shared memory
-    // before every matvec, and the gathers read it there; the entries (at
-    // most list_cap) then come with their own values (entry q: ei[q], and
-    // ev[q] or ev2[q]), staged in shared memory too
-    int xs;
     // eo1: one list per output over all terms of an operator with mixed
-    // derivatives (offset of output g; ei, ev), read from L2 in order with x
-    // staged; else null
+    // derivatives (offset of output g; entry q: index of x ei[q], value
+    // ev[q]), read from L2 in order, with the whole gathered vector (8 n
+    // bytes) staged in shared memory before every matvec; else null
     const int* eo1;
     const unsigned short* ei;
     const double* ev;
-    const float2* ev2;
     const double* v;
     double* V;  // column c at V + c n
     double* w0;
@@ -110,93 +105,6 @@ __device__ __forceinline__ bool grid_barrier(unsigned* bar, unsigned target, int
     }
     __syncthreads();
     return *s_ok != 0;
-}
-
-// Gather of one output from the staged x, with the virtual lanes of
-// gmv_accumulate_list (entry q of a direction's row in lane q mod 8): a
-// thread's 8 / G virtual lanes are independent chains side by side, and the
-// sum does not depend on G.
-//
-// FP64: the directions one after another in two chains per virtual lane, the
-// order of gmv_accumulate_list, so that staging x changes no bit.  A rounding
-// is not harmless here: ten decaying heat steps of 192 coefficients amplify
-// one to more than 1e-9 of the result for a quarter of the initial data.
-template <int D, int G>
-__device__ __forceinline__ double gather_staged(const unsigned short* ei, const double* ev, const double* xs,
-                                                const int* eo, bool live, int r, int ncorr, const double* hc,
-                                                const double* zc, int64_t zld) {
-    constexpr int VL = 8, PER = VL / G;
-    double b[PER], s1[PER];
-#pragma unroll
-    for (int k = 0; k < PER; ++k) b[k] = s1[k] = 0.0;
-    if (live) {
-#pragma unroll
-        for (int i = 0; i < D; ++i) {
-            const int qe = eo[i + 1];
-            for (int q = eo[i] + r; q < qe; q += 2 * VL)
-#pragma unroll
-                for (int k = 0; k < PER; ++k) {
-                    const int qk = q + k * G;
-                    if (qk < qe) b[k] += ev[qk] * xs[ei[qk]];
-                    if (qk + VL < qe) s1[k] += ev[qk + VL] * xs[ei[qk + VL]];
-                }
-        }
-        double c0[PER];
-#pragma unroll
-        for (int k = 0; k < PER; ++k) c0[k] = 0.0;
-        for (int c = r; c < ncorr; c += VL)
-#pragma unroll
-            for (int k = 0; k < PER; ++k)
-                if (c + k * G < ncorr) c0[k] += hc[c + k * G] * zc[(c + k * G) * zld];
-#pragma unroll
-        for (int k = 0; k < PER; ++k) b[k] = (b[k] + s1[k]) - c0[k];
-    }
-#pragma unroll
-    for (int o = 1; o < G; o <<= 1)
-#pragma unroll
-        for (int k = 0; k < PER; ++k) b[k] += __shfl_xor_sync(0xffffffffu, b[k], o);
-#pragma unroll
-    for (int m = 1; m < PER; m <<= 1)
-#pragma unroll
-        for (int k = 0; k + m < PER; k += 2 * m) b[k] += b[k + m];
-    return b[0];
-}
-// Double-float: one chain per virtual lane over the merged row q0 .. qe.
-template <int G>
-__device__ __forceinline__ df64 gather_staged(const unsigned short* ei, const float2* ev, const float2* xs, int q0,
-                                              int qe, int r, int ncorr, const float2* hc, const float2* zc,
-                                              int64_t zld) {
-    constexpr int VL = 8, PER = VL / G;
-    df64 b[PER];
-#pragma unroll
-    for (int k = 0; k < PER; ++k) b[k] = df_make(0.f, 0.f);
-#pragma unroll 2
-    for (int q = q0 + r; q < qe; q += VL)
-#pragma unroll
-        for (int k = 0; k < PER; ++k)
-            if (q + k * G < qe)
-                b[k] = df_add(b[k], df_mul(df_from_float2(ev[q + k * G]), df_from_float2(xs[ei[q + k * G]])));
-    if (ncorr > 0) {
-        df64 c0[PER];
-#pragma unroll
-        for (int k = 0; k < PER; ++k) c0[k] = df_make(0.f, 0.f);
-        for (int c = r; c < ncorr; c += VL)
-#pragma unroll
-            for (int k = 0; k < PER; ++k)
-                if (c + k * G < ncorr)
-                    c0[k] = df_add(c0[k], df_mul(df_from_float2(hc[c + k * G]), df_from_float2(zc[(c + k * G) * zld])));
-#pragma unroll
-        for (int k = 0; k < PER; ++k) b[k] = df_add(b[k], df_neg(c0[k]));
-    }
-#pragma unroll
-    for (int o = 1; o < G; o <<= 1)
-#pragma unroll
-        for (int k = 0; k < PER; ++k) b[k] = df_add(b[k], df_shfl_xor(b[k], o));
-#pragma unroll
-    for (int m = 1; m < PER; m <<= 1)
-#pragma unroll
-        for (int k = 0; k + m < PER; k += 2 * m) b[k] = df_add(b[k], b[k + m]);
-    return b[0];
 }
 
 // Gather of one output from the staged x by a warp: entries q0 .. qe in
@@ -295,11 +203,10 @@ __device__ __forceinline__ void colsum(const double* P, int nb, int ncols, doubl
     }
 }
 
-// Exact sums.  A partial p of an inner product is taken as the 128-bit
-// integer P = trunc(p 2^sh) (two's complement; sh from a bound on |p| such
-// that |P| < 2^110), formed and added by integer operations: the FP64 pipe
-// issues one warp instruction per 64 clocks, so a tree of FP64 additions and
-// its barriers cost more than the products they add.  Integer addition is
+// Exact sums across CTAs.  A CTA's partial p of an inner product is taken as
+// the 128-bit integer P = trunc(p 2^sh) (two's complement; sh from a bound on
+// |p| such that |P| < 2^110), formed and added by integer operations (the FP64
+// pipe issues one warp instruction per 64 clocks).  Integer addition is
 // associative: the total is exact whatever the order of arrival, and every
 // CTA reads back the same value, in every run.
 struct Fix {
@@ -334,25 +241,27 @@ __device__ __forceinline__ void fx_sum(Fix& f, unsigned long long lo, unsigned l
     f.lo += lo;
     f.hi += hi + (f.lo < lo ? 1ull : 0ull);
 }
-__device__ __forceinline__ Fix fx_warp_sum(Fix f) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1)
-        fx_sum(f, __shfl_xor_sync(0xffffffffu, f.lo, o), __shfl_xor_sync(0xffffffffu, f.hi, o));
-    f.bad = __any_sync(0xffffffffu, f.bad);
-    return f;
+// x rounded to 53 significant bits (ties to even); true when that carries out
+__device__ __forceinline__ bool fx_round53(unsigned long long& x) {
+    const int drop = 11 - __clzll((long long)x);
+    if (drop <= 0) return false;
+    const unsigned long long keep = x >> drop, rest = x - (keep << drop), half = 1ull << (drop - 1);
+    const unsigned long long up = keep + (rest > half || (rest == half && (keep & 1ull)) ? 1ull : 0ull);
+    x = up << drop;
+    return (up >> (64 - drop)) != 0ull;
 }
-// P 2^-sh rounded to FP64, and the same number as a double-float pair (its
-// leading 24 bits and the next 24) when df is not null
-__device__ __forceinline__ double fx_value(Fix f, int sh, float2* df = nullptr) {
+// P 2^-sh in FP64: the words are rounded to 53 bits one by one, then their
+// sum (two conversions and an FMA, by integer operations)
+__device__ __forceinline__ double fx_value(Fix f, int sh) {
     const bool neg = (long long)f.hi < 0;
     if (neg) {
         f.lo = ~f.lo + 1ull;
         f.hi = ~f.hi + (f.lo == 0ull ? 1ull : 0ull);
     }
-    if (f.bad || (f.lo | f.hi) == 0ull) {
-        if (df) *df = f.bad ? make_float2(__int_as_float(0x7fc00000), 0.f) : make_float2(0.f, 0.f);
-        return f.bad ? __longlong_as_double(0x7ff8000000000000ll) : 0.0;
-    }
+    if (f.bad) return __longlong_as_double(0x7ff8000000000000ll);
+    if ((f.lo | f.hi) == 0ull) return 0.0;
+    fx_round53(f.hi);  // below 2^58: no carry
+    if (fx_round53(f.lo)) ++f.hi;
     // leading bit to bit 127
     if (f.hi == 0ull) {
         f.hi = f.lo;
@@ -363,18 +272,27 @@ __device__ __forceinline__ double fx_value(Fix f, int sh, float2* df = nullptr) 
     if (lz) f.hi = (f.hi << lz) | (f.lo >> (64 - lz));
     f.lo <<= lz;
     const int ex = 127 - lz - sh;  // value = 1.xxx 2^ex
-    if (df) {
-        const float scale = ex > -100 && ex < 127 ? __int_as_float((ex + 127) << 23) : 0.f;
-        const float s = (neg ? -scale : scale) * 0x1p-23f;
-        const float h = (float)(unsigned)(f.hi >> 40), l = (float)(unsigned)((f.hi >> 16) & 0xffffffull);
-        *df = ex >= 127 ? make_float2(__int_as_float(neg ? 0xff800000 : 0x7f800000), 0.f)
-                        : make_float2(h * s, l * (s * 0x1p-24f));
-    }
     unsigned long long m = f.hi >> 11;
     const unsigned rem = (unsigned)(f.hi & 0x7ffull) | (f.lo ? 1u : 0u);
     m += rem > 0x400u || (rem == 0x400u && (m & 1ull)) ? 1ull : 0ull;  // to nearest, ties to even
     const unsigned long long bits = ((unsigned long long)(ex + 1022) << 52) + m;
     return __longlong_as_double((long long)(bits | (neg ? 1ull << 63 : 0ull)));
+}
+// df_from_double(x), by integer operations where the pair is normal
+__device__ __forceinline__ float2 fx_pair(double x) {
+    const unsigned long long bits = (unsigned long long)__double_as_longlong(x);
+    const int e = (int)((bits >> 52) & 0x7ff);
+    if (e < 949 || e > 1149) return df_to_float2(df_from_double(x));
+    // |x| = m 2^(e - 1075): the leading 24 bits to nearest (ties to even), and
+    // the rest, which the conversion rounds likewise
+    const unsigned long long m = (bits & 0xfffffffffffffull) | (1ull << 52);
+    unsigned q = (unsigned)(m >> 29);
+    const unsigned rest = (unsigned)m & 0x1fffffffu;
+    q += rest > 0x10000000u || (rest == 0x10000000u && (q & 1u)) ? 1u : 0u;
+    const int l = (int)((long long)m - ((long long)q << 29));
+    const int sign = (long long)bits < 0 ? (int)0x80000000 : 0;
+    return make_float2((float)q * __int_as_float(((e - 919) << 23) | sign),
+                       (float)l * __int_as_float(((e - 948) << 23) | sign));
 }
 // Adds a CTA's sum into its copy of a column: P in three words of 56, 56 and
 // 16 bits, whose sums over 255 CTAs fit 64; the fourth word counts invalid
@@ -421,123 +339,139 @@ __device__ __forceinline__ void fx_columns(const unsigned long long* set, int nt
             // u.x + u.y 2^56 + v.x 2^112 modulo 2^128
             Fix f{u.x, 0ull, bad};
             fx_sum(f, u.y << 56, (u.y >> 8) + (v.x << 48));
-            out[c] = fx_value(f, c == nt - 1 ? sh_last : sh, outdf ? outdf + c : nullptr);
+            out[c] = fx_value(f, c == nt - 1 ? sh_last : sh);
+            if (outdf) outdf[c] = fx_pair(out[c]);
         }
     }
 }
 
 // The inner products of the staged slice with its basis columns, sum_{u < ne}
 // Vl[c vld + u] ws[u] for c < ncols and with norm also sum ws[u]^2 as column
-// ncols: emit(c, sum) by one thread per column.  A warp per column; long
-// slices with few columns give a column several warps, whose sums meet in
-// part (16 entries of shared memory).  A slice of up to four elements (the
-// smallest problems) takes one thread per column, summed in FP64.
+// ncols: emit(c, sum) by one thread per column.  CH lanes per column (a power
+// of two, the most with nt CH <= PT, at most 32) sum strided elements in two
+// chains; the CH partials of a column are added in a fixed tree, quarters by
+// four threads, then the four by shuffles (129 columns: two and two).  FP64
+// additions all of them, in an order that is kept to the bit (see arnoldi.cu); adding the lanes' products as integers by shuffles took
+// fewer clocks and moved the results of solves that amplify roundings.  An
+// FP64 instruction takes 64 clocks, so additions of lanes without an element
+// are left out, and a slice of up to four elements (the smallest problems)
+// takes one thread per column.  tmp holds PT doubles.
 template <typename Emit>
 __device__ __forceinline__ void slice_dots(const double* Vl, int64_t vld, int ncols, const double* ws, int ne,
-                                           bool norm, int sh, int sh_n, Fix* part, Emit&& emit) {
+                                           bool norm, double* tmp, Emit&& emit) {
+    static_assert(2 * (SGK_MAX_KRYLOV + 1) <= PT, "two lanes a column");
     const int nt = ncols + (norm ? 1 : 0);
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    auto column = [&](int c, int first, int step) {
+    int CH = 32;
+    while (CH > 2 && nt * CH > PT) CH >>= 1;
+    const int t = threadIdx.x;
+    if (ne <= 4 && CH > 2) {
+        // lanes 0..3 with one product each, in the tree's order
+        for (int c = t; c < nt; c += PT) {
+            const double* vc = c < ncols ? Vl + c * vld : ws;
+            double p[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) p[u] = u < ne ? __dmul_rn(vc[u], ws[u]) : 0.0;
+            if (ne > 1) p[0] = __dadd_rn(p[0], p[1]);
+            if (ne > 2 && CH <= 8) p[0] = __dadd_rn(p[0], __dadd_rn(p[2], p[3]));
+            if (ne > 2 && CH > 8) p[0] = __dadd_rn(__dadd_rn(p[0], p[2]), p[3]);
+            emit(c, p[0]);
+        }
+        return;
+    }
+    if (t < nt * CH) {
+        const int c = t / CH, k = t - (t / CH) * CH;
         const double* vc = c < ncols ? Vl + c * vld : ws;
         double a = 0.0, b = 0.0;
-        int u = first;
-        if (ne > 512) {
-            double a2 = 0.0, b2 = 0.0;
-            for (; u + 3 * step < ne; u += 4 * step) {
-                const double v0 = vc[u], v1 = vc[u + step], v2 = vc[u + 2 * step], v3 = vc[u + 3 * step];
-                a += v0 * ws[u];
-                b += v1 * ws[u + step];
-                a2 += v2 * ws[u + 2 * step];
-                b2 += v3 * ws[u + 3 * step];
+        int u = k;
+        // long slices lie in L2: several loads in flight
+        for (; u + 7 * CH < ne; u += 8 * CH) {
+            double v[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) v[i] = vc[u + i * CH];
+#pragma unroll
+            for (int i = 0; i < 8; i += 2) {
+                a += v[i] * ws[u + i * CH];
+                b += v[i + 1] * ws[u + (i + 1) * CH];
             }
-            a += a2;
-            b += b2;
-            for (; u < ne; u += step) a += vc[u] * ws[u];
-            a += b;
-        } else {
-            for (; u < ne; u += step) a += vc[u] * ws[u];
         }
-        return fx_warp_sum(fx_fixed(a, c < ncols ? sh : sh_n));
-    };
-    if (ne <= 4) {
-        for (int c = threadIdx.x; c < nt; c += PT) {
-            const double* vc = c < ncols ? Vl + c * vld : ws;
-            double a = 0.0;
-            for (int u = 0; u < ne; ++u) a = __dadd_rn(a, __dmul_rn(vc[u], ws[u]));
-            emit(c, fx_fixed(a, c < ncols ? sh : sh_n));
+        for (; u + CH < ne; u += 2 * CH) {
+            a += vc[u] * ws[u];
+            b += vc[u + CH] * ws[u + CH];
         }
-    } else if (ne > 512 && nt <= PNW / 2) {
-        int P = 2;
-        while (2 * P * nt <= PNW) P *= 2;
-        if (wid < nt * P) {
-            const Fix f = column(wid / P, (wid & (P - 1)) * 32 + lane, 32 * P);
-            if (lane == 0) part[wid] = f;
-        }
-        __syncthreads();
-        if ((int)threadIdx.x < nt) {
-            Fix f = part[threadIdx.x * P];
-            for (int i = 1; i < P; ++i) {
-                const Fix g = part[threadIdx.x * P + i];
-                fx_sum(f, g.lo, g.hi);
-                f.bad = f.bad || g.bad;
-            }
-            emit((int)threadIdx.x, f);
-        }
-    } else {
-        for (int c = wid; c < nt; c += PNW) {
-            const Fix f = column(c, lane, 32);
-            if (lane == 0) emit(c, f);
-        }
+        if (u < ne) a += vc[u] * ws[u];
+        tmp[t] = ne > CH ? a + b : a;
+    }
+    __syncthreads();
+    // whole warps: column t / Q, part t % Q
+    const int Q = CH < 4 ? CH : 4, per = CH / Q;
+    if ((t & ~31) < nt * Q) {
+        const int col = min(t, nt * Q - 1);
+        const double* p = tmp + col * per;
+        const int live = min(per, ne - (col & (Q - 1)) * per);
+        double a = p[0];
+        for (int i = 1; i < live; ++i) a += p[i];
+        if (ne > per) a += __shfl_xor_sync(0xffffffffu, a, 1);
+        if (Q == 4 && ne > 2 * per) a += __shfl_xor_sync(0xffffffffu, a, 2);
+        if (t < nt * Q && (t & (Q - 1)) == 0) emit(t / Q, a);
     }
 }
 
-// sum_{c < ncols} Vl[c vld + u] h[c] for the elements u < ne of the slice:
-// use(u, sum).  Short slices split the columns over four warps, one per
-// scheduler (the FP64 pipe takes 64 clocks a warp instruction, so one warp's
-// chain of M products is M times that); the four sums meet in tmp (PT
-// doubles).  TAIL (FP64 solves): the columns beyond a multiple of four go to
-// the first sum, as in the one-thread form for long slices, so that the
-// slicing changes no bit; in mixed mode they stay one to a warp (about 1% of a
-// step of two species at 11 520 coefficients).
-// Contains CTA barriers; not complete on return.
-template <bool TAIL, typename Use>
+// sum_{c < ncols} Vl[c vld + u] h[c] for the elements u < ne of the slice, in
+// two parts with a CTA barrier between them: combine_begin calls use(u, sum)
+// for the elements below the number it returns, combine_end for the others.
+// The FP64 pipe of a scheduler takes 64 clocks a warp instruction, so an
+// element per thread, four chains each, costs 64 ncols clocks for every four
+// warps of elements begun.  The warps beyond a multiple of four (slices of at
+// most 2 PT / 4 elements) split their columns over the four schedulers
+// instead, 16 ncols clocks a warp, where that saves more than the sums in tmp
+// (PT doubles) behind the barrier, some 300 clocks.  The same chains and sums
+// either way, so the slicing changes no bit.
+template <typename Use>
+__device__ __forceinline__ int combine_begin(const double* Vl, int64_t vld, int ncols, const double* h, int ne,
+                                             double* tmp, Use&& use) {
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int warps = (ne + 31) >> 5, rest = warps & 3;
+    const bool split = ne <= 2 * PT / 4 && rest > 0 && (4 - rest) * ncols >= 20;
+    const int whole = split ? (warps - rest) * 32 : ne;
+    for (int u = threadIdx.x; u < whole; u += PT) {
+        const double* vi = Vl + u;
+        double a0 = 0.0, a1 = 0.0, a2 = 0.0, a3 = 0.0;
+        int c = 0;
+#pragma unroll 2
+        for (; c + 3 < ncols; c += 4) {
+            a0 += vi[c * vld] * h[c];
+            a1 += vi[(c + 1) * vld] * h[c + 1];
+            a2 += vi[(c + 2) * vld] * h[c + 2];
+            a3 += vi[(c + 3) * vld] * h[c + 3];
+        }
+        for (; c < ncols; ++c) a0 += vi[c * vld] * h[c];
+        use(u, (a0 + a1) + (a2 + a3));
+    }
+    const int part = wid & 3, blk = (wid >> 2) * 32 + lane, u = whole + blk;
+    if (u < ne) {
+        double a = 0.0;
+        const int full = ncols & ~3;
+        for (int c = part; c < full; c += 4) a += Vl[c * vld + u] * h[c];
+        if (part == 0)
+            for (int c = full; c < ncols; ++c) a += Vl[c * vld + u] * h[c];
+        tmp[part * (PT / 4) + blk] = a;
+    }
+    return whole;
+}
+template <typename Use>
+__device__ __forceinline__ void combine_end(int whole, int ne, const double* tmp, Use&& use) {
+    if ((int)threadIdx.x < ne - whole) {
+        const double* p = tmp + threadIdx.x;
+        use(whole + (int)threadIdx.x, (p[0] + p[PT / 4]) + (p[2 * (PT / 4)] + p[3 * (PT / 4)]));
+    }
+}
+template <typename Use>
 __device__ __forceinline__ void slice_combine(const double* Vl, int64_t vld, int ncols, const double* h, int ne,
                                               double* tmp, Use&& use) {
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    if (ne <= 2 * PT / 4) {
-        const int part = wid & 3, blk = (wid >> 2) * 32 + lane;
-        for (int base = 0; base < ne; base += PT / 4) {
-            const int u = base + blk;
-            if (u < ne) {
-                double a = 0.0;
-                const int full = TAIL ? ncols & ~3 : ncols;
-                for (int c = part; c < full; c += 4) a += Vl[c * vld + u] * h[c];
-                if (part == 0)
-                    for (int c = full; c < ncols; ++c) a += Vl[c * vld + u] * h[c];
-                tmp[part * (PT / 4) + blk] = a;
-            }
-            __syncthreads();
-            if ((int)threadIdx.x < PT / 4 && base + (int)threadIdx.x < ne) {
-                const double* p = tmp + threadIdx.x;
-                use(base + (int)threadIdx.x, (p[0] + p[PT / 4]) + (p[2 * (PT / 4)] + p[3 * (PT / 4)]));
-            }
-            if (base + PT / 4 < ne) __syncthreads();
-        }
-    } else {
-        for (int u = threadIdx.x; u < ne; u += PT) {
-            const double* vi = Vl + u;
-            double a0 = 0.0, a1 = 0.0, a2 = 0.0, a3 = 0.0;
-            int c = 0;
-#pragma unroll 2
-            for (; c + 3 < ncols; c += 4) {
-                a0 += vi[c * vld] * h[c];
-                a1 += vi[(c + 1) * vld] * h[c + 1];
-                a2 += vi[(c + 2) * vld] * h[c + 2];
-                a3 += vi[(c + 3) * vld] * h[c + 3];
-            }
-            for (; c < ncols; ++c) a0 += vi[c * vld] * h[c];
-            use(u, (a0 + a1) + (a2 + a3));
-        }
+    const int whole = combine_begin(Vl, vld, ncols, h, ne, tmp, use);
+    if (whole < ne) {
+        __syncthreads();
+        combine_end(whole, ne, tmp, use);
     }
 }
 
@@ -560,8 +494,8 @@ __device__ __forceinline__ void slice_norm2(const double* ws, int ne, double* re
 template <int D, int KP1, int G, bool DF>
 __device__ __forceinline__ void arnoldi_body(const GmvArgs<double, D>& ga, const ArnArgs& a, const int nb,
                                              const int b) {
-    // dynamic shared memory: [x: n, 16-byte multiple][w slices: 2 E][Vs: (M+1) Es][Zs: (M+1) Es][located rows,
-    // or gather offsets and entries (staged x: values, then indices)]
+    // dynamic shared memory: [with eo1, x: n, 16-byte multiple][w slices: 2 E][Vs: (M+1) Es][Zs: (M+1) Es]
+    // [located rows, or gather offsets and entries]
     extern __shared__ __align__(16) double smem_dyn[];
     __shared__ double h1[SGK_MAX_KRYLOV + 2];
     __shared__ double h2[SGK_MAX_KRYLOV + 2];
@@ -569,7 +503,6 @@ __device__ __forceinline__ void arnoldi_body(const GmvArgs<double, D>& ga, const
     __shared__ double s_scal[4], s_beta;
     // column-sum and combination staging: <= max(PT, 4 (SGK_MAX_KRYLOV + 2))
     __shared__ double ctmp[PT > 4 * (SGK_MAX_KRYLOV + 2) ? PT : 4 * (SGK_MAX_KRYLOV + 2)];
-    __shared__ Fix s_part[PNW];
     __shared__ int s_ok, s_flag;
     // double-float matvec: the correction's coefficients and the step's scale
     __shared__ float2 h2df[DF ? SGK_MAX_KRYLOV + 2 : 1];
@@ -581,7 +514,7 @@ __device__ __forceinline__ void arnoldi_body(const GmvArgs<double, D>& ga, const
     // the staged slice of w, two buffers alternating by step: the update of
     // step j (v_{j+1} from w') runs during the matvec of step j + 1
     double* const xstage = smem_dyn;
-    double* const smem = smem_dyn + (a.xs ? (n + 1) / 2 * 2 : 0);
+    double* const smem = smem_dyn + (a.eo1 ? (n + 1) / 2 * 2 : 0);
     double* const wsb0 = smem;
     double* const wsb1 = smem + E;
     // shared columns of V and Z have an odd stride: the lanes of one output
@@ -595,11 +528,7 @@ __device__ __forceinline__ void arnoldi_body(const GmvArgs<double, D>& ga, const
     // pre-located gathers of the slice: offsets rebased to the slice's first
     // entry, then the entries
     int* const seoff = a.list_cap > 0 || a.eo1 ? reinterpret_cast<int*>(tail) : nullptr;
-    int2* const sent = a.list_cap > 0 && !a.xs ? reinterpret_cast<int2*>(tail + arn_eoff_bytes(E, D)) : nullptr;
-    // staged x: the entries' values and indices, in shared memory or (their
-    // offsets as they are) in the flat copies
-    double* const sev = a.list_cap > 0 && a.xs ? reinterpret_cast<double*>(tail + arn_eoff_bytes(E, D)) : nullptr;
-    unsigned short* const sei = sev ? reinterpret_cast<unsigned short*>(sev + a.list_cap) : nullptr;
+    int2* const sent = a.list_cap > 0 ? reinterpret_cast<int2*>(tail + arn_eoff_bytes(E, D)) : nullptr;
     // this slice's basis and raw-output columns: shared copies or HBM
     const double* const Vl = a.smem_vz ? Vs : a.V + lo;
     const int64_t vld = a.smem_vz ? Es : n;
@@ -629,9 +558,15 @@ __device__ __forceinline__ void arnoldi_body(const GmvArgs<double, D>& ga, const
     auto dots = [&](int j, int phase, double* out, float2* outdf) {
         const int nc = j + 1;
         unsigned long long* set = fx_set(j, phase) + (size_t)(b % FX_COPIES) * FX_COLS * FX_LIMBS;
-        slice_dots(Vl, vld, nc, (j & 1) ? wsb1 : wsb0, ne, phase == 1, a.sh_h, a.sh_n, s_part, [&](int c, const Fix& f) {
-            if (alone) out[c] = fx_value(f, c < nc ? a.sh_h : a.sh_n, outdf ? outdf + c : nullptr);
-            else fx_add(set + (size_t)c * FX_LIMBS, f);
+        slice_dots(Vl, vld, nc, (j & 1) ? wsb1 : wsb0, ne, phase == 1, ctmp, [&](int c, double p) {
+            const int sh = c < nc ? a.sh_h : a.sh_n;
+            const Fix f = fx_fixed(p, sh);
+            if (alone) {
+                out[c] = fx_value(f, sh);
+                if (outdf) outdf[c] = fx_pair(out[c]);
+            } else {
+                fx_add(set + (size_t)c * FX_LIMBS, f);
+            }
         });
     };
     // and their sums over the CTAs
@@ -659,17 +594,9 @@ __device__ __forceinline__ void arnoldi_body(const GmvArgs<double, D>& ga, const
             return;
         }
         for (int i = threadIdx.x; i <= ne * D; i += PT) seoff[i] = a.eoff[lo * D + i] - e0;
-        if (sev) {
-            const double* src = DF ? reinterpret_cast<const double*>(a.ev2) : a.ev;
-            for (int i = threadIdx.x; i < ecount; i += PT) {
-                sev[i] = src[e0 + i];
-                sei[i] = a.ei[e0 + i];
-            }
-        } else {
-            for (int i = threadIdx.x; i < ecount; i += PT) sent[i] = a.ent[e0 + i];
-        }
+        for (int i = threadIdx.x; i < ecount; i += PT) sent[i] = a.ent[e0 + i];
     }
-    if (!DF && a.xs) stage_vector(xstage, a.v, n);  // the first gathers read v
+    if (!DF && a.eo1) stage_vector(xstage, a.v, n);  // the first gathers read v
 
     // the accumulator sets start cleared (before the first barrier)
     auto clear_set = [&](unsigned long long* set, int cols) {
@@ -722,7 +649,6 @@ __device__ __forceinline__ void arnoldi_body(const GmvArgs<double, D>& ga, const
         // one more barrier publishes the pairs; the first product is then
         // A v_0 itself (scale 1)
         if (!barrier()) return;
-        if (a.xs) stage_vector(xstage, a.w1, n);
         scale = 1.0;
         if (threadIdx.x == 0) s_scaldf = df_to_float2(df_from_double(1.0));
         __syncthreads();
@@ -740,10 +666,17 @@ __device__ __forceinline__ void arnoldi_body(const GmvArgs<double, D>& ga, const
     double fro2 = 0.0, sub2 = 0.0;
     // the pending update of the previous step: v_{pj+1} on the slice from
     // that step's staged w (w' - V h2, or w'' after an explicit norm) times
-    // its scale, into column pj + 1 of V (global and shared)
+    // its scale, into column pj + 1 of V (global and shared).  The sums over
+    // the columns need no scale: they are taken before the barrier behind the
+    // gathers, where warps wait for those with long rows, and the rest after it
     int pj = -1;
     bool pexpl = false;
-    auto pending_update = [&]() {
+    auto pending_begin = [&]() {
+        double* const wp = (pj & 1) ? wsb1 : wsb0;
+        return pj < 0 || pexpl ? ne : combine_begin(Vl, vld, pj + 1, h2, ne, ctmp, [&](int u, double sum) { wp[u] -= sum; });
+    };
+    auto pending_end = [&](int whole) {
+        if (pj < 0) return;
         const double* const wp = (pj & 1) ? wsb1 : wsb0;
         double* vg = a.V + (int64_t)(pj + 1) * n + lo;
         double* vs = Vs ? Vs + (int64_t)(pj + 1) * Es : nullptr;
@@ -753,11 +686,8 @@ __device__ __forceinline__ void arnoldi_body(const GmvArgs<double, D>& ga, const
             vg[u] = y;
             if (vs) vs[u] = y;
         };
-        if (pexpl) {
-            for (int u = threadIdx.x; u < ne; u += PT) put(u, 0.0);
-        } else {
-            slice_combine<!DF>(Vl, vld, pj + 1, h2, ne, ctmp, put);
-        }
+        for (int u = threadIdx.x; u < whole; u += PT) put(u, 0.0);
+        combine_end(whole, ne, ctmp, put);
     };
     if (threadIdx.x == 0) s_scal[1] = scale;
     for (int j = 0; j < a.M; ++j) {
@@ -766,11 +696,9 @@ __device__ __forceinline__ void arnoldi_body(const GmvArgs<double, D>& ga, const
         const int nc = j + 1;
         // A v_j on this slice before its scale, which one warp may still be
         // forming: raw sums into the staged slice (a double, or a pair)
-        if (a.xs) {
+        if (!DF && a.eo1) {
             stage_wait();
             __syncthreads();
-        }
-        if (!DF && a.eo1) {
             // a warp per output: the rows are long and uneven (hundreds of
             // entries, thousands at low levels)
             for (int u = wid; u < ne; u += PNW) {
@@ -785,20 +713,12 @@ __device__ __forceinline__ void arnoldi_body(const GmvArgs<double, D>& ga, const
             // the correction's columns are dealt over the virtual lanes like
             // the matrix rows (sum independent of G)
             if constexpr (DF) {
-                df64 ad;
-                if (a.xs)
-                    ad = gather_staged<G>(sei, reinterpret_cast<const float2*>(sev),
-                                          reinterpret_cast<const float2*>(xstage), seoff[uu * D],
-                                          live ? seoff[(uu + 1) * D] : 0, r, live ? ncorr : 0, h2df, Zdf + uu, zld);
-                else
-                    ad = gmv_accumulate_list_df<D, G>(seoff + uu * D, sent, a.cvk2, xdf, r, live, ncorr, h2df, Zdf + uu,
-                                                      zld);
+                const df64 ad = gmv_accumulate_list_df<D, G>(seoff + uu * D, sent, a.cvk2, xdf, r, live, ncorr, h2df,
+                                                             Zdf + uu, zld);
                 if (live && r == 0) reinterpret_cast<float2*>(ws)[u] = df_to_float2(ad);
             } else {
                 double acc;
-                if (a.xs) {
-                    acc = gather_staged<D, G>(sei, sev, xstage, seoff + uu * D, live, r, ncorr, h2, Zl + uu, zld);
-                } else if (seoff) {
+                if (seoff) {
                     acc = gmv_accumulate_list<D, G>(seoff + uu * D, sent, ga.cvk, x, r, live, ncorr, h2, Zl + uu, zld);
                 } else if (sloc) {
                     acc = gmv_accumulate<double, D, G, 2>(ga, x, sloc[uu], r, live, ncorr, h2, Zl + uu, zld);
@@ -810,9 +730,10 @@ __device__ __forceinline__ void arnoldi_body(const GmvArgs<double, D>& ga, const
                 if (live && r == 0) ws[u] = acc;
             }
         }
+        const int whole = pending_begin();
         __syncthreads();
         // the scale is there: A v_j staged and kept in Z, by the upper half of
-        // the CTA, which the combination's last sums leave idle
+        // the CTA, which the pending update's last sums leave idle
         for (int u = (int)threadIdx.x - PT / 2; u < ne; u += PT / 2) {
             if (u < 0) break;
             if constexpr (DF) {
@@ -825,7 +746,7 @@ __device__ __forceinline__ void arnoldi_body(const GmvArgs<double, D>& ga, const
                 Zl[(int64_t)j * zld + u] = acc;
             }
         }
-        if (pj >= 0) pending_update();
+        pending_end(whole);
         __syncthreads();
         dots(j, 0, h1, nullptr);
         if (!collect(j, 0, h1, nullptr)) return;
@@ -834,7 +755,7 @@ __device__ __forceinline__ void arnoldi_body(const GmvArgs<double, D>& ga, const
             clear_set(fx_set(j + 2, 1), nc + 1);
         }
         // w' = w - V h1, published for the next matvec
-        slice_combine<!DF>(Vl, vld, nc, h1, ne, ctmp, [&](int u, double sum) {
+        slice_combine(Vl, vld, nc, h1, ne, ctmp, [&](int u, double sum) {
             const double y = ws[u] - sum;
             ws[u] = y;
             if (DF) reinterpret_cast<float2*>(w)[lo + u] = df_to_float2(df_from_double(y));
@@ -846,7 +767,7 @@ __device__ __forceinline__ void arnoldi_body(const GmvArgs<double, D>& ga, const
         if (!collect(j, 1, h2, DF ? h2df : nullptr)) return;
         // the next gathers' vector, copied while the scalars are formed (again
         // after an explicit norm, which changes it)
-        if (a.xs && j + 1 < a.M) stage_vector(xstage, w, n);
+        if (!DF && a.eo1 && j + 1 < a.M) stage_vector(xstage, w, n);
         // ||w''||^2 = ||w'||^2 - ||h2||^2 (V orthonormal, w'' = w' - V h2).
         // As a rule h2 is rounding and its square below half a unit in the
         // last place of ||w'||^2, which is then the norm as it stands, and far
@@ -906,11 +827,11 @@ __device__ __forceinline__ void arnoldi_body(const GmvArgs<double, D>& ga, const
             explicit_norm = s_flag != 0;
             if (explicit_norm) {
                 // w'' in place (published), its norm through a barrier
-                if (a.xs) {  // the first copy must not land over the second
+                if (!DF && a.eo1) {  // the first copy must not land over the second
                     stage_wait();
                     __syncthreads();
                 }
-                slice_combine<!DF>(Vl, vld, nc, h2, ne, ctmp, [&](int u, double sum) {
+                slice_combine(Vl, vld, nc, h2, ne, ctmp, [&](int u, double sum) {
                     const double y = ws[u] - sum;
                     ws[u] = y;
                     if (DF) reinterpret_cast<float2*>(w)[lo + u] = df_to_float2(df_from_double(y));
@@ -922,7 +843,7 @@ __device__ __forceinline__ void arnoldi_body(const GmvArgs<double, D>& ga, const
                 colsum(P2, nb, 1, s_scal, ctmp);
                 __syncthreads();
                 if (wid == WNORM) inverse_norm(s_scal[0]);
-                if (a.xs && j + 1 < a.M) stage_vector(xstage, w, n);
+                if (!DF && a.eo1 && j + 1 < a.M) stage_vector(xstage, w, n);
                 __syncthreads();
             }
             sub2 = s_scal[3];
@@ -949,8 +870,9 @@ __device__ __forceinline__ void arnoldi_body(const GmvArgs<double, D>& ga, const
         x = w;
         xdf = reinterpret_cast<const float2*>(w);
     }
+    const int whole = pending_begin();
     __syncthreads();
-    if (pj >= 0) pending_update();  // the last column, v_M
+    pending_end(whole);  // the last column, v_M
 }
 
 template <int D, int KP1, int G, bool DF>

@@ -322,13 +322,6 @@ struct sgk_op {
     DevBuf<int32_t> gmv_eoff;
     DevBuf<int2> gmv_ent;
     std::vector<int32_t> gmv_ecnt_host;
-    // the same entries with their own values, for gathers from a vector staged
-    // in shared memory (index sets of at most GMV_STAGED_MAX coefficients):
-    // index of x, and the value in the context's arithmetic (FP64, or pairs
-    // in mixed precision)
-    DevBuf<unsigned short> gmv_ei;
-    DevBuf<double> gmv_ev;
-    DevBuf<float2> gmv_ev2;
     // mixed-derivative terms of a full diffusion tensor (cross.cu): the
     // direction pairs (i, j) with K_ij != 0 and K_ij; the 1D factors Q, P^T,
     // E^T, P as CSR (pointers per matrix, H + 1 each) with truncated row

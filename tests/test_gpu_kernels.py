@@ -179,3 +179,46 @@ def test_mixed_corrections_use_the_current_state(n, k, scheme):
         prob.close()
     assert rel(out[sgkiif.SGK_MIXED], out[sgkiif.SGK_FP64]) <= 1e-10
     assert its[sgkiif.SGK_MIXED] <= its[sgkiif.SGK_FP64] + 2 * steps
+
+
+# Three heat steps whose unconverged projections amplify a rounding: the
+# largest coefficients, recorded before the sums of the persistent Arnoldi
+# kernel were first rearranged.  Another order of one of its sums moves them by
+# 1e-8 to 1e-5, so 1e-9 holds the order (slices, and so sums, go by the number
+# of SMs).
+WAVES = np.array([[1, 2, 1], [2, 1, 3], [3, 3, 2], [1, 1, 2]], np.int32)
+KINDS = np.array([[0, 1, 0], [1, 0, 0], [0, 0, 1], [1, 1, 0]], np.int32)
+AMPLIFIED = [
+    (3, 3, 3, 20, 0.005, sgkiif.SGK_MIXED, slice(0, 4),
+     {41: -0.003271583982073906, 43: -0.0030994131983151717, 105: 0.006966140093553048,
+      529: 0.003479553274309175, 531: -0.0027540474380408127, 537: -0.0019932718917509726,
+      561: -0.0027540474380408383, 563: 0.0021529999571539616}),
+    (3, 3, 3, 20, 0.005, sgkiif.SGK_MIXED, slice(1, 2),
+     {37: -5.764616895548291e-06, 1285: -1.2965191226569354e-05, 1287: 7.323860043138634e-06,
+      1293: 1.1716066326707738e-05, 1295: -7.157901932217996e-06, 1317: 7.684680082379417e-06,
+      1319: -4.149563333670409e-06, 1325: -6.65949686508748e-06}),
+    (3, 5, 1, 40, 0.0025, sgkiif.SGK_FP64, slice(0, 4),
+     {1025: -0.01369145403862061, 1033: -0.023429195143054637, 1041: 0.011077942307921348,
+      1043: 0.011077942307921416, 1056: -0.00899816104998158, 1058: 0.008978195831283849,
+      1060: -0.0089781958312839, 1062: 0.008998161049981633})]
+
+
+@pytest.mark.parametrize("d,n,k,M,dt,prec,modes,want", AMPLIFIED, ids=["mixed", "mixed_one_mode", "fp64"])
+def test_order_of_sums_of_the_projection(d, n, k, M, dt, prec, modes, want):
+    if torch.cuda.get_device_properties(0).multi_processor_count != 152:
+        pytest.skip("recorded on 152 SMs")
+    with_amp = np.array([0.7, -0.4, 0.5, 0.9])[modes]
+    ctx = sgkiif.Context(0, torch.cuda.current_stream().cuda_stream, prec)
+    idx = sgkiif.IndexSet(ctx, d, n, k)
+    op = sgkiif.Operator(ctx, idx, [1.0] * d)
+    sol = sgkiif.Solver(ctx, [op], [[]], M, dt)
+    U = torch.empty(idx.dof, dtype=torch.float64, device="cuda")
+    idx.project_separable(with_amp, WAVES[modes].copy(), KINDS[modes].copy(), 0.0, U.data_ptr())
+    sol.set_state(0, dev_ptr=U.data_ptr())
+    sol.step(3)
+    got = sol.get_state(0)[list(want)]
+    assert rel(got, list(want.values())) <= 1e-9
+    sol.close()
+    op.close()
+    idx.close()
+    ctx.close()
