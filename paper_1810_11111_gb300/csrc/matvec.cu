@@ -8,12 +8,13 @@
 // tree), so results are deterministic.
 #include <algorithm>
 #include <cmath>
+#include <type_traits>
 
 #include "sgk_gmv.h"
 
 namespace {
 
-template <typename T, int D, int KP1, int G, typename IX>
+template <typename T, int D, int KP1, int G, bool SIDE, typename IX>
 __global__ void __launch_bounds__(256) gmv_kernel(const GmvArgs<T, D> a, const T* __restrict__ x,
                                                   T* __restrict__ y) {
     // G consecutive lanes share one output coefficient (more loads in flight
@@ -28,8 +29,29 @@ __global__ void __launch_bounds__(256) gmv_kernel(const GmvArgs<T, D> a, const T
         const bool live = g < a.n;
         GmvLoc<D, IX> L;
         if (live) gmv_locate<T, D, KP1>(a, g, L);
-        const T acc = gmv_accumulate<T, D, G, 0>(a, x, L, r, live);
+        const T acc = gmv_accumulate<T, D, G, 0, SIDE>(a, x, L, r, live);
         if (live && r == 0) y[g] = acc;
+    }
+}
+
+// How a thread goes through its virtual lanes (the sums are the same, see
+// gmv_accumulate), and the index width, each where it was the faster one.
+// Short rows (d > 2) go side by side, more loads in flight, in FP32 and with
+// one virtual lane per thread (FP32, d = 4, level 6, degree 2: 13.9 against
+// 17.9 us; FP64, d = 3, level 4, degree 3: 5.6 and 6.2); two or four FP64
+// lanes one after the other, which keeps more warps on an SM (d = 3, level 7,
+// degree 3: 26.9 and 31.8 us).  The long rows of d = 2 go one after the other
+// with 64-bit indices (FP64, level 8, degree 3: 9.7 us, 10.3 with 32-bit ones,
+// 10.5 side by side), short FP32 vectors with 32-bit ones (7.2, 8.2, 8.2).
+template <typename T, int D, int KP1, int G>
+void gmv_launch(const GmvArgs<T, D>& a, int grid, int threads, cudaStream_t st, const T* x, T* y) {
+    if constexpr (G == 1) {
+        if (a.n < (int64_t(1) << 31)) gmv_kernel<T, D, KP1, 1, true, int><<<grid, threads, 0, st>>>(a, x, y);
+        else gmv_kernel<T, D, KP1, 1, true, int64_t><<<grid, threads, 0, st>>>(a, x, y);
+    } else {
+        constexpr bool side = D > 2 && (sizeof(T) == 4 || G == 8);
+        constexpr bool wide = D == 2 && (sizeof(T) == 8 || G < 8);
+        gmv_kernel<T, D, KP1, G, side, std::conditional_t<wide, int64_t, int>><<<grid, threads, 0, st>>>(a, x, y);
     }
 }
 
@@ -46,16 +68,12 @@ void gmv_dispatch(const sgk_op* op, const T* x, T* y) {
     const int64_t blocks = (idx->dof * G + threads - 1) / threads;
     const int grid = (int)std::min<int64_t>(blocks, (int64_t)ctx->num_sms * 8);
     KTimer kt(ctx, KC_MATVEC);
-#define SGK_GMV(K, GG) gmv_kernel<T, D, K, GG, int><<<grid, threads, 0, ctx->stream>>>(a, x, y)
-#define SGK_GMV_K(K)                         \
-    switch (G) {                             \
-        case 1:                              \
-            if (idx->dof < (int64_t(1) << 31)) SGK_GMV(K, 1);                                             \
-            else gmv_kernel<T, D, K, 1, int64_t><<<grid, threads, 0, ctx->stream>>>(a, x, y);              \
-            break;                           \
-        case 2: SGK_GMV(K, 2); break;        \
-        case 4: SGK_GMV(K, 4); break;        \
-        default: SGK_GMV(K, 8); break;       \
+#define SGK_GMV_K(K)                                                                    \
+    switch (G) {                                                                        \
+        case 1: gmv_launch<T, D, K, 1>(a, grid, threads, ctx->stream, x, y); break;     \
+        case 2: gmv_launch<T, D, K, 2>(a, grid, threads, ctx->stream, x, y); break;     \
+        case 4: gmv_launch<T, D, K, 4>(a, grid, threads, ctx->stream, x, y); break;     \
+        default: gmv_launch<T, D, K, 8>(a, grid, threads, ctx->stream, x, y); break;    \
     }
     switch (idx->k + 1) {
         case 2: SGK_GMV_K(2) break;
@@ -64,7 +82,6 @@ void gmv_dispatch(const sgk_op* op, const T* x, T* y) {
         default: throw SgkError{SGK_EUNSUPPORTED, "matvec: degree must be 1..3"};
     }
 #undef SGK_GMV_K
-#undef SGK_GMV
     check_launch("gmv_kernel");
     count_launch(ctx);
 }

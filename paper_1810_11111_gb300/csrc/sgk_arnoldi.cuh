@@ -721,11 +721,11 @@ __device__ __forceinline__ void arnoldi_body(const GmvArgs<double, D>& ga, const
                 if (seoff) {
                     acc = gmv_accumulate_list<D, G>(seoff + uu * D, sent, ga.cvk, x, r, live, ncorr, h2, Zl + uu, zld);
                 } else if (sloc) {
-                    acc = gmv_accumulate<double, D, G, 2>(ga, x, sloc[uu], r, live, ncorr, h2, Zl + uu, zld);
+                    acc = gmv_accumulate<double, D, G, 2, true>(ga, x, sloc[uu], r, live, ncorr, h2, Zl + uu, zld);
                 } else {
                     GmvLoc<D, int> l1;
                     if (live) gmv_locate<double, D, KP1>(ga, lo + u, l1);
-                    acc = gmv_accumulate<double, D, G, 2>(ga, x, l1, r, live, ncorr, h2, Zl + uu, zld);
+                    acc = gmv_accumulate<double, D, G, 2, true>(ga, x, l1, r, live, ncorr, h2, Zl + uu, zld);
                 }
                 if (live && r == 0) ws[u] = acc;
             }

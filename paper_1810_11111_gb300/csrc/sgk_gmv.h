@@ -102,67 +102,99 @@ __device__ __forceinline__ void gmv_locate(const GmvArgs<T, D>& a, int64_t g, Gm
 // correction sum_c h_c z_c whose columns are dealt the same way, and the 8
 // virtual sums are added in one fixed binary tree -- physical lanes hold 8/G
 // virtual lanes, the lower tree levels are shuffles, the upper ones local.  A
-// thread goes through its virtual lanes side by side, 16 / G loads in flight.
-// With one lane per output (long vectors) the row is taken in order by eight
-// chains.  The result is returned in every lane of the group.  LD selects the
-// loads of x: 0 plain (read-only for the kernel), 1 L2 only, 2 cached in L1
-// through the coherent path (for vectors written by other CTAs of the same
-// persistent kernel and published by a barrier whose acquire made L1
-// current).
-template <typename T, int D, int G, int LD, typename IX>
+// thread goes through its virtual lanes side by side, 16 / G loads in flight
+// (SIDE), or one after the other; the sum is the same.  With one lane per
+// output (long vectors) the row is taken in order by eight chains.  The result
+// is returned in every lane of the group.  LD selects the loads of x: 0 plain
+// (read-only for the kernel), 1 L2 only, 2 cached in L1 through the coherent
+// path (for vectors written by other CTAs of the same persistent kernel and
+// published by a barrier whose acquire made L1 current).
+template <typename T, int D, int G, int LD, bool SIDE, typename IX>
 __device__ __forceinline__ T gmv_accumulate(const GmvArgs<T, D>& a, const T* __restrict__ x, const GmvLoc<D, IX>& L,
                                             int r, bool live, int ncorr = 0, const T* hc = nullptr,
                                             const T* zc = nullptr, int64_t zld = 0) {
-    constexpr int VL = 8, PER = VL / G, CH = G == 1 ? 1 : 2;  // chains of a virtual lane
-    T s[CH][PER];
-#pragma unroll
-    for (int k = 0; k < PER; ++k)
-#pragma unroll
-        for (int h = 0; h < CH; ++h) s[h][k] = T(0);
-    if (live) {
-#pragma unroll
-        for (int i = 0; i < D; ++i) {
-            const int64_t* __restrict__ base = a.cb + L.cbrow[i];
-            const T* __restrict__ cv = a.cvk + i * a.nnz;
-            const IX oI = L.oI[i], I = L.I[i];
-            const T* __restrict__ xi = x + L.in[i];
-            auto ld = [&](int pk) {
-                const int lb = pk >> 16, p = pk & 0xffff;
-                const T* px = xi + ((IX)base[lb] + (lb ? (oI << (lb - 1)) : oI) + (IX)p * I);
-                if constexpr (LD == 1) return __ldcg(px);
-                else if constexpr (LD == 2) return __ldca(px);
-                else return *px;
-            };
-            const int qe = L.qe[i];
-            int q = L.q0[i] + r;
-            // whole rounds (one entry for every chain) without tests, then the rest
-            for (; q - r + CH * VL <= qe; q += CH * VL) {
-                T xv[CH][PER];
-#pragma unroll
-                for (int h = 0; h < CH; ++h)
-#pragma unroll
-                    for (int k = 0; k < PER; ++k) xv[h][k] = ld(a.ce[q + h * VL + k * G]);
-#pragma unroll
-                for (int h = 0; h < CH; ++h)
-#pragma unroll
-                    for (int k = 0; k < PER; ++k) s[h][k] += cv[q + h * VL + k * G] * xv[h][k];
-            }
-#pragma unroll
-            for (int h = 0; h < CH; ++h)
-#pragma unroll
-                for (int k = 0; k < PER; ++k)
-                    if (q + h * VL + k * G < qe) s[h][k] += cv[q + h * VL + k * G] * ld(a.ce[q + h * VL + k * G]);
-        }
-    }
+    constexpr int VL = 8, PER = VL / G;
+    static_assert(SIDE || G > 1, "one lane per output: side by side");
     T b[PER];
 #pragma unroll
-    for (int k = 0; k < PER; ++k) {
-        b[k] = CH == 2 ? s[0][k] + s[CH - 1][k] : s[0][k];
-        if (live && ncorr > 0) {
-            T c0 = T(0);
-            for (int c = r + k * G; c < ncorr; c += VL) c0 += hc[c] * zc[c * zld];
-            b[k] -= c0;
+    for (int k = 0; k < PER; ++k) b[k] = T(0);
+    if (live) {
+        // x at a packed entry of a row
+        auto load = [&](const int64_t* __restrict__ base, const T* __restrict__ xi, IX oI, IX I, IX in, int pk) {
+            const int lb = pk >> 16, p = pk & 0xffff;
+            const T* px = xi + ((IX)base[lb] + (lb ? (oI << (lb - 1)) : oI) + (IX)p * I + in);
+            if constexpr (LD == 1) return __ldcg(px);
+            else if constexpr (LD == 2) return __ldca(px);
+            else return *px;
+        };
+        if constexpr (SIDE) {
+            constexpr int CH = G == 1 ? 1 : 2;  // chains of a virtual lane
+            T s[CH][PER];
+#pragma unroll
+            for (int k = 0; k < PER; ++k)
+#pragma unroll
+                for (int h = 0; h < CH; ++h) s[h][k] = T(0);
+#pragma unroll
+            for (int i = 0; i < D; ++i) {
+                const int64_t* __restrict__ base = a.cb + L.cbrow[i];
+                const T* __restrict__ cv = a.cvk + i * a.nnz;
+                const IX oI = L.oI[i], I = L.I[i];
+                const T* __restrict__ xi = x + L.in[i];
+                const int qe = L.qe[i];
+                int q = L.q0[i] + r;
+                // whole rounds (one entry for every chain) without tests, then the rest
+                for (; q - r + CH * VL <= qe; q += CH * VL) {
+                    T xv[CH][PER];
+#pragma unroll
+                    for (int h = 0; h < CH; ++h)
+#pragma unroll
+                        for (int k = 0; k < PER; ++k) xv[h][k] = load(base, xi, oI, I, 0, a.ce[q + h * VL + k * G]);
+#pragma unroll
+                    for (int h = 0; h < CH; ++h)
+#pragma unroll
+                        for (int k = 0; k < PER; ++k) s[h][k] += cv[q + h * VL + k * G] * xv[h][k];
+                }
+#pragma unroll
+                for (int h = 0; h < CH; ++h)
+#pragma unroll
+                    for (int k = 0; k < PER; ++k)
+                        if (q + h * VL + k * G < qe)
+                            s[h][k] += cv[q + h * VL + k * G] * load(base, xi, oI, I, 0, a.ce[q + h * VL + k * G]);
+            }
+#pragma unroll
+            for (int k = 0; k < PER; ++k) b[k] = CH == 2 ? s[0][k] + s[CH - 1][k] : s[0][k];
+        } else {
+#pragma unroll
+            for (int k = 0; k < PER; ++k) {
+                T s0 = T(0), s1 = T(0);
+#pragma unroll
+                for (int i = 0; i < D; ++i) {
+                    const int64_t* __restrict__ base = a.cb + L.cbrow[i];
+                    const T* __restrict__ cv = a.cvk + i * a.nnz;
+                    const IX oI = L.oI[i], I = L.I[i];
+                    const T* __restrict__ xi = D > 2 ? x : x + L.in[i];
+                    const IX in = D > 2 ? L.in[i] : 0;
+                    const int qe = L.qe[i];
+                    int q = L.q0[i] + r + k * G;
+#pragma unroll 2
+                    for (; q + VL < qe; q += 2 * VL) {
+                        const int p0 = a.ce[q], p1 = a.ce[q + VL];
+                        const T v0 = cv[q], v1 = cv[q + VL];
+                        s0 += v0 * load(base, xi, oI, I, in, p0);
+                        s1 += v1 * load(base, xi, oI, I, in, p1);
+                    }
+                    if (q < qe) s0 += cv[q] * load(base, xi, oI, I, in, a.ce[q]);
+                }
+                b[k] = s0 + s1;
+            }
         }
+        if (ncorr > 0)
+#pragma unroll
+            for (int k = 0; k < PER; ++k) {
+                T c0 = T(0);
+                for (int c = r + k * G; c < ncorr; c += VL) c0 += hc[c] * zc[c * zld];
+                b[k] -= c0;
+            }
     }
 #pragma unroll
     for (int o = 1; o < G; o <<= 1)

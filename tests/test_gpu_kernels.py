@@ -222,3 +222,20 @@ def test_order_of_sums_of_the_projection(d, n, k, M, dt, prec, modes, want):
     op.close()
     idx.close()
     ctx.close()
+
+
+@pytest.mark.parametrize("d,n,k", [(2, 5, 3), (2, 9, 3), (3, 4, 3), (3, 7, 2), (3, 7, 3), (4, 4, 2), (4, 4, 3), (4, 6, 2)])
+def test_matvec_lanes_per_output(ctx, d, n, k):
+    # eight, four and two lanes per output in every dimension
+    idx = sgkiif.IndexSet(ctx, d, n, k)
+    kap = [1.0, 0.5, 0.1, 0.7][:d]
+    op = sgkiif.Operator(ctx, idx, kap)
+    dtype, tol = ((torch.float64, 1e-12) if ctx.precision == sgkiif.SGK_FP64 else (torch.float32, 1e-5))
+    xd = dev(np.random.default_rng(n).standard_normal(idx.dof), dtype)
+    yd = torch.empty_like(xd)
+    op.matvec(xd.data_ptr(), yd.data_ptr(), ctx.precision)
+    torch.cuda.synchronize()
+    want = sparse_matvec(OIndex(d, n, k), sipg_1d(n, k), kap, xd.double().cpu().numpy())
+    assert rel(yd.double().cpu().numpy(), want) <= tol
+    op.close()
+    idx.close()
