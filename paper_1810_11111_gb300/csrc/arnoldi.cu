@@ -88,8 +88,9 @@ static size_t smem_budget(const sgk_ctx* ctx) {
     return ctx->smem_optin > 16 * 1024 ? ctx->smem_optin - 13 * 1024 : 32 * 1024;
 }
 
-std::vector<int64_t> arnoldi_balanced_bounds(const sgk_ctx* ctx, const sgk_op* op, int M, int64_t* E,
+std::vector<int64_t> arnoldi_balanced_bounds(const sgk_ctx* ctx, const sgk_op* const* ops, int nops, int M, int64_t* E,
                                              int64_t* list_ent) {
+    const sgk_op* op = ops[0];
     const int nb = persistent_ctas(ctx);
     const int64_t n = op->idx->dof;
     const int d = op->idx->d;
@@ -103,23 +104,19 @@ std::vector<int64_t> arnoldi_balanced_bounds(const sgk_ctx* ctx, const sgk_op* o
                          sgk_arn::arn_eoff_bytes((int)cap_len, d);
     const size_t budget = smem_budget(ctx);
     // one list per output (mixed derivatives): its entries stay in device memory
-    if (op->x1_off.p) {
-        std::vector<int64_t> b1 = arnoldi_slice_bounds(op, nb, 2 * M, cap_len, int64_t(1) << 40);
-        *E = 0;
-        *list_ent = 0;
-        for (size_t i = 0; i + 1 < b1.size(); ++i) *E = std::max<int64_t>(*E, b1[i + 1] - b1[i]);
-        return b1;
-    }
-    int64_t cap_ent = (op->gmv_ecnt_host.empty() || fixed >= budget) ? (int64_t(1) << 40)
-                                                                      : (int64_t)((budget - fixed) / sizeof(int2));
+    int64_t cap_ent = (op->x1_off.p || op->gmv_ecnt_host.empty() || fixed >= budget)
+                          ? (int64_t(1) << 40)
+                          : (int64_t)((budget - fixed) / sizeof(int2));
     std::vector<int64_t> b = arnoldi_slice_bounds(op, nb, 2 * M, cap_len, cap_ent);
     *E = 0;
     *list_ent = 0;
     for (size_t i = 0; i + 1 < b.size(); ++i) {
         *E = std::max<int64_t>(*E, b[i + 1] - b[i]);
-        if (!op->gmv_ecnt_host.empty()) {
+        for (int s = 0; s < nops; ++s) {
+            const std::vector<int32_t>& ecnt = ops[s]->gmv_ecnt_host;
+            if (ops[s]->npairs > 0 || ecnt.empty()) continue;  // no lists in shared memory
             int64_t e = 0;
-            for (int64_t g = b[i]; g < b[i + 1]; ++g) e += op->gmv_ecnt_host[g];
+            for (int64_t g = b[i]; g < b[i + 1]; ++g) e += ecnt[g];
             *list_ent = std::max(*list_ent, e);
         }
     }

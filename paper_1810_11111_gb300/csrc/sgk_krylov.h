@@ -70,9 +70,10 @@ size_t arnoldi_persistent_pbuf_size(const sgk_ctx* ctx, int M);
 bool arnoldi_persistent_takes(const sgk_ctx* ctx, const sgk_op* op);
 // Work-balanced slices for the persistent kernel (arnoldi_slice_bounds with
 // the caps that keep the slice's pre-located gathers and Krylov columns in
-// shared memory); empty when no such partition exists.  E and list_ent
-// receive the longest slice and its most gather entries.
-std::vector<int64_t> arnoldi_balanced_bounds(const sgk_ctx* ctx, const sgk_op* op, int M, int64_t* E,
+// shared memory) for operators on one index set, balanced for the first;
+// empty when no such partition exists.  E and list_ent receive the longest
+// slice and the most gather entries of one slice that any operator stages.
+std::vector<int64_t> arnoldi_balanced_bounds(const sgk_ctx* ctx, const sgk_op* const* ops, int nops, int M, int64_t* E,
                                              int64_t* list_ent);
 // gamma, V (M + 1 columns), H and m_eff of the Krylov space of v, in one
 // cooperative launch.

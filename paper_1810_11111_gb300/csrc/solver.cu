@@ -1546,9 +1546,11 @@ void solver_alloc(sgk_solver* s) {
         s->pbuf.alloc(arnoldi_persistent_pbuf_size(s->ctx, M));
         s->pbar.alloc(2 * S);
         SGK_CUDA_CHECK(cudaMemsetAsync(s->pbar.p, 0, 2 * S * sizeof(unsigned), s->ctx->stream));
-        // slices of about equal work (the species share one index set)
+        // slices of about equal work (the species share one index set, and
+        // the slices of the first one; a list may be longer in another, whose
+        // tensor is of another kind)
         int64_t E = 0, lent = 0;
-        const std::vector<int64_t> bnd = arnoldi_balanced_bounds(s->ctx, s->ops[0], M, &E, &lent);
+        const std::vector<int64_t> bnd = arnoldi_balanced_bounds(s->ctx, s->ops, S, M, &E, &lent);
         if (!bnd.empty() && E >= 1 && E <= 12 * 1024) {  // else equal slices
             s->aE = E;
             s->alist = lent;

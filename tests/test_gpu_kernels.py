@@ -239,3 +239,41 @@ def test_matvec_lanes_per_output(ctx, d, n, k):
     assert rel(yd.double().cpu().numpy(), want) <= tol
     op.close()
     idx.close()
+
+
+@pytest.mark.parametrize("full", [(True, False), (False, True)], ids=["full_diagonal", "diagonal_full"])
+@pytest.mark.parametrize("d,n,k,M", [(2, 4, 2, 20), (3, 3, 1, 12)])
+def test_full_and_diagonal_tensor_in_one_system(ctx, d, n, k, M, full, monkeypatch):
+    # the species share the slices of the persistent kernel, one with a merged
+    # list per output, one with gather entries in shared memory
+    kap = np.linspace(1.0, 0.6, d)
+    K = np.diag(kap) + 0.1 * (np.eye(d, k=1) + np.eye(d, k=-1))
+    idx = sgkiif.IndexSet(ctx, d, n, k)
+    ops = [sgkiif.Operator(ctx, idx, K if f else list(kap)) for f in full]
+    P, E = cross_blocks_1d(n, k, PERIODIC)
+    ref, S = OIndex(d, n, k), sipg_1d(n, k)
+    V = np.random.default_rng(d).standard_normal((2, idx.dof))
+    dt, launches, states = 1e-5, [], []
+    for off in (False, True):
+        if off:
+            monkeypatch.setenv("SGK_NO_PERSISTENT", "1")
+        sol = sgkiif.Solver(ctx, ops, [[(-1.0, (1, 0))], [(0.5, (1, 1))]], M, dt)
+        for s, f in enumerate(full):
+            vd, wd = dev(V[s]), torch.empty(idx.dof, dtype=torch.float64, device="cuda")
+            before = ctx.launches
+            sol.krylov_expv(s, vd.data_ptr(), wd.data_ptr())
+            launches.append(ctx.launches - before)
+            want, _ = krylov_expv(lambda x: sparse_matvec_general(ref, S, P, E, K, x) if f else
+                                  sparse_matvec(ref, S, kap, x), V[s], dt, M)
+            assert rel(wd.cpu().numpy(), want) <= (1e-10 if f or ctx.precision == sgkiif.SGK_FP64 else 1e-9)
+        for s in range(2):
+            sol.set_state(s, 0.1 * V[s])
+        sol.step(2)
+        states.append(np.concatenate([sol.get_state(s) for s in range(2)]))
+        sol.close()
+    # one launch for the process and a few around it, against several a step
+    assert max(launches[:2]) < M < min(launches[2:])
+    assert rel(states[0], states[1]) <= 1e-9
+    for o in ops:
+        o.close()
+    idx.close()
