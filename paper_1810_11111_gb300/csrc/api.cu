@@ -524,9 +524,10 @@ int sgk_solver_create_form(sgk_ctx* ctx, int nspecies, const sgk_op* const* ops,
             const int q = std::max(1, (p * k + k + 1 + 1) / 2);
             SGK_REQUIRE(q <= 8, SGK_EUNSUPPORTED, "reaction degree too high for the quadrature tables");
             quad_build(s->Q, idx, q, nspecies, true);
-            s->Q.fused = pencil_supported(idx->d, idx->k + 1, q, nspecies, idx->n, s->rx, ctx->smem_optin) &&
+            s->Q.fused = pencil_supported(idx->d, idx->k + 1, q, nspecies, idx->n, s->rx, fp64, ctx->smem_optin) &&
                          std::getenv("SGK_NO_FUSED") == nullptr;
-            s->Q.fused_df = s->Q.fused && pencil_df_supported(idx->d, idx->k + 1, q, nspecies);
+            s->Q.fused_df =
+                s->Q.fused && pencil_df_supported(idx->d, idx->k + 1, q, nspecies, idx->n, ctx->smem_optin);
             const size_t elem = fp64 ? 8 : 4;
             const double need = (double)((2 * nspecies + 1) * s->Q.full_size) * elem;
             size_t free_b = 0, total_b = 0;

@@ -21,11 +21,14 @@ SGK_PENCIL_DECLARE(pencil_df_d34)
 
 namespace {
 
-// the largest shared memory of a shape's passes (FP64; FP32 takes half)
+// shared memory of one line in a shape's F passes, in FP64 or double-float,
+// and in its Jacobian passes, in FP64 or FP32
 template <int D, int K, int S>
-size_t shape_smem(int H) {
+size_t line_bytes(int H, bool jac, bool fp64) {
     using namespace sgk_pen;
-    return std::max(PencilShape<double, D, K, S, false>::bytes(H), PencilShape<double, D, K, S, true>::bytes(H));
+    if (jac)
+        return fp64 ? PencilShape<double, D, K, S, true>::bytes(H) : PencilShape<float, D, K, S, true>::bytes(H);
+    return fp64 ? PencilShape<double, D, K, S, false>::bytes(H) : PencilShape<df2, D, K, S, false>::bytes(H);
 }
 
 bool reaction_fits(const ReactionDev& rx, int S) {
@@ -37,21 +40,25 @@ bool reaction_fits(const ReactionDev& rx, int S) {
 
 }  // namespace
 
-bool pencil_df_supported(int d, int kp1, int q, int S) {
+bool pencil_df_supported(int d, int kp1, int q, int S, int N, size_t smem_optin) {
+    if (N == 0) return false;
+    const int H = kp1 << N;
 #define SGK_PENCIL_OK(DD, KK, QQ, SS) \
-    if (d == DD && kp1 == KK && q == QQ && S == SS) return true;
+    if (d == DD && kp1 == KK && q == QQ && S == SS) return line_bytes<DD, KK, SS>(H, false, false) <= smem_optin;
     SGK_PENCIL_DF_D2(SGK_PENCIL_OK)
     SGK_PENCIL_DF_D34(SGK_PENCIL_OK)
 #undef SGK_PENCIL_OK
     return false;
 }
 
-bool pencil_supported(int d, int kp1, int q, int S, int N, const ReactionDev& rx, size_t smem_optin) {
+bool pencil_supported(int d, int kp1, int q, int S, int N, const ReactionDev& rx, bool fp64, size_t smem_optin) {
     if (N == 0 || !reaction_fits(rx, S)) return false;  // one cell: nothing to pair
-    if (pencil_df_supported(d, kp1, q, S)) return true;
     const int H = kp1 << N;
-#define SGK_PENCIL_OK(DD, KK, QQ, SS) \
-    if (d == DD && kp1 == KK && q == QQ && S == SS) return shape_smem<DD, KK, SS>(H) <= smem_optin;
+    const bool df = !fp64 && pencil_df_supported(d, kp1, q, S, N, smem_optin);
+#define SGK_PENCIL_OK(DD, KK, QQ, SS)                                                        \
+    if (d == DD && kp1 == KK && q == QQ && S == SS)                                          \
+        return (df || line_bytes<DD, KK, SS>(H, false, true) <= smem_optin) &&               \
+               line_bytes<DD, KK, SS>(H, true, fp64) <= smem_optin;
     SGK_PENCIL_D2(SGK_PENCIL_OK)
     SGK_PENCIL_D34(SGK_PENCIL_OK)
 #undef SGK_PENCIL_OK

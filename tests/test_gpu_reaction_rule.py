@@ -1,0 +1,60 @@
+"""Which reaction passes a solver takes: sizes and coefficients at which a pass
+does not serve, against the general passes and closed values."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+from paper_1810_11111_gb300 import sgkiif  # noqa: E402
+
+pytestmark = [pytest.mark.gpu,
+              pytest.mark.skipif(not torch.cuda.is_available(), reason="needs a CUDA device")]
+
+CUBIC = [[(-2.0, (3,)), (0.7, (2,)), (-0.3, (0,))]]
+PAIR = [[(0.1, (0, 0)), (-1.0, (1, 0)), (1.0, (2, 1))], [(0.9, (0, 0)), (-1.0, (2, 1))]]
+
+
+def rel(a, b):
+    return float(np.linalg.norm(np.asarray(a) - np.asarray(b)) / max(np.linalg.norm(b), 1e-300))
+
+
+def passes(ctx, d, n, k, rx, U, W):
+    """F(U) and J_F(U) W of a fresh solver."""
+    idx = sgkiif.IndexSet(ctx, d, n, k)
+    ops = [sgkiif.Operator(ctx, idx, [1.0] * d) for _ in rx]
+    sol = sgkiif.Solver(ctx, ops, rx, 2, 0.01)
+    Ud, Wd = (torch.from_numpy(x).cuda() for x in (U, W))
+    Fd, Jd = torch.empty_like(Ud), torch.empty_like(Ud)
+    sol.reaction_eval(Ud.data_ptr(), Fd.data_ptr())
+    sol.jacobian_apply(Ud.data_ptr(), Wd.data_ptr(), Jd.data_ptr())
+    torch.cuda.synchronize()
+    out = Fd.cpu().numpy(), Jd.cpu().numpy()
+    sol.close()
+    for o in ops:
+        o.close()
+    idx.close()
+    return out
+
+
+@pytest.fixture(scope="module", params=[sgkiif.SGK_FP64, sgkiif.SGK_MIXED], ids=["fp64", "mixed"])
+def ctx(request):
+    c = sgkiif.Context(0, torch.cuda.current_stream().cuda_stream, request.param)
+    yield c
+    c.close()
+
+
+@pytest.mark.parametrize("n,k,rx", [(10, 2, PAIR), (11, 1, CUBIC), (11, 2, CUBIC)])
+def test_lines_beyond_shared_memory(ctx, n, k, rx, monkeypatch):
+    # 2D lines of which not every pass fits a CTA's shared memory: the general
+    # passes serve them.  Sums of at most some thousand terms in another
+    # order: 1e-12, FP32 Jacobian 1e-5
+    S, dof = len(rx), sgkiif.dof_of(2, n, k)
+    rng = np.random.default_rng(n)
+    U = 0.3 * rng.standard_normal(S * dof) / np.sqrt(dof)
+    U[::dof] += 0.5
+    W = rng.standard_normal(S * dof)
+    F, J = passes(ctx, 2, n, k, rx, U, W)
+    monkeypatch.setenv("SGK_NO_FUSED", "1")
+    F1, J1 = passes(ctx, 2, n, k, rx, U, W)
+    assert rel(F, F1) <= 1e-12
+    assert rel(J, J1) <= (1e-12 if ctx.precision == sgkiif.SGK_FP64 else 1e-5)
