@@ -31,6 +31,33 @@ size_t line_bytes(int H, bool jac, bool fp64) {
     return fp64 ? PencilShape<double, D, K, S, false>::bytes(H) : PencilShape<df2, D, K, S, false>::bytes(H);
 }
 
+// Lowest levels at which a shape is fused, in FP64 and in mixed mode (1 where
+// it is not listed).  A thread takes one cell, so on a coarse grid the pass
+// lasts as long as one thread's points while most of the machine idles; the
+// general cell pass spreads a cell's points over threads.  Microseconds of F /
+// J at the level below the limit and at it, fused against general, FP64:
+//   (3,4,7,2)  level 5  2870/3665, 2036/3161 (level 6 has 13 warps a
+//              scheduler instead of two)
+//   (3,4,7,1)  4   274/ 346,  177/ 251;  5   701/ 864,  882/1254
+//   (3,3,5,2)  4   345/ 396,  254/ 357;  5   627/ 826,  853/1227
+//   (4,3,5,1)  3   432/ 515,  282/ 381;  4  1805/2382, 2688/4108
+//   (4,2,3,2)  3   312/ 350,  208/ 269;  4   847/ 921,  985/1532
+//   (2,4,7,2)  2   132/ 148,   94/ 136;  3   155/ 182,  178/ 209
+// In mixed mode the FP32 Jacobian products, which are most of the passes, gain
+// earlier: (3,4,7,2) F 928 and J 129 us at level 3, general 227 and 180; 941
+// and 157 at level 4, general 390 and 296.
+struct Lowest {
+    int d, kp1, q, S, fp64, mixed;
+};
+constexpr Lowest LOWEST[] = {{2, 4, 7, 1, 2, 1}, {2, 4, 7, 2, 3, 1}, {3, 2, 3, 2, 2, 1}, {3, 3, 4, 1, 2, 1},
+                             {3, 3, 5, 2, 5, 2}, {3, 4, 7, 1, 5, 2}, {3, 4, 7, 2, 6, 4}, {4, 3, 5, 1, 4, 3},
+                             {4, 2, 3, 2, 4, 1}};
+int lowest_level(int d, int kp1, int q, int S, bool fp64) {
+    for (const Lowest& l : LOWEST)
+        if (l.d == d && l.kp1 == kp1 && l.q == q && l.S == S) return fp64 ? l.fp64 : l.mixed;
+    return 1;
+}
+
 bool reaction_fits(const ReactionDev& rx, int S) {
     for (int m = 0; m < rx.nmono; ++m)
         for (int r = 0; r < S; ++r)
@@ -52,7 +79,7 @@ bool pencil_df_supported(int d, int kp1, int q, int S, int N, size_t smem_optin)
 }
 
 bool pencil_supported(int d, int kp1, int q, int S, int N, const ReactionDev& rx, bool fp64, size_t smem_optin) {
-    if (N == 0 || !reaction_fits(rx, S)) return false;  // one cell: nothing to pair
+    if (N < lowest_level(d, kp1, q, S, fp64) || !reaction_fits(rx, S)) return false;  // level 0: nothing to pair
     const int H = kp1 << N;
     const bool df = !fp64 && pencil_df_supported(d, kp1, q, S, N, smem_optin);
 #define SGK_PENCIL_OK(DD, KK, QQ, SS)                                                        \
