@@ -40,6 +40,7 @@
 // belong to the whole pencil, are stored in both.
 #pragma once
 #include <algorithm>
+#include <cmath>
 #include <type_traits>
 
 #include "sgk_pencil.h"
@@ -83,7 +84,7 @@ struct QuadTab {
 template <typename T, int S, int NP>
 struct Poly {
     Cst<T> c[NP][Pow<PDEG, S>::v];
-    unsigned char rows[NP], mask[NP][PDEG];
+    unsigned char rows[NP], mask[NP][PDEG], monic;
 };
 
 // The largest total degree of f whose pass has q points at k + 1 = K: q =
@@ -92,8 +93,12 @@ __host__ __device__ constexpr int max_degree(int K, int Q) { return (2 * Q - K) 
 
 // One species in FP64: the polynomial is divided by its leading coefficient,
 // which goes into the outermost table of the moments (one multiplication less
-// at every point: -c u^3 takes two).  Not in the narrower types, whose range
-// would not hold the bare powers of a decayed state.
+// at every point: -c u^3 takes two), where that stays in range: with a leading
+// coefficient of at least 1 no bare power overflows where the term does not,
+// below 2^128 it underflows only where the term does by 2^-894, and the other
+// coefficients keep their digits in the quotients (Poly::monic).  Not in the
+// narrower types, whose range would not hold the bare powers of a decayed
+// state.
 template <typename T, int S>
 constexpr bool MONIC = std::is_same<T, double>::value && S == 1;
 
@@ -117,7 +122,7 @@ __device__ __forceinline__ T poly_value(const Poly<T, 1, NP>& P, int i, const T 
         if (!SKIP || ((P.rows[i] >> e) & 1)) {
             if (state == 0) {
                 f = cvalue(P.c[i][e]);
-                state = MONIC<T, 1> ? 1 : 2;
+                state = MONIC<T, 1> && P.monic ? 1 : 2;
             } else {
                 f = add(f, cvalue(P.c[i][e]));
             }
@@ -704,15 +709,21 @@ Poly<T, S, (JAC ? S * S : S)> make_poly(const ReactionDev& rx, double s, double*
         }
     }
     *lead = 1.0;
+    Poly<T, S, NP> p{};
     if (MONIC<T, S>)
         for (int j = NCOEF - 1; j >= 0; --j)
             if (c[0][j] != 0.0) {
-                *lead = c[0][j];
-                for (int l = 0; l < j; ++l) c[0][l] /= *lead;
-                c[0][j] = 1.0;
+                const double a = std::fabs(c[0][j]);
+                bool fits = a >= 1.0 && a <= 0x1p128;
+                for (int l = 0; l < j; ++l) fits = fits && (c[0][l] == 0.0 || std::fabs(c[0][l]) / a >= 0x1p-900);
+                if (fits) {
+                    p.monic = 1;
+                    *lead = c[0][j];
+                    for (int l = 0; l < j; ++l) c[0][l] /= *lead;
+                    c[0][j] = 1.0;
+                }
                 break;
             }
-    Poly<T, S, NP> p{};
     for (int i = 0; i < NP; ++i)
         for (int j = 0; j < NCOEF; ++j) {
             cst_set(p.c[i][j], c[i][j]);

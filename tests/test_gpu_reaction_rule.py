@@ -58,3 +58,27 @@ def test_lines_beyond_shared_memory(ctx, n, k, rx, monkeypatch):
     F1, J1 = passes(ctx, 2, n, k, rx, U, W)
     assert rel(F, F1) <= 1e-12
     assert rel(J, J1) <= (1e-12 if ctx.precision == sgkiif.SGK_FP64 else 1e-5)
+
+
+@pytest.mark.parametrize("c,u", [(1e-300, 1e110), (-1e-220, 1e105), (1e200, 1e-110)])
+@pytest.mark.parametrize("low", [0.0, 0.5])
+def test_coefficients_near_the_ends_of_the_range(c, u, low):
+    # FP64, f(u) = c u^3 + low c u^2 u_0 with u_0 the state's size: c u^3 is
+    # finite where u^3 is not.  F scales like c u^3, J like c u^2
+    fp64 = sgkiif.Context(0, torch.cuda.current_stream().cuda_stream, sgkiif.SGK_FP64)
+    d, n, k = 3, 3, 2
+    rng = np.random.default_rng(3)
+    U = 0.1 * rng.standard_normal(sgkiif.dof_of(d, n, k))
+    U[0] = 1.0
+    W = rng.standard_normal(U.size)
+
+    def terms(c, u0):
+        return [[(c, (3,))] + ([(low * c * u0, (2,))] if low else [])]
+
+    # the oracle scales by powers of two, which are exact
+    su = 2.0 ** round(np.log2(u))
+    F1, J1 = passes(fp64, d, n, k, terms(1.0, 1.0), U, W)
+    F, J = passes(fp64, d, n, k, terms(c, su), su * U, W)
+    assert rel(F / (c * su) / su / su, F1) <= 1e-12
+    assert rel(J / (c * su) / su, J1) <= 1e-12
+    fp64.close()
