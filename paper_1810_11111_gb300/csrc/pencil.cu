@@ -58,10 +58,23 @@ int lowest_level(int d, int kp1, int q, int S, bool fp64) {
     return 1;
 }
 
-bool reaction_fits(const ReactionDev& rx, int S) {
-    for (int m = 0; m < rx.nmono; ++m)
-        for (int r = 0; r < S; ++r)
+// h^{-d/2}, the scale between the pass's basis and the orthonormal one
+double basis_scale(int d, int N) { return std::ldexp((d * N) % 2 ? 1.4142135623730951 : 1.0, d * N / 2); }
+
+// The exponents have places in the tables, and the coefficients of the scaled
+// basis, c s^{degree + 1}, stand far enough inside the range of FP64 or, in
+// mixed mode, of FP32 (c itself may be within it and they not: 1e32 u^3 on
+// 64^2 cells).
+bool reaction_fits(const ReactionDev& rx, int S, int d, int N, bool fp64) {
+    const double s = basis_scale(d, N);
+    for (int m = 0; m < rx.nmono; ++m) {
+        double v = std::fabs(rx.coef[m]) * s;
+        for (int r = 0; r < S; ++r) {
             if (rx.exps[m][r] >= sgk_pen::PDEG) return false;
+            v *= std::pow(s, rx.exps[m][r]);
+        }
+        if (!(v <= (fp64 ? 0x1p1000 : 0x1p100))) return false;
+    }
     return true;
 }
 
@@ -79,7 +92,7 @@ bool pencil_df_supported(int d, int kp1, int q, int S, int N, size_t smem_optin)
 }
 
 bool pencil_supported(int d, int kp1, int q, int S, int N, const ReactionDev& rx, bool fp64, size_t smem_optin) {
-    if (N < lowest_level(d, kp1, q, S, fp64) || !reaction_fits(rx, S)) return false;  // level 0: nothing to pair
+    if (N < lowest_level(d, kp1, q, S, fp64) || !reaction_fits(rx, S, d, N, fp64)) return false;  // level 0: nothing to pair
     const int H = kp1 << N;
     const bool df = !fp64 && pencil_df_supported(d, kp1, q, S, N, smem_optin);
 #define SGK_PENCIL_OK(DD, KK, QQ, SS)                                                        \
@@ -95,8 +108,7 @@ bool pencil_supported(int d, int kp1, int q, int S, int N, const ReactionDev& rx
 template <typename T>
 void pencil_launch(sgk_ctx* ctx, const PencilArgs& a, int d, int kp1, int q, int S, bool jac, const double* B,
                    const double* w, const double* two_scale, const ReactionDev& rx) {
-    // s = h^{-d/2}
-    const double scale = std::ldexp((d * a.N) % 2 ? 1.4142135623730951 : 1.0, d * a.N / 2);
+    const double scale = basis_scale(d, a.N);
     KTimer kt(ctx, KC_CELL);
     bool ok = false;
     if constexpr (std::is_same<T, dfloat>::value) {

@@ -82,3 +82,18 @@ def test_coefficients_near_the_ends_of_the_range(c, u, low):
     assert rel(F / (c * su) / su / su, F1) <= 1e-12
     assert rel(J / (c * su) / su, J1) <= 1e-12
     fp64.close()
+
+
+@pytest.mark.parametrize("d,n,k", [(2, 6, 2), (3, 5, 2), (4, 3, 1)])
+def test_large_coefficients_of_a_small_state(ctx, d, n, k):
+    # 1e32 u^3 at u = 1e-11: within FP32's range in the orthonormal basis, not
+    # in the pass's scaled one.  F to 1e-12 in both modes, an FP32 J to 1e-5
+    c, u = 2.0 ** 106, 2.0 ** -36
+    rng = np.random.default_rng(n)
+    U = 0.1 * rng.standard_normal(sgkiif.dof_of(d, n, k)) / (1 + np.arange(sgkiif.dof_of(d, n, k)))
+    U[0] = 1.0
+    W = rng.standard_normal(U.size)
+    F1, J1 = passes(ctx, d, n, k, [[(1.0, (3,))]], U, W)
+    F, J = passes(ctx, d, n, k, [[(c, (3,))]], u * U, W)
+    assert rel(F / c / u ** 3, F1) <= 1e-12
+    assert rel(J / c / u ** 2, J1) <= (1e-12 if ctx.precision == sgkiif.SGK_FP64 else 1e-5)
