@@ -24,11 +24,12 @@
 // prefix of the row.  cross_rows_kernel adds -K_ij B_ij x to y after the
 // diagonal gather (gmv_kernel): one warp per output, the lanes striding over
 // the row.  Index sets whose table would exceed X2_MAX_ENT entries (level 8,
-// degree 2 holds 42 M of the 67 M, level 8, degree 3 twice the limit) keep
-// cross_kernel: one thread per output, the two factors' rows walked as a
+// degree 2 holds 42 M of the 67 M, level 8, degree 3 twice the limit), and
+// operators for whose table the device has no memory left, keep cross_kernel: one thread per output, the two factors' rows walked as a
 // sum-factorised double loop.
 #include <algorithm>
 #include <cmath>
+#include <cstdlib>
 #include <map>
 
 #include "sgk_internal.h"
@@ -308,6 +309,20 @@ __global__ void __launch_bounds__(256) cross_kernel(int64_t dof, int d, int N, i
 
 }  // namespace
 
+// Takes the memory of an optional table; false when the device has too little
+// left (SGK_TEST_NO_TABLE_MEMORY in the environment: as if it had).
+template <typename F>
+static bool take_memory(F&& allocate) {
+    try {
+        if (std::getenv("SGK_TEST_NO_TABLE_MEMORY")) throw SgkError{SGK_ENOMEM, "no memory for a table"};
+        allocate();
+        return true;
+    } catch (const SgkError& e) {
+        if (e.code != SGK_ENOMEM) throw;
+        return false;
+    }
+}
+
 // Tables of the mixed-derivative terms of op for the tensor K (d x d,
 // row-major, symmetric); no-op when K is diagonal.
 void build_cross_tables(sgk_op* op, const double* K) {
@@ -447,20 +462,30 @@ void build_cross_tables(sgk_op* op, const double* K) {
             total += n;
         }
     }
-    if (total <= X2_MAX_ENT && idx->dof < (int64_t(1) << 31) && len2.size() < (size_t(1) << 31)) {
-        cudaStream_t s2 = op->ctx->stream;
-        DevBuf<int> d_uptr, d_ucol, d_upto;
-        DevBuf<double> d_uval;
-        d_uptr.upload(uptr, s2);
-        d_ucol.upload(ucol, s2);
-        d_uval.upload(uval, s2);
-        d_upto.upload(upto, s2);
-        op->x2_ptr.upload(ptr2, s2);
-        op->x2_len.upload(len2, s2);
-        op->x2_row.upload(row2, s2);
-        op->x2_ent.alloc(total);
-        op->x2_val.alloc(total);
-        op->x2_valf.alloc(total);
+    cudaStream_t s2 = op->ctx->stream;
+    DevBuf<int> d_uptr, d_ucol, d_upto;
+    DevBuf<double> d_uval;
+    if (total <= X2_MAX_ENT && idx->dof < (int64_t(1) << 31) && len2.size() < (size_t(1) << 31) &&
+        !take_memory([&]() {
+            op->x2_val.alloc(total);
+            op->x2_valf.alloc(total);
+            op->x2_ptr.upload(ptr2, s2);
+            op->x2_len.upload(len2, s2);
+            op->x2_row.upload(row2, s2);
+            d_uptr.upload(uptr, s2);
+            d_ucol.upload(ucol, s2);
+            d_uval.upload(uval, s2);
+            d_upto.upload(upto, s2);
+            op->x2_ent.alloc(total);  // last: tells that the table is there
+        })) {
+        // cross_kernel serves an operator without the table
+        op->x2_val.release();
+        op->x2_valf.release();
+        op->x2_ptr.release();
+        op->x2_len.release();
+        op->x2_row.release();
+    }
+    if (op->x2_ent.p) {
         cross_fill_kernel<<<H, 256, 0, s2>>>(H, N, kp1, d_uptr.p, d_ucol.p, d_uval.p, d_upto.p, op->x2_row.p,
                                              op->x2_ptr.p, op->x2_len.p, op->x2_ent.p, op->x2_val.p, op->x2_valf.p);
         check_launch("cross_fill_kernel");
@@ -523,17 +548,21 @@ void build_cross_tables(sgk_op* op, const double* K) {
             if (total1 > X1_MAX_ENT) break;
             off1.push_back((int)total1);
         }
-        if (total1 <= X1_MAX_ENT) {
-            op->x1_off.upload(off1, s);
-            op->x1_ei.alloc(total1);
-            op->x1_ev.alloc(total1);
+        if (total1 <= X1_MAX_ENT && take_memory([&]() {
+                op->x1_ei.alloc(total1);
+                op->x1_ev.alloc(total1);
+                op->x1_off.upload(off1, s);
+            })) {
             cross_merge_kernel<<<(int)((idx->dof + 7) / 8), 256, 0, s>>>(
                 (int)idx->dof, d, N, kp1, (int)nt, idx->d_levels.p, idx->d_offsets.p, op->gmv_eoff.p, op->gmv_ent.p,
                 op->gmv_cvk.p, op->npairs, op->x_pairs.p, op->x_kij.p, op->x2_row.p, op->x2_ptr.p, op->x2_len.p,
                 op->x2_ent.p, op->x2_val.p, op->x_grp.p, op->x_off.p, op->x1_off.p, op->x1_ei.p, op->x1_ev.p);
             check_launch("cross_merge_kernel");
             count_launch(op->ctx);
-        } else {
+        } else {  // the launch sequence serves it
+            op->x1_off.release();
+            op->x1_ei.release();
+            op->x1_ev.release();
             op->x1_cnt.clear();
         }
     }
