@@ -418,21 +418,23 @@ __device__ __forceinline__ void slice_dots(const double* Vl, int64_t vld, int nc
 
 // sum_{c < ncols} Vl[c vld + u] h[c] for the elements u < ne of the slice, in
 // two parts with a CTA barrier between them: combine_begin calls use(u, sum)
-// for the elements below the number it returns, combine_end for the others.
-// The FP64 pipe of a scheduler takes 64 clocks a warp instruction, so an
-// element per thread, four chains each, costs 64 ncols clocks for every four
-// warps of elements begun.  The warps beyond a multiple of four (slices of at
-// most 2 PT / 4 elements) split their columns over the four schedulers
-// instead, 16 ncols clocks a warp, where that saves more than the sums in tmp
-// (PT doubles) behind the barrier, some 300 clocks.  The same chains and sums
-// either way, so the slicing changes no bit.
+// for the elements below the number it returns (all or none), combine_end for
+// the others.  The FP64 pipe of a scheduler takes 64 clocks a warp
+// instruction, so an element per thread, four chains each, costs 64 ncols
+// clocks for every four warps of elements begun.  Slices of one to three warps
+// split their columns over the four schedulers instead, 16 ncols clocks a
+// warp, where that saves more than the sums in tmp (PT doubles) behind the
+// barrier, some 300 clocks.  Per exponential, FP64, never split against this:
+// 432 x 30 457 -> 443 us, 1 024 x 30 493 -> 478, 5 504 x 25 432 -> 424, 11 520 x
+// 40 839 -> 820; splitting the part beyond four warps of longer slices as well
+// made 20 480 x 40 1130 us out of 1087.  The same chains and sums either way,
+// so the slicing changes no bit.
 template <typename Use>
 __device__ __forceinline__ int combine_begin(const double* Vl, int64_t vld, int ncols, const double* h, int ne,
                                              double* tmp, Use&& use) {
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const int warps = (ne + 31) >> 5, rest = warps & 3;
-    const bool split = ne <= 2 * PT / 4 && rest > 0 && (4 - rest) * ncols >= 20;
-    const int whole = split ? (warps - rest) * 32 : ne;
+    const int warps = (ne + 31) >> 5;
+    const int whole = warps < 4 && (4 - warps) * ncols >= 20 ? 0 : ne;
     for (int u = threadIdx.x; u < whole; u += PT) {
         const double* vi = Vl + u;
         double a0 = 0.0, a1 = 0.0, a2 = 0.0, a3 = 0.0;
