@@ -57,27 +57,10 @@ __device__ __forceinline__ dfloat operator-(dfloat a) { return dfloat(-a.hi, -a.
 __device__ __forceinline__ dfloat operator-(dfloat a, dfloat b) { return a + (-b); }
 __device__ __forceinline__ dfloat& operator+=(dfloat& a, dfloat b) { return a = a + b; }
 
-// renormalised pair: |lo| <= ulp(hi) / 2
-__device__ __forceinline__ dfloat df_norm(dfloat a) {
-    const float h = __fadd_rn(a.hi, a.lo);
-    return dfloat(h, __fsub_rn(a.lo, __fsub_rn(h, a.hi)));
-}
-
 __device__ __forceinline__ double df_value(dfloat a) { return (double)a.hi + (double)a.lo; }
 __device__ __forceinline__ float df_float(dfloat a) { return __fadd_rn(a.hi, a.lo); }
 __device__ __forceinline__ dfloat df_split(double x) {
     const float h = __double2float_rn(x);
     return dfloat(h, __double2float_rn(x - (double)h));
-}
-
-// read through volatile pointers (the element re-read at every use)
-template <typename T>
-__device__ __forceinline__ T volatile_read(const T* p) {
-    return *reinterpret_cast<const volatile T*>(p);
-}
-template <>
-__device__ __forceinline__ dfloat volatile_read<dfloat>(const dfloat* p) {
-    const volatile float* f = reinterpret_cast<const volatile float*>(p);
-    return dfloat(f[0], f[1]);
 }
 #endif

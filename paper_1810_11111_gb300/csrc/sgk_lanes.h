@@ -218,14 +218,6 @@ __device__ __forceinline__ df2 maddc(const Cst<df2>& k, df2 x, df2 a) {
     const f2 err = sub(sub(a.hi, sub(s, bb)), add(np, bb));
     return df2{s, add(err, add(a.lo, e))};
 }
-__device__ __forceinline__ df2 nmaddc(const Cst<df2>& k, df2 x, df2 a) {
-    f2 np, e;
-    prodc(k, x, np, e);
-    const f2 s = add(a.hi, np);  // a - p
-    const f2 bb = sub(s, a.hi);
-    const f2 err = add(sub(a.hi, sub(s, bb)), sub(np, bb));
-    return df2{s, add(err, sub(a.lo, e))};
-}
 __device__ __forceinline__ df2 cvalue(const Cst<df2>& k) { return df2{from(k.ch), from(k.cl)}; }
 __device__ __forceinline__ df2 add_signed(df2 a, df2 b, bool n0, bool n1) {
     const f2 s = signs(n0, n1);

@@ -663,12 +663,6 @@ __global__ void __maxnreg__(MAX_REGS<T>)
                 for (int u = threadIdx.x; u < np * P; u += blockDim.x)
                     bwd_root<T, K, PS>(buf(u / P, mbuf), buf(u / P, NSETS - 1), u % P, F);
                 __syncthreads();
-            } else if (N == 0) {  // one cell: the moments are the coefficients
-                for (int u = threadIdx.x; u < np * K * PS; u += blockDim.x) {
-                    const int pp = u / (K * PS), i = u - pp * (K * PS);
-                    buf(pp, NSETS - 1)[i] = buf(pp, mbuf)[i];
-                }
-                __syncthreads();
             }
             Elem* dst = reinterpret_cast<Elem*>(args.out[s]);
             each_position([&](int pp, int pos, int lane, int, long long base, int nl) {

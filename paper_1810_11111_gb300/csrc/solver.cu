@@ -1512,9 +1512,9 @@ void solver_alloc(sgk_solver* s) {
         s->W2.alloc(N);
     }
     SGK_CUDA_CHECK(cudaMemsetAsync(s->U.p, 0, N * sizeof(double), s->ctx->stream));
-    // the fused Gram-Schmidt kernels read whole 128-element slices (past n in
-    // the last one, multiplied by zero): pad the basis and keep it finite
-    s->V64.alloc((M + 1) * n + 128);
+    // finite from the start: sgk_krylov_export copies every column, also those
+    // behind a breakdown
+    s->V64.alloc((M + 1) * n);
     SGK_CUDA_CHECK(cudaMemsetAsync(s->V64.p, 0, s->V64.n * sizeof(double), s->ctx->stream));
     s->w64.alloc(n);
     s->Hm.alloc((M + 1) * M);
