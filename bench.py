@@ -150,7 +150,7 @@ PENCIL_TRAFFIC = {(3, 6, 2, "mixed"): 56705536 + 9454336}
 # one persistent Arnoldi launch (one exponential), keyed by (d, level,
 # degree, M, precision): profiles/arnoldi_kernel_cubic3d_l6k2_m30.md (the
 # mixed-precision variant, double-float gather)
-ARNOLDI_TRAFFIC = {(3, 6, 2, 30, "mixed"): 6505728 + 105216}
+ARNOLDI_TRAFFIC = {(3, 6, 2, 30, "mixed"): 6524672 + 68352}
 
 
 def pencil_q(cfg):

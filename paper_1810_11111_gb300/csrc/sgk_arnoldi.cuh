@@ -351,11 +351,13 @@ __device__ __forceinline__ void fx_columns(const unsigned long long* set, int nt
 // of two, the most with nt CH <= PT, at most 32) sum strided elements in two
 // chains; the CH partials of a column are added in a fixed tree, quarters by
 // four threads, then the four by shuffles (129 columns: two and two).  FP64
-// additions all of them, in an order that is kept to the bit (see arnoldi.cu); adding the lanes' products as integers by shuffles took
-// fewer clocks and moved the results of solves that amplify roundings.  An
-// FP64 instruction takes 64 clocks, so additions of lanes without an element
-// are left out, and a slice of up to four elements (the smallest problems)
-// takes one thread per column.  tmp holds PT doubles.
+// additions all of them, in an order that is kept to the bit (see arnoldi.cu);
+// adding the lanes' products as integers by shuffles took fewer clocks and
+// moved the results of solves that amplify roundings.  An FP64 instruction
+// takes 64 clocks, so additions of lanes without an element are left out, and
+// a slice of up to four elements (the smallest problems) takes one thread per
+// column (432 x 30: 443 us per exponential, 467 without).  tmp holds PT
+// doubles.
 template <typename Emit>
 __device__ __forceinline__ void slice_dots(const double* Vl, int64_t vld, int ncols, const double* ws, int ne,
                                            bool norm, double* tmp, Emit&& emit) {
