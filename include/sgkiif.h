@@ -186,7 +186,10 @@ int sgk_operator_assemble(sgk_ctx* ctx, const sgk_index* idx, const double* kapp
  * launches (the diagonal gather, then the mixed terms); solvers on such an
  * operator keep the FP64 matvec inside the Arnoldi process in both precision
  * modes, in the persistent kernel when every output's entries of all terms
- * fit one list (some 26 000 coefficients), else as a sequence of launches. */
+ * fit one list (some 26 000 coefficients), else as a sequence of launches.
+ * The tables behind both (up to 1.7 GB) are left out where the device has no
+ * memory for them; setting the environment variable SGK_TEST_NO_TABLE_MEMORY
+ * at assembly does the same, for tests. */
 int sgk_operator_assemble_full(sgk_ctx* ctx, const sgk_index* idx, const double* K, int bc, double sigma,
                                sgk_op** out);
 /* Multiply-adds of one sgk_matvec: the entries of the 1D matrix rows each

@@ -84,7 +84,8 @@ size_t arnoldi_persistent_pbuf_size(const sgk_ctx* ctx, int M) {
 }
 
 static size_t smem_budget(const sgk_ctx* ctx) {
-    // the kernel's static shared memory stays below 13 KB
+    // the kernel's static shared memory stays below 13 KB (7.5; the slices, and
+    // with them the order of the sums, go by this budget)
     return ctx->smem_optin > 16 * 1024 ? ctx->smem_optin - 13 * 1024 : 32 * 1024;
 }
 
