@@ -277,3 +277,23 @@ def test_full_and_diagonal_tensor_in_one_system(ctx, d, n, k, M, full, monkeypat
     for o in ops:
         o.close()
     idx.close()
+
+
+@pytest.mark.parametrize("d,n,k", [(2, 4, 1), (2, 5, 2), (3, 4, 2)])
+def test_projection_with_the_most_columns(ctx, d, n, k):
+    # 128 columns and the norm: two lanes a column instead of four.  Converged
+    # for this dt: 1e-10, with the double-float matvec 1e-9
+    idx = sgkiif.IndexSet(ctx, d, n, k)
+    kap = [1.0, 0.5, 0.1][:d]
+    op = sgkiif.Operator(ctx, idx, kap)
+    M, dt = 128, 1e-4
+    sol = sgkiif.Solver(ctx, [op], [[]], M, dt)
+    v = np.random.default_rng(n).standard_normal(idx.dof)
+    vd, wd = dev(v), torch.empty(idx.dof, dtype=torch.float64, device="cuda")
+    sol.krylov_expv(0, vd.data_ptr(), wd.data_ptr())
+    ref, S = OIndex(d, n, k), sipg_1d(n, k)
+    want, _ = krylov_expv(lambda x: sparse_matvec(ref, S, kap, x), v, dt, M)
+    assert rel(wd.cpu().numpy(), want) <= (1e-10 if ctx.precision == sgkiif.SGK_FP64 else 1e-9)
+    sol.close()
+    op.close()
+    idx.close()
